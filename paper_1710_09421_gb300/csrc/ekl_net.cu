@@ -23,6 +23,7 @@
 #include <stdint.h>
 #include <string.h>
 
+#include <mutex>
 #include <vector>
 
 #include <new>
@@ -38,7 +39,6 @@ namespace {
 
 using namespace ekl;
 
-constexpr int C = 16;     // hidden channels
 constexpr int K27 = 27;
 constexpr int NT = 256;   // threads per block of the CUDA-core kernels
 // parameter offsets
@@ -50,7 +50,8 @@ static_assert(NPARAM == EKL_NET_PARAMS, "parameter count");
 struct NetGrid {
     int nx, ny, nz;
     int per[3];
-    int N;
+    int N;      // nodes of one sample
+    int total;  // nodes of all samples of the pass (ns N): node n belongs to sample n / N
 };
 
 // neighbour of node (x,y,z) at offset k; -1 beyond a closed face
@@ -81,25 +82,59 @@ __device__ __forceinline__ void xyz_of(const NetGrid &g, int n, int &x, int &y, 
     y = r - z * g.ny;
 }
 
+// coordinates of node n of a pass over several samples; returns the first
+// node of its sample
+__device__ __forceinline__ int sample_xyz(const NetGrid &g, int n, int &x, int &y, int &z)
+{
+    const int base = (n / g.N) * g.N;
+    xyz_of(g, n - base, x, y, z);
+    return base;
+}
+
+// Network input of the samples of a pass: sample s is x + 2 N smp[s] (smp
+// null: the samples in order), two channels of N nodes.
+struct NetInput {
+    const float *x;
+    const int *smp;
+};
+__device__ __forceinline__ const float *sample_x(const NetGrid &g, const NetInput &in, int s)
+{
+    return in.x + 2 * (size_t)g.N * (in.smp ? in.smp[s] : s);
+}
+
 // ---------------------------------------------------------------- layer 1
 // act1[n][co] = relu(b1[co] + sum_k sum_ci W1[co][ci][k] x[ci][n + off_k])
-__global__ void __launch_bounds__(NT) l1_fwd(NetGrid g, const float *__restrict__ x, const float *__restrict__ w,
+__global__ void __launch_bounds__(NT) l1_fwd(NetGrid g, NetInput in, const float *__restrict__ w,
                                              __nv_bfloat16 *__restrict__ act)
 {
-    __shared__ float sw[16 * 2 * 27 + 16];
-    for (int t = threadIdx.x; t < 16 * 2 * 27 + 16; t += blockDim.x) sw[t] = w[OW1 + t];
+    // weights as [offset and channel][16 outputs]: one 16-byte load per four outputs
+    __shared__ __align__(16) float sw[16 * 2 * 27 + 16];
+    for (int t = threadIdx.x; t < 16 * 54; t += blockDim.x) {
+        const int c = t / 54, r = t - 54 * c, ci = r / 27, k = r - 27 * ci;
+        sw[(2 * k + ci) * 16 + c] = w[OW1 + t];
+    }
+    if (threadIdx.x < 16) sw[16 * 54 + threadIdx.x] = w[OB1 + threadIdx.x];
     __syncthreads();
     const int n = blockIdx.x * blockDim.x + threadIdx.x;
-    if (n >= g.N) return;
+    if (n >= g.total) return;
     int X, Y, Z;
-    xyz_of(g, n, X, Y, Z);
+    const float *x = sample_x(g, in, sample_xyz(g, n, X, Y, Z) / g.N);
     float acc[16];
+#pragma unroll
     for (int c = 0; c < 16; c++) acc[c] = sw[16 * 54 + c];
+#pragma unroll 3
     for (int k = 0; k < K27; k++) {
         const int j = nbr_off(g, X, Y, Z, k);
         if (j < 0) continue;
         const float x0 = x[j], x1 = x[g.N + j];
-        for (int c = 0; c < 16; c++) acc[c] += sw[c * 54 + k] * x0 + sw[c * 54 + 27 + k] * x1;
+#pragma unroll
+        for (int c = 0; c < 16; c += 4) {
+            const float4 w0 = *(const float4 *)(sw + 32 * k + c), w1 = *(const float4 *)(sw + 32 * k + 16 + c);
+            acc[c] += w0.x * x0 + w1.x * x1;
+            acc[c + 1] += w0.y * x0 + w1.y * x1;
+            acc[c + 2] += w0.z * x0 + w1.z * x1;
+            acc[c + 3] += w0.w * x0 + w1.w * x1;
+        }
     }
     for (int c = 0; c < 16; c += 2) {
         __nv_bfloat162 v = __floats2bfloat162_rn(fmaxf(acc[c], 0.f), fmaxf(acc[c + 1], 0.f));
@@ -131,22 +166,23 @@ __global__ void __launch_bounds__(256) conv16_mma(NetGrid g, const __nv_bfloat16
     const int lane = threadIdx.x & 31, gid = lane >> 2, tig = lane & 3;
     const int warp_global = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
     const int n0 = warp_global * 16;
-    if (n0 >= g.N) return;
+    if (n0 >= g.total) return;
     const int na = n0 + gid, nb = n0 + gid + 8;
     int xa, ya, za, xb, yb, zb;
-    xyz_of(g, na < g.N ? na : 0, xa, ya, za);
-    xyz_of(g, nb < g.N ? nb : 0, xb, yb, zb);
+    const int basea = sample_xyz(g, na < g.total ? na : 0, xa, ya, za);
+    const int baseb = sample_xyz(g, nb < g.total ? nb : 0, xb, yb, zb);
     float d[2][4] = {{0.f, 0.f, 0.f, 0.f}, {0.f, 0.f, 0.f, 0.f}};
     const uint32_t *in32 = (const uint32_t *)in;
     for (int k = 0; k < K27; k++) {
         const int kk = flip ? 26 - k : k;
-        const int ja = na < g.N ? nbr_off(g, xa, ya, za, kk) : -1;
-        const int jb = nb < g.N ? nbr_off(g, xb, yb, zb, kk) : -1;
+        const int ja = na < g.total ? nbr_off(g, xa, ya, za, kk) : -1;
+        const int jb = nb < g.total ? nbr_off(g, xb, yb, zb, kk) : -1;
+        const uint32_t *pa = in32 + (size_t)(basea + ja) * 8, *pb = in32 + (size_t)(baseb + jb) * 8;
         uint32_t a[4];
-        a[0] = ja >= 0 ? in32[(size_t)ja * 8 + tig] : 0u;
-        a[1] = jb >= 0 ? in32[(size_t)jb * 8 + tig] : 0u;
-        a[2] = ja >= 0 ? in32[(size_t)ja * 8 + tig + 4] : 0u;
-        a[3] = jb >= 0 ? in32[(size_t)jb * 8 + tig + 4] : 0u;
+        a[0] = ja >= 0 ? pa[tig] : 0u;
+        a[1] = jb >= 0 ? pb[tig] : 0u;
+        a[2] = ja >= 0 ? pa[tig + 4] : 0u;
+        a[3] = jb >= 0 ? pb[tig + 4] : 0u;
 #pragma unroll
         for (int h = 0; h < 2; h++) {
             const int co = h * 8 + gid;
@@ -168,46 +204,151 @@ __global__ void __launch_bounds__(256) conv16_mma(NetGrid g, const __nv_bfloat16
             for (int q = 0; q < 4; q++) v[q] = fmaxf(v[q], 0.f);
         // gradient through the ReLU of the layer that produced `relu_mask_src`
         if (relu_mask_src) {
-            if (na < g.N) {
+            if (na < g.total) {
                 if (!(__bfloat162float(relu_mask_src[(size_t)na * 16 + co]) > 0.f)) v[0] = 0.f;
                 if (!(__bfloat162float(relu_mask_src[(size_t)na * 16 + co + 1]) > 0.f)) v[1] = 0.f;
             }
-            if (nb < g.N) {
+            if (nb < g.total) {
                 if (!(__bfloat162float(relu_mask_src[(size_t)nb * 16 + co]) > 0.f)) v[2] = 0.f;
                 if (!(__bfloat162float(relu_mask_src[(size_t)nb * 16 + co + 1]) > 0.f)) v[3] = 0.f;
             }
         }
         if (OUT_F32) {
             float *o = (float *)out;
-            if (na < g.N) { o[(size_t)na * 16 + co] = v[0]; o[(size_t)na * 16 + co + 1] = v[1]; }
-            if (nb < g.N) { o[(size_t)nb * 16 + co] = v[2]; o[(size_t)nb * 16 + co + 1] = v[3]; }
+            if (na < g.total) { o[(size_t)na * 16 + co] = v[0]; o[(size_t)na * 16 + co + 1] = v[1]; }
+            if (nb < g.total) { o[(size_t)nb * 16 + co] = v[2]; o[(size_t)nb * 16 + co + 1] = v[3]; }
         } else {
             __nv_bfloat16 *o = (__nv_bfloat16 *)out;
-            if (na < g.N) *(__nv_bfloat162 *)(o + (size_t)na * 16 + co) = __floats2bfloat162_rn(v[0], v[1]);
-            if (nb < g.N) *(__nv_bfloat162 *)(o + (size_t)nb * 16 + co) = __floats2bfloat162_rn(v[2], v[3]);
+            if (na < g.total) *(__nv_bfloat162 *)(o + (size_t)na * 16 + co) = __floats2bfloat162_rn(v[0], v[1]);
+            if (nb < g.total) *(__nv_bfloat162 *)(o + (size_t)nb * 16 + co) = __floats2bfloat162_rn(v[2], v[3]);
         }
     }
 }
 
+// ---------------------------------------------------------------- tiles
+// The layers that read hidden activations work on tiles of tx x ty nodes and
+// TL_Z planes, staged with a one-node halo in shared memory as one list of
+// rows (x fastest, then y, then z; W = tx + 2 rows per line, H = ty + 2 lines
+// per plane; zero rows beyond closed faces).  In that list the neighbour at
+// offset (dx, dy, dz) of row p is row p + dx + W dy + W H dz for every p, so
+// a layer's 27 shifted operands are the same rows from 27 starting points.  A
+// plane's outputs are the TC_M rows from its first node on; tx and ty are
+// chosen so that these hold all of them (rows that fall on the halo are
+// computed and dropped).  The eight channels of each half of a row have
+// their own plane of 16-byte rows.
+constexpr int TC_M = 128;
+constexpr int TL_Z = 2;
+constexpr int TL_T = 256;   // threads of a block: one per output row of the planes
+constexpr int TL_U = 4;     // rows a thread has in flight while staging
+struct NetTile {
+    int tx, ty, W, H;       // nodes per tile along x and y, padded extents
+    int ntx, nty, ntz;      // tiles per sample
+    int rows;               // staged rows, with the slack the last plane's shifted operands reach
+};
+__host__ inline int split_even(int n, int most) { return (n + (n + most - 1) / most - 1) / ((n + most - 1) / most); }
+__host__ inline NetTile make_tile(const NetGrid &g)
+{
+    NetTile T;
+    T.tx = split_even(g.nx, 30);
+    T.W = T.tx + 2;
+    T.ty = split_even(g.ny, (TC_M - T.tx) / T.W + 1);
+    T.H = T.ty + 2;
+    T.ntx = (g.nx + T.tx - 1) / T.tx;
+    T.nty = (g.ny + T.ty - 1) / T.ty;
+    T.ntz = (g.nz + TL_Z - 1) / TL_Z;
+    T.rows = T.W * T.H * (TL_Z + 2) + TC_M;
+    return T;
+}
+struct TilePos {
+    int x0, y0, z0, base;   // first node of the tile and of its sample
+};
+__device__ __forceinline__ TilePos tile_pos(const NetGrid &g, const NetTile &T, int blk)
+{
+    TilePos P;
+    int t = blk / T.ntx;
+    P.x0 = (blk - t * T.ntx) * T.tx;
+    int u = t / T.nty;
+    P.y0 = (t - u * T.nty) * T.ty;
+    const int s = u / T.ntz;
+    P.z0 = (u - s * T.ntz) * TL_Z;
+    P.base = s * g.N;
+    return P;
+}
+// rows of the tile and its halo into sA (two planes of T.rows 16-byte rows);
+// the slack rows are zeroed
+__device__ __forceinline__ void tile_stage(const NetGrid &g, const NetTile &T, const TilePos &P,
+                                           const __nv_bfloat16 *__restrict__ in, uint4 *sA)
+{
+    const int WH = T.W * T.H, real = WH * (TL_Z + 2);
+    for (int p0 = threadIdx.x; p0 < T.rows; p0 += TL_U * TL_T) {
+        uint4 v[TL_U][2];
+#pragma unroll
+        for (int u = 0; u < TL_U; u++) {
+            const int p = p0 + u * TL_T;
+            v[u][0] = v[u][1] = make_uint4(0u, 0u, 0u, 0u);
+            if (p >= real) continue;
+            const int lz = p / WH, r = p - lz * WH, ly = r / T.W, lx = r - ly * T.W;
+            int X = P.x0 + lx - 1, Y = P.y0 + ly - 1, Z = P.z0 + lz - 1;
+            // rows past a ragged tile's last neighbour are never used
+            bool ok = X <= g.nx && Y <= g.ny && Z <= g.nz;
+            if (X < 0 || X >= g.nx) {
+                ok = ok && g.per[0];
+                X = X < 0 ? X + g.nx : X - g.nx;
+            }
+            if (Y < 0 || Y >= g.ny) {
+                ok = ok && g.per[1];
+                Y = Y < 0 ? Y + g.ny : Y - g.ny;
+            }
+            if (Z < 0 || Z >= g.nz) {
+                ok = ok && g.per[2];
+                Z = Z < 0 ? Z + g.nz : Z - g.nz;
+            }
+            if (ok) {
+                const uint4 *src = (const uint4 *)(in + (size_t)(P.base + X + g.nx * (Y + g.ny * Z)) * 16);
+                v[u][0] = __ldg(src);
+                v[u][1] = __ldg(src + 1);
+            }
+        }
+#pragma unroll
+        for (int u = 0; u < TL_U; u++) {
+            const int p = p0 + u * TL_T;
+            if (p >= T.rows) continue;
+            sA[p] = v[u][0];
+            sA[T.rows + p] = v[u][1];
+        }
+    }
+}
+// node of output row r (0 .. TC_M - 1) of the tile's plane lz, -1 on halo rows and past the grid
+__device__ __forceinline__ int tile_node(const NetGrid &g, const NetTile &T, const TilePos &P, int r, int lz)
+{
+    const int q = r + 1, ly = q / T.W, lx = q - ly * T.W - 1;  // row r is (lx, ly) + the first node
+    const int X = P.x0 + lx, Y = P.y0 + ly, Z = P.z0 + lz;
+    if (lx < 0 || lx >= T.tx || ly >= T.ty || X >= g.nx || Y >= g.ny || Z >= g.nz) return -1;
+    return P.base + X + g.nx * (Y + g.ny * Z);
+}
+
 // ---------------------------------------------------------------- 16 -> 16 on tcgen05
 // The same layer as an implicit GEMM on the fifth-generation tensor cores:
-// a block takes 128 consecutive nodes (M = 128), N = 16 output channels, and
-// K = 27 offsets x 16 input channels as 27 MMAs of K = 16 (one per offset),
-// BF16 operands from shared memory, FP32 accumulation in tensor memory.
-//   * A (per offset): the 16 input channels of each node's neighbour, 128 x 16
-//     BF16, K-major without swizzle: core matrices of 8 rows x 16 bytes,
-//     row-group g and K-half h at byte g * 256 + h * 128 (LBO = 128 between
-//     the K-halves, SBO = 256 between row groups);
-//   * B (per offset): W[co][ci], 16 x 16 BF16, the same layout;
-//   * D: TMEM lanes 0..127 = nodes, columns 0..15 = output channels; warp w
-//     reads lanes 32w..32w+31 back with tcgen05.ld (32x32b, 16 columns).
-// One thread issues the 27 MMAs and commits them to an mbarrier; the wait is
-// bounded (on giving up the block raises tc_status and skips the epilogue),
-// and the block frees its tensor memory on every path.
-constexpr int TC_M = 128;
-constexpr int TC_A_BYTES = TC_M * 32;           // one offset's A tile
+// per plane of a tile M = 128 rows, N = 16 output channels, and K = 27 offsets
+// x 16 input channels as 27 MMAs of K = 16 (one per offset), BF16 operands
+// from shared memory, FP32 accumulation in tensor memory.
+//   * A (per offset): the tile's rows from the plane's first node plus the
+//     offset's shift, K-major without swizzle: core matrices of 8 rows x 16
+//     bytes are 128 contiguous bytes (SBO), the K-halves lie a plane apart
+//     (LBO), and the start address (16-byte units) carries the shift, so no
+//     operand is staged twice;
+//   * B (per offset): W[co][ci], 16 x 16 BF16, row-group g and K-half h at
+//     byte g * 256 + h * 128;
+//   * D: TMEM lanes = rows, 16 columns per plane; warp w reads lanes
+//     32w..32w+31 back with tcgen05.ld (32x32b, 16 columns).
+// One thread issues the MMAs of all planes and commits them to an mbarrier;
+// the wait is bounded (on giving up the block raises tc_status and skips the
+// epilogue), and the block frees its tensor memory on every path.
+// What bounds it: staging.  With a copy of the rows per offset (27 x 4 KB a
+// block, one block per SM) a 65 536-node layer took 45 us, now 11 us.
 constexpr int TC_B_BYTES = 16 * 32;             // one offset's B tile
-constexpr int TC_SMEM = K27 * (TC_A_BYTES + TC_B_BYTES) + 64;
+constexpr int TC_SMEM_MOST = 72 * 1024;          // above any tile shape's (55 KB at most)
+constexpr int TC_COLS = TL_Z * 16;              // TMEM columns (a power of two, at least 32)
 
 __device__ int tc_status;  // nonzero after a bounded wait gave up
 
@@ -238,50 +379,37 @@ __device__ __forceinline__ uint32_t tc_wait(uint64_t *mbar)
     return done;
 }
 
+inline size_t tc_smem(const NetTile &T) { return (size_t)T.rows * 32 + K27 * TC_B_BYTES + 64; }
+
 template <bool RELU>
-__global__ void __launch_bounds__(TC_M) conv16_tc(NetGrid g, const __nv_bfloat16 *__restrict__ in,
+__global__ void __launch_bounds__(TL_T) conv16_tc(NetGrid g, NetTile T, const __nv_bfloat16 *__restrict__ in,
                                                   const __nv_bfloat16 *__restrict__ Wt,
                                                   const float *__restrict__ bias, int flip,
                                                   __nv_bfloat16 *__restrict__ out,
                                                   const __nv_bfloat16 *__restrict__ relu_mask_src)
 {
     extern __shared__ __align__(1024) uint8_t tc_sm[];
-    uint8_t *sA = tc_sm;                              // [27][TC_A_BYTES]
-    uint8_t *sB = tc_sm + K27 * TC_A_BYTES;           // [27][TC_B_BYTES]
+    uint8_t *sB = tc_sm;                              // [27][TC_B_BYTES]
     uint64_t *mbar = (uint64_t *)(sB + K27 * TC_B_BYTES);
     uint32_t *tmem_slot = (uint32_t *)(mbar + 1);
+    uint4 *sA = (uint4 *)(sB + K27 * TC_B_BYTES + 64);  // [2][T.rows]
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-    const int n = blockIdx.x * TC_M + tid;
-    const bool valid = n < g.N;
 
-    // tensor memory: 32 columns (the smallest allocation) for the 16 of D
     if (warp == 0) {
-        asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], 32;\n" ::"r"(smem_u32(tmem_slot)));
+        asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;\n" ::"r"(smem_u32(tmem_slot)),
+                     "n"(TC_COLS));
         asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;\n");
     }
     if (tid == 0) {
         asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;\n" ::"r"(smem_u32(mbar)));
     }
-    // operands: B tiles (weights of every offset), A tiles (this thread's
-    // node's neighbour at every offset, zero beyond a closed face)
-    for (int t = tid; t < K27 * 16 * 2; t += TC_M) {
+    for (int t = tid; t < K27 * 16 * 2; t += TL_T) {
         const int k = t >> 5, co = (t >> 1) & 15, h = t & 1;
         const uint4 v = *(const uint4 *)(Wt + ((size_t)k * 16 + co) * 16 + 8 * h);
         *(uint4 *)(sB + k * TC_B_BYTES + tc_off(co, 8 * h)) = v;
     }
-    int X = 0, Y = 0, Z = 0;
-    if (valid) xyz_of(g, n, X, Y, Z);
-    for (int k = 0; k < K27; k++) {
-        const int j = valid ? nbr_off(g, X, Y, Z, flip ? 26 - k : k) : -1;
-        uint4 v0 = make_uint4(0u, 0u, 0u, 0u), v1 = v0;
-        if (j >= 0) {
-            const uint4 *src = (const uint4 *)(in + (size_t)j * 16);
-            v0 = src[0];
-            v1 = src[1];
-        }
-        *(uint4 *)(sA + k * TC_A_BYTES + tc_off(tid, 0)) = v0;
-        *(uint4 *)(sA + k * TC_A_BYTES + tc_off(tid, 8)) = v1;
-    }
+    const TilePos P = tile_pos(g, T, blockIdx.x);
+    tile_stage(g, T, P, in, sA);
     // make the generic-proxy writes visible to the tensor cores' async proxy
     asm volatile("fence.proxy.async.shared::cta;\n" ::: "memory");
     asm volatile("tcgen05.fence::before_thread_sync;\n" ::: "memory");
@@ -290,14 +418,20 @@ __global__ void __launch_bounds__(TC_M) conv16_tc(NetGrid g, const __nv_bfloat16
     const uint32_t tmem = *tmem_slot;
     if (tid == 0) {
         const uint32_t a0 = smem_u32(sA), b0 = smem_u32(sB);
-        for (int k = 0; k < K27; k++) {
-            const uint64_t ad = tc_desc(a0 + k * TC_A_BYTES, 128, 256);
-            const uint64_t bd = tc_desc(b0 + k * TC_B_BYTES, 128, 256);
-            const uint32_t acc = k > 0;
-            asm volatile(
-                "{\n .reg .pred p;\n setp.ne.b32 p, %4, 0;\n"
-                " tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n}\n" ::"r"(tmem),
-                "l"(ad), "l"(bd), "r"(TC_IDESC), "r"(acc));
+        const int WH = T.W * T.H;
+        for (int z = 0; z < TL_Z; z++) {
+            const int first = 1 + T.W + WH * (z + 1);  // the plane's first node
+            for (int k = 0; k < K27; k++) {
+                const int kk = flip ? 26 - k : k;
+                const int row = first + (kk % 3 - 1) + T.W * ((kk / 3) % 3 - 1) + WH * (kk / 9 - 1);
+                const uint64_t ad = tc_desc(a0 + 16u * (uint32_t)row, 16u * (uint32_t)T.rows, 128);
+                const uint64_t bd = tc_desc(b0 + k * TC_B_BYTES, 128, 256);
+                const uint32_t acc = k > 0;
+                asm volatile(
+                    "{\n .reg .pred p;\n setp.ne.b32 p, %4, 0;\n"
+                    " tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n}\n" ::"r"(tmem + 16u * (uint32_t)z),
+                    "l"(ad), "l"(bd), "r"(TC_IDESC), "r"(acc));
+            }
         }
         asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];\n" ::"r"(
             smem_u32(mbar)));
@@ -311,8 +445,12 @@ __global__ void __launch_bounds__(TC_M) conv16_tc(NetGrid g, const __nv_bfloat16
         if (lane == 0) atomicExch(&tc_status, 1);
         done = tc_wait(mbar);
     } else {
+        // warps 0-3 read the first plane's columns, warps 4-7 the second's
+        // (a warp reaches the 32 lanes of its number modulo 4)
+        static_assert(TL_T == TL_Z * TC_M, "one warp group per plane");
+        const int z = warp >> 2;
         uint32_t d[16];
-        const uint32_t taddr = tmem + ((uint32_t)(warp * 32) << 16);
+        const uint32_t taddr = tmem + 16u * (uint32_t)z + ((uint32_t)((warp & 3) * 32) << 16);
         asm volatile(
             "tcgen05.ld.sync.aligned.32x32b.x16.b32 {%0, %1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, "
             "%14, %15}, [%16];\n"
@@ -320,23 +458,33 @@ __global__ void __launch_bounds__(TC_M) conv16_tc(NetGrid g, const __nv_bfloat16
               "=r"(d[8]), "=r"(d[9]), "=r"(d[10]), "=r"(d[11]), "=r"(d[12]), "=r"(d[13]), "=r"(d[14]), "=r"(d[15])
             : "r"(taddr));
         asm volatile("tcgen05.wait::ld.sync.aligned;\n" ::: "memory");
-        if (valid) {
+        const int n = tile_node(g, T, P, tid & (TC_M - 1), z);
+        if (n >= 0) {
+            uint4 m[2];
+            if (relu_mask_src) {
+                m[0] = __ldg((const uint4 *)(relu_mask_src + (size_t)n * 16));
+                m[1] = __ldg((const uint4 *)(relu_mask_src + (size_t)n * 16) + 1);
+            }
+            const __nv_bfloat16 *mv = (const __nv_bfloat16 *)m;
             float v[16];
 #pragma unroll
             for (int co = 0; co < 16; co++) {
                 v[co] = __uint_as_float(d[co]) + (bias ? bias[co] : 0.f);
                 if (RELU) v[co] = fmaxf(v[co], 0.f);
                 // gradient through the ReLU of the layer that produced relu_mask_src
-                if (relu_mask_src && !(__bfloat162float(relu_mask_src[(size_t)n * 16 + co]) > 0.f)) v[co] = 0.f;
+                if (relu_mask_src && !(__bfloat162float(mv[co]) > 0.f)) v[co] = 0.f;
             }
-            __nv_bfloat162 *o = (__nv_bfloat162 *)(out + (size_t)n * 16);
+            __align__(16) __nv_bfloat162 o[8];
 #pragma unroll
             for (int c = 0; c < 8; c++) o[c] = __floats2bfloat162_rn(v[2 * c], v[2 * c + 1]);
+            uint4 *dst = (uint4 *)(out + (size_t)n * 16);
+            dst[0] = ((const uint4 *)o)[0];
+            dst[1] = ((const uint4 *)o)[1];
         }
     }
     asm volatile("tcgen05.fence::before_thread_sync;\n" ::: "memory");
     __syncthreads();
-    if (warp == 0) asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, 32;\n" ::"r"(tmem));
+    if (warp == 0) asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;\n" ::"r"(tmem), "n"(TC_COLS));
 }
 
 // which kernel runs the 16 -> 16 layers: 1 = tcgen05 (default), 0 = mma.sync
@@ -347,62 +495,82 @@ void conv16(const NetGrid &g, const __nv_bfloat16 *in, const __nv_bfloat16 *Wt, 
             __nv_bfloat16 *out, const __nv_bfloat16 *relu_mask_src, cudaStream_t s)
 {
     if (g_tensor_path) {
-        static bool attr = false;
-        if (!attr) {
-            cudaFuncSetAttribute(conv16_tc<RELU>, cudaFuncAttributeMaxDynamicSharedMemorySize, TC_SMEM);
-            attr = true;
-        }
-        conv16_tc<RELU><<<(g.N + TC_M - 1) / TC_M, TC_M, TC_SMEM, s>>>(g, in, Wt, bias, flip, out, relu_mask_src);
+        const NetTile T = make_tile(g);
+        static std::once_flag attr;  // the largest tile of any grid
+        std::call_once(attr, [] {
+            cudaFuncSetAttribute(conv16_tc<RELU>, cudaFuncAttributeMaxDynamicSharedMemorySize, TC_SMEM_MOST);
+        });
+        const int blocks = T.ntx * T.nty * T.ntz * (g.total / g.N);
+        conv16_tc<RELU><<<blocks, TL_T, tc_smem(T), s>>>(g, T, in, Wt, bias, flip, out, relu_mask_src);
     } else {
-        conv16_mma<RELU, false><<<(g.N + 127) / 128, 256, 0, s>>>(g, in, Wt, bias, flip, out, relu_mask_src);
+        conv16_mma<RELU, false><<<(g.total + 127) / 128, 256, 0, s>>>(g, in, Wt, bias, flip, out, relu_mask_src);
     }
 }
 
-// BF16 B-operand tables of a 16->16 layer: forward Wt[k][co][ci] = W[co][ci][k];
-// data gradient Wb[k][ci][co] = W[co][ci][k] (used with flipped offsets).
-__global__ void prep_w16(const float *__restrict__ w, int ow, __nv_bfloat16 *__restrict__ Wf, __nv_bfloat16 *__restrict__ Wb)
+// BF16 B-operand tables of the two 16->16 layers: forward Wt[k][co][ci] =
+// W[co][ci][k]; data gradient Wb[k][ci][co] = W[co][ci][k] (used with flipped
+// offsets).
+__global__ void prep_w16(const float *__restrict__ w, __nv_bfloat16 *__restrict__ W2f, __nv_bfloat16 *__restrict__ W2b,
+                         __nv_bfloat16 *__restrict__ W3f, __nv_bfloat16 *__restrict__ W3b)
 {
     int t = blockIdx.x * blockDim.x + threadIdx.x;
-    if (t >= 27 * 16 * 16) return;
-    int k = t / 256, r = t % 256, co = r / 16, ci = r % 16;
-    float v = w[ow + (co * 16 + ci) * 27 + k];
-    Wf[(k * 16 + co) * 16 + ci] = __float2bfloat16_rn(v);
-    Wb[(k * 16 + ci) * 16 + co] = __float2bfloat16_rn(v);
+    const bool third = t >= 27 * 256;
+    if (third) t -= 27 * 256;
+    if (t >= 27 * 256) return;
+    const int k = t / 256, r = t % 256, co = r / 16, ci = r % 16;
+    const __nv_bfloat16 v = __float2bfloat16_rn(w[(third ? OW3 : OW2) + (co * 16 + ci) * 27 + k]);
+    (third ? W3f : W2f)[(k * 16 + co) * 16 + ci] = v;
+    (third ? W3b : W2b)[(k * 16 + ci) * 16 + co] = v;
 }
 
 // ---------------------------------------------------------------- layer 4
-__global__ void __launch_bounds__(NT) l4_fwd(NetGrid g, const __nv_bfloat16 *__restrict__ act, const float *__restrict__ w,
-                                             float *__restrict__ y)
+// y[n] = b4 + sum_k sum_ci W4[ci][k] act[n + off_k][ci] in FP32, one thread
+// per row of a staged tile's plane (27 row reads of 32 bytes each: from
+// shared memory, not from L1 with the neighbours' indices worked out per
+// offset: 11 us for 65 536 nodes against 23)
+__global__ void __launch_bounds__(TL_T) l4_fwd(NetGrid g, NetTile T, const __nv_bfloat16 *__restrict__ act,
+                                               const float *__restrict__ w, float *__restrict__ y)
 {
-    __shared__ float sw[16 * 27 + 1];
-    for (int t = threadIdx.x; t < 16 * 27 + 1; t += blockDim.x) sw[t] = w[OW4 + t];
+    extern __shared__ __align__(1024) uint8_t tc_sm[];
+    float *sw = (float *)tc_sm;                              // [offset][channel], then the bias
+    uint4 *sA = (uint4 *)(tc_sm + K27 * TC_B_BYTES + 64);    // as in conv16_tc
+    for (int t = threadIdx.x; t < 16 * 27; t += blockDim.x) sw[(t % 27) * 16 + t / 27] = w[OW4 + t];
+    if (threadIdx.x == 0) sw[16 * 27] = w[OB4];
+    const TilePos P = tile_pos(g, T, blockIdx.x);
+    tile_stage(g, T, P, act, sA);
     __syncthreads();
-    const int n = blockIdx.x * blockDim.x + threadIdx.x;
-    if (n >= g.N) return;
-    int X, Y, Z;
-    xyz_of(g, n, X, Y, Z);
-    float acc = sw[16 * 27];
-    for (int k = 0; k < K27; k++) {
-        const int j = nbr_off(g, X, Y, Z, k);
-        if (j < 0) continue;
-        const __nv_bfloat162 *a = (const __nv_bfloat162 *)(act + (size_t)j * 16);
-        for (int c = 0; c < 8; c++) {
-            float2 v = __bfloat1622float2(a[c]);
-            acc += sw[(2 * c) * 27 + k] * v.x + sw[(2 * c + 1) * 27 + k] * v.y;
+    const int WH = T.W * T.H;
+    const int z = threadIdx.x / TC_M, r = threadIdx.x & (TC_M - 1);
+    const int n = tile_node(g, T, P, r, z);
+    if (n >= 0) {
+        const int first = 1 + T.W + WH * (z + 1) + r;
+        float acc = sw[16 * 27];
+#pragma unroll 3
+        for (int k = 0; k < K27; k++) {
+            const int row = first + (k % 3 - 1) + T.W * ((k / 3) % 3 - 1) + WH * (k / 9 - 1);
+            const uint4 v[2] = {sA[row], sA[T.rows + row]};
+            const __nv_bfloat162 *a = (const __nv_bfloat162 *)v;
+#pragma unroll
+            for (int c = 0; c < 8; c++) {
+                const float2 f = __bfloat1622float2(a[c]);
+                acc += sw[16 * k + 2 * c] * f.x + sw[16 * k + 2 * c + 1] * f.y;
+            }
         }
+        y[n] = acc;
     }
-    y[n] = acc;
 }
 
-// loss gradient g = 2 (y - t) / cnt on masked nodes; per-block loss partials
-__global__ void __launch_bounds__(NT) loss_grad_k(int N, const float *y, const float *t, const uint8_t *mask, float inv_cnt,
-                                                  float *g, double *part)
+// loss gradient g = 2 (y - t) / cnt on masked nodes (target of sample s:
+// t + N smp[s]); per-block loss partials
+__global__ void __launch_bounds__(NT) loss_grad_k(NetGrid gr, const float *y, const float *t, const int *smp,
+                                                  const uint8_t *mask, float inv_cnt, float *g, double *part)
 {
     __shared__ double sh[NT / 32];
     const int n = blockIdx.x * blockDim.x + threadIdx.x;
     float l = 0.f;
-    if (n < N) {
-        float d = (mask == nullptr || mask[n]) ? y[n] - t[n] : 0.f;
+    if (n < gr.total) {
+        const int s = n / gr.N, i = n - s * gr.N;
+        float d = (mask == nullptr || mask[i]) ? y[n] - t[(size_t)gr.N * (smp ? smp[s] : s) + i] : 0.f;
         g[n] = 2.f * d * inv_cnt;
         l = d * d;
     }
@@ -410,24 +578,43 @@ __global__ void __launch_bounds__(NT) loss_grad_k(int N, const float *y, const f
     if (threadIdx.x == 0) part[blockIdx.x] = s;
 }
 
+// loss[0] (+)= scale * (sum of the block partials, in a fixed order)
+__global__ void __launch_bounds__(NT) loss_sum_k(const double *part, int n, double scale, int add, double *loss)
+{
+    __shared__ double sh[NT / 32];
+    double v = 0.0;
+    for (int k = threadIdx.x; k < n; k += blockDim.x) v += part[k];
+    const double t = block_sum(v, sh);
+    if (threadIdx.x == 0) *loss = (add ? *loss : 0.0) + scale * t;
+}
+
 // d_act3[m][ci] = relu'(act3) * sum_k W4[ci][k] g[m - off_k]  (BF16 out)
 __global__ void __launch_bounds__(NT) l4_bwd_data(NetGrid g, const float *__restrict__ gy, const float *__restrict__ w,
                                                   const __nv_bfloat16 *__restrict__ act3, __nv_bfloat16 *__restrict__ dz)
 {
-    __shared__ float sw[16 * 27];
-    for (int t = threadIdx.x; t < 16 * 27; t += blockDim.x) sw[t] = w[OW4 + t];
+    __shared__ __align__(16) float sw[16 * 27];  // [offset][channel]
+    for (int t = threadIdx.x; t < 16 * 27; t += blockDim.x) sw[(t % 27) * 16 + t / 27] = w[OW4 + t];
     __syncthreads();
     const int m = blockIdx.x * blockDim.x + threadIdx.x;
-    if (m >= g.N) return;
+    if (m >= g.total) return;
     int X, Y, Z;
-    xyz_of(g, m, X, Y, Z);
+    const int base = sample_xyz(g, m, X, Y, Z);
     float acc[16];
+#pragma unroll
     for (int c = 0; c < 16; c++) acc[c] = 0.f;
+#pragma unroll 3
     for (int k = 0; k < K27; k++) {
         const int j = nbr_off(g, X, Y, Z, 26 - k);  // m - off_k
         if (j < 0) continue;
-        const float gv = gy[j];
-        for (int c = 0; c < 16; c++) acc[c] += sw[c * 27 + k] * gv;
+        const float gv = gy[base + j];
+#pragma unroll
+        for (int c = 0; c < 16; c += 4) {
+            const float4 w4 = *(const float4 *)(sw + 16 * k + c);
+            acc[c] += w4.x * gv;
+            acc[c + 1] += w4.y * gv;
+            acc[c + 2] += w4.z * gv;
+            acc[c + 3] += w4.w * gv;
+        }
     }
     for (int c = 0; c < 16; c += 2) {
         float v0 = __bfloat162float(act3[(size_t)m * 16 + c]) > 0.f ? acc[c] : 0.f;
@@ -437,74 +624,190 @@ __global__ void __launch_bounds__(NT) l4_bwd_data(NetGrid g, const float *__rest
 }
 
 // ---------------------------------------------------------------- weight gradients
-// Per-block partials of dW[co][ci][k] = sum_n dz[n][co] a[ci][n + off_k] and
-// db[co] = sum_n dz[n][co], for CI input channels stored either as BF16
-// node-major [n][16] (hidden) or FP32 channel-major [ci][N] (network input),
-// CO output channels stored as BF16 [n][16] or FP32 [N] (CO = 1).
+// dW[co][ci][k] = sum_n dz[n][co] a[ci][n + off_k], db[co] = sum_n dz[n][co],
+// with a BF16 node-major [n][16] (CI = 16) or the FP32 network input (CI = 2),
+// dz BF16 [n][16] (CO = 16) or FP32 [n] (CO = 1).  FP32 sums in a fixed
+// order: WG_CH consecutive nodes of a sample in one FMA chain, the chains of
+// a block's WG_NODES nodes added in order, one partial per block, the
+// partials of a sample added in order (grad_reduce), then the samples.
+//
+// A block stages the 27 neighbour rows of WG_CH nodes as FP32 in shared
+// memory (16 bytes of BF16 channels per load, the next chunk's loads in
+// flight under this chunk's arithmetic), and a thread keeps 4 x 4 outputs (4
+// output by 4 input channels of one offset), so two 16-byte shared loads feed
+// 16 FMAs.  What bounds it: FMA issue, 6928 per node for a 16 -> 16 layer.
+// The form before gathered one value per thread with its index arithmetic and
+// two scalar shared loads per FMA: 710 us per layer on an 8192-node sample,
+// against 30 us now for eight samples in one launch.
+constexpr int WG_CH = 16;
+constexpr int WG_NODES = 512;
+constexpr int WG_T = 448;
+
+template <int CI, int CO> constexpr int wg_smem() { return 2 * WG_CH * (27 * CI + CO) * (int)sizeof(float); }
+
 template <int CI, int CO>
-__global__ void __launch_bounds__(NT) wgrad_partial(NetGrid g, const void *a_in, int a_bf16, const void *dz, int dz_bf16,
-                                                    float *part)
+__global__ void __launch_bounds__(WG_T) wgrad_k(NetGrid g, NetInput in, const __nv_bfloat16 *__restrict__ a,
+                                                const void *__restrict__ dz, float *__restrict__ part)
 {
     constexpr int NW = CO * CI * 27 + CO;
-    constexpr int CH = 16;  // nodes per shared-memory chunk
-    __shared__ float sa[CH][CI][27];
-    __shared__ float sd[CH][CO];
-    float acc[(NW + NT - 1) / NT];
-    for (int q = 0; q < (NW + NT - 1) / NT; q++) acc[q] = 0.f;
-    const int base = blockIdx.x * 512;
-    for (int chunk = 0; chunk < 512; chunk += CH) {
-        __syncthreads();
-        for (int t = threadIdx.x; t < CH * CI * 27; t += blockDim.x) {
-            int nn = t / (CI * 27), r = t % (CI * 27), ci = r / 27, k = r % 27;
-            int n = base + chunk + nn;
-            float v = 0.f;
-            if (n < g.N) {
-                int X, Y, Z;
-                xyz_of(g, n, X, Y, Z);
-                int j = nbr_off(g, X, Y, Z, k);
-                if (j >= 0)
-                    v = a_bf16 ? __bfloat162float(((const __nv_bfloat16 *)a_in)[(size_t)j * 16 + ci])
-                               : ((const float *)a_in)[(size_t)ci * g.N + j];
-            }
-            sa[nn][ci][k] = v;
-        }
-        for (int t = threadIdx.x; t < CH * CO; t += blockDim.x) {
-            int nn = t / CO, co = t % CO, n = base + chunk + nn;
-            float v = 0.f;
-            if (n < g.N)
-                v = dz_bf16 ? __bfloat162float(((const __nv_bfloat16 *)dz)[(size_t)n * 16 + co])
-                            : ((const float *)dz)[n];
-            sd[nn][co] = v;
-        }
-        __syncthreads();
-        for (int q = 0; q < (NW + NT - 1) / NT; q++) {
-            int wi = q * NT + threadIdx.x;
-            if (wi >= NW) break;
-            float s = 0.f;
-            if (wi < CO * CI * 27) {
-                int co = wi / (CI * 27), r = wi % (CI * 27), ci = r / 27, k = r % 27;
-                for (int nn = 0; nn < CH; nn++) s += sd[nn][co] * sa[nn][ci][k];
-            } else {
-                int co = wi - CO * CI * 27;
-                for (int nn = 0; nn < CH; nn++) s += sd[nn][co];
-            }
-            acc[q] += s;
-        }
+    constexpr int VC = CI == 16 ? 8 : 1;                 // channels per staged load
+    constexpr int PER = 27 * CI / VC;                    // loads per node (54)
+    constexpr int LOADS = (WG_CH * PER + WG_T - 1) / WG_T;
+    constexpr int TI = CI == 16 ? 4 : 1, TO = CO == 16 ? 4 : 1;  // outputs per thread
+    constexpr int JI = 27 * CI / TI, JO = CO / TO;       // thread grid
+    static_assert(JI * JO + CO <= WG_T, "threads");
+    // double-buffered chunks (57 KB for a 16 -> 16 layer: dynamic)
+    extern __shared__ __align__(1024) uint8_t tc_sm[];
+    float(*sa)[WG_CH][27 * CI] = (float(*)[WG_CH][27 * CI])tc_sm;
+    float(*sd)[WG_CH][CO] = (float(*)[WG_CH][CO])(tc_sm + 2 * sizeof(float) * WG_CH * 27 * CI);
+    const int per_sample = (g.N + WG_NODES - 1) / WG_NODES;
+    const int s = blockIdx.x / per_sample, base = (blockIdx.x - s * per_sample) * WG_NODES;
+    const float *x = CI == 16 ? nullptr : sample_x(g, in, s);
+    const int tid = threadIdx.x;
+    // this thread's staged loads: node nn of the chunk, offset k, channels
+    int nn_[LOADS], k_[LOADS], c_[LOADS];
+#pragma unroll
+    for (int l = 0; l < LOADS; l++) {
+        const int it = tid + l * WG_T;
+        nn_[l] = it < WG_CH * PER ? it / PER : -1;
+        const int r = it - (it / PER) * PER;
+        k_[l] = CI == 16 ? r >> 1 : r % 27;
+        c_[l] = CI == 16 ? 8 * (r & 1) : r / 27;
     }
-    for (int q = 0; q < (NW + NT - 1) / NT; q++) {
-        int wi = q * NT + threadIdx.x;
-        if (wi < NW) part[(size_t)blockIdx.x * NW + wi] = acc[q];
+    uint4 va[LOADS];
+    float vx[LOADS], vd1 = 0.f;
+    uint4 vd = make_uint4(0u, 0u, 0u, 0u);
+    auto load = [&](int chunk) {
+#pragma unroll
+        for (int l = 0; l < LOADS; l++) {
+            va[l] = make_uint4(0u, 0u, 0u, 0u);
+            vx[l] = 0.f;
+            const int n = base + chunk + nn_[l];
+            if (nn_[l] < 0 || n >= g.N) continue;
+            int X, Y, Z;
+            xyz_of(g, n, X, Y, Z);
+            const int j = nbr_off(g, X, Y, Z, k_[l]);
+            if (j < 0) continue;
+            if constexpr (CI == 16)
+                va[l] = __ldg((const uint4 *)(a + ((size_t)s * g.N + j) * 16 + c_[l]));
+            else
+                vx[l] = __ldg(x + (size_t)c_[l] * g.N + j);
+        }
+        if (tid < WG_CH * (CO == 16 ? 2 : 1)) {
+            const int n = base + chunk + (CO == 16 ? tid >> 1 : tid);
+            vd = make_uint4(0u, 0u, 0u, 0u);
+            vd1 = 0.f;
+            if (n < g.N) {
+                if constexpr (CO == 16)
+                    vd = __ldg((const uint4 *)((const __nv_bfloat16 *)dz + ((size_t)s * g.N + n) * 16 + 8 * (tid & 1)));
+                else
+                    vd1 = __ldg((const float *)dz + (size_t)s * g.N + n);
+            }
+        }
+    };
+    auto unpack = [](const uint4 &v, float *dst) {
+        const __nv_bfloat162 *p = (const __nv_bfloat162 *)&v;
+        const float2 f0 = __bfloat1622float2(p[0]), f1 = __bfloat1622float2(p[1]), f2 = __bfloat1622float2(p[2]),
+                     f3 = __bfloat1622float2(p[3]);
+        ((float4 *)dst)[0] = make_float4(f0.x, f0.y, f1.x, f1.y);
+        ((float4 *)dst)[1] = make_float4(f2.x, f2.y, f3.x, f3.y);
+    };
+    auto store = [&](int buf) {
+#pragma unroll
+        for (int l = 0; l < LOADS; l++) {
+            if (nn_[l] < 0) continue;
+            float *dst = &sa[buf][nn_[l]][k_[l] * CI + c_[l]];
+            if constexpr (CI == 16) unpack(va[l], dst);
+            else *dst = vx[l];
+        }
+        if constexpr (CO == 16) {
+            if (tid < 2 * WG_CH) unpack(vd, &sd[buf][tid >> 1][8 * (tid & 1)]);
+        } else {
+            if (tid < WG_CH) sd[buf][tid][0] = vd1;
+        }
+    };
+    const int ji = tid % JI, jo = tid / JI;
+    const bool mine = tid < JI * JO, bias = tid >= JI * JO && tid < JI * JO + CO;
+    float acc[TO][TI], accb = 0.f;
+#pragma unroll
+    for (int o = 0; o < TO; o++)
+#pragma unroll
+        for (int i = 0; i < TI; i++) acc[o][i] = 0.f;
+    load(0);
+    store(0);
+    __syncthreads();
+    const int nodes = min(WG_NODES, g.N - base);
+    int buf = 0;
+    for (int chunk = 0; chunk < nodes; chunk += WG_CH, buf ^= 1) {
+        const bool more = chunk + WG_CH < nodes;
+        if (more) load(chunk + WG_CH);
+        if (mine) {
+            float t[TO][TI];
+#pragma unroll
+            for (int o = 0; o < TO; o++)
+#pragma unroll
+                for (int i = 0; i < TI; i++) t[o][i] = 0.f;
+#pragma unroll
+            for (int nn = 0; nn < WG_CH; nn++) {
+                float av[TI], dv[TO];
+                if constexpr (TI == 4) *(float4 *)av = *(const float4 *)&sa[buf][nn][4 * ji];
+                else av[0] = sa[buf][nn][ji];
+                if constexpr (TO == 4) *(float4 *)dv = *(const float4 *)&sd[buf][nn][4 * jo];
+                else dv[0] = sd[buf][nn][0];
+#pragma unroll
+                for (int o = 0; o < TO; o++)
+#pragma unroll
+                    for (int i = 0; i < TI; i++) t[o][i] += dv[o] * av[i];
+            }
+#pragma unroll
+            for (int o = 0; o < TO; o++)
+#pragma unroll
+                for (int i = 0; i < TI; i++) acc[o][i] += t[o][i];
+        } else if (bias) {
+            float t = 0.f;
+#pragma unroll
+            for (int nn = 0; nn < WG_CH; nn++) t += sd[buf][nn][tid - JI * JO];
+            accb += t;
+        }
+        if (more) store(buf ^ 1);
+        __syncthreads();
+    }
+    float *P = part + (size_t)blockIdx.x * NW;
+    if (mine) {
+#pragma unroll
+        for (int o = 0; o < TO; o++)
+#pragma unroll
+            for (int i = 0; i < TI; i++) {
+                const int q = TI * ji + i, k = q / CI, ci = q - k * CI;
+                P[((TO * jo + o) * CI + ci) * 27 + k] = acc[o][i];
+            }
+    } else if (bias) {
+        P[CO * CI * 27 + tid - JI * JO] = accb;
     }
 }
 
-// grad[o + i] += sum over blocks (fixed order) of part[b][i]
-__global__ void reduce_partials(const float *part, int nblocks, int nw, float *grad, int o)
+// grad[i] (+)= sum over samples of (sum over the sample's blocks, in order, of
+// part[b][i - first parameter of its layer]), for every parameter
+__global__ void __launch_bounds__(64) grad_reduce(const float *part1, const float *part2, const float *part3,
+                                                  const float *part4, int per_sample, int ns, int add, float *grad)
 {
-    int i = blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= nw) return;
-    float s = 0.f;
-    for (int b = 0; b < nblocks; b++) s += part[(size_t)b * nw + i];
-    grad[o + i] += s;
+    const int i = blockIdx.x * blockDim.x + threadIdx.x;
+    if (i >= NPARAM) return;
+    const float *p;
+    int nw, o;
+    if (i < OW2) { p = part1; nw = OW2 - OW1; o = OW1; }
+    else if (i < OW3) { p = part2; nw = OW3 - OW2; o = OW2; }
+    else if (i < OW4) { p = part3; nw = OW4 - OW3; o = OW3; }
+    else { p = part4; nw = NPARAM - OW4; o = OW4; }
+    p += i - o;
+    float t = add ? grad[i] : 0.f;
+    for (int s = 0; s < ns; s++) {
+        float v = 0.f;
+#pragma unroll 16
+        for (int b = 0; b < per_sample; b++) v += __ldg(p + (size_t)(s * per_sample + b) * nw);
+        t += v;
+    }
+    grad[i] = t;
 }
 
 // Adam (Kingma & Ba) on the FP32 master parameters
@@ -520,104 +823,139 @@ __global__ void adam_k(int n, float *w, const float *g, float *m, float *v, floa
 }
 
 // ---------------------------------------------------------------- host side
+// Device buffers of one network pass over up to cap nodes (samples x nodes),
+// carved out of one allocation.
 struct NetWork {
     NetGrid g;
-    float *x = nullptr;         // [2][N]
+    float *x = nullptr;         // [2][N]: the in-step warm start's input
     __nv_bfloat16 *a1 = nullptr, *a2 = nullptr, *a3 = nullptr, *dz = nullptr, *dz2 = nullptr;
     float *y = nullptr, *gy = nullptr;
     float *w = nullptr, *grad = nullptr;
     __nv_bfloat16 *W2f = nullptr, *W2b = nullptr, *W3f = nullptr, *W3b = nullptr;
-    float *part = nullptr;
-    double *lpart = nullptr;
-    size_t part_floats = 0;
-    int cap = 0;
+    float *part[4] = {};        // weight-gradient partials per layer
+    double *lpart = nullptr, *loss = nullptr;
+    void *arena = nullptr;
 };
 
 int cuda_err(cudaError_t e) { return e == cudaSuccess ? EKL_OK : EKL_ERR_CUDA; }
 
-int work_alloc(NetWork &W, int N)
+constexpr int LAYER_PARAMS[4] = {OW2 - OW1, OW3 - OW2, OW4 - OW3, NPARAM - OW4};
+
+// buffers for passes over `samples` samples of W.g; `extra` bytes more
+// (256-byte aligned) at *extra_out
+int work_alloc(NetWork &W, int samples, bool train, size_t extra = 0, char **extra_out = nullptr)
 {
-    if (N <= W.cap) return EKL_OK;
-    cudaFree(W.x); cudaFree(W.a1); cudaFree(W.a2); cudaFree(W.a3); cudaFree(W.dz); cudaFree(W.dz2);
-    cudaFree(W.y); cudaFree(W.gy); cudaFree(W.part); cudaFree(W.lpart);
-    const int nblk_w = (N + 511) / 512;
-    W.part_floats = (size_t)nblk_w * (16 * 16 * 27 + 16);
-    cudaError_t e = cudaMalloc(&W.x, 2 * (size_t)N * 4);
-    if (e == cudaSuccess) e = cudaMalloc(&W.a1, (size_t)N * 32);
-    if (e == cudaSuccess) e = cudaMalloc(&W.a2, (size_t)N * 32);
-    if (e == cudaSuccess) e = cudaMalloc(&W.a3, (size_t)N * 32);
-    if (e == cudaSuccess) e = cudaMalloc(&W.dz, (size_t)N * 32);
-    if (e == cudaSuccess) e = cudaMalloc(&W.dz2, (size_t)N * 32);
-    if (e == cudaSuccess) e = cudaMalloc(&W.y, (size_t)N * 4);
-    if (e == cudaSuccess) e = cudaMalloc(&W.gy, (size_t)N * 4);
-    if (e == cudaSuccess) e = cudaMalloc(&W.part, W.part_floats * 4);
-    if (e == cudaSuccess) e = cudaMalloc(&W.lpart, ((N + NT - 1) / NT) * sizeof(double));
-    if (!W.w) {
-        if (e == cudaSuccess) e = cudaMalloc(&W.w, NPARAM * 4);
-        if (e == cudaSuccess) e = cudaMalloc(&W.grad, NPARAM * 4);
-        if (e == cudaSuccess) e = cudaMalloc(&W.W2f, 27 * 256 * 2);
-        if (e == cudaSuccess) e = cudaMalloc(&W.W2b, 27 * 256 * 2);
-        if (e == cudaSuccess) e = cudaMalloc(&W.W3f, 27 * 256 * 2);
-        if (e == cudaSuccess) e = cudaMalloc(&W.W3b, 27 * 256 * 2);
+    size_t off = 0;
+    auto carve = [&](size_t bytes) {
+        const size_t at = off;
+        off += (bytes + 255) & ~(size_t)255;
+        return at;
+    };
+    const size_t n = (size_t)samples * W.g.N;
+    const size_t ox = carve(2 * n * 4), o1 = carve(n * 32), o2 = carve(n * 32), o3 = carve(n * 32), oy = carve(n * 4);
+    const size_t ow = carve(NPARAM * 4), of2 = carve(27 * 512), ob2 = carve(27 * 512), of3 = carve(27 * 512),
+                 ob3 = carve(27 * 512);
+    size_t od = 0, od2 = 0, og = 0, ogr = 0, ol = 0, op[4] = {}, oloss = 0;
+    if (train) {
+        od = carve(n * 32);
+        od2 = carve(n * 32);
+        og = carve(n * 4);
+        ogr = carve(NPARAM * 4);
+        ol = carve(((n + NT - 1) / NT) * sizeof(double));
+        oloss = carve(sizeof(double));
+        const size_t nb = (size_t)samples * ((W.g.N + WG_NODES - 1) / WG_NODES);
+        for (int l = 0; l < 4; l++) op[l] = carve(nb * LAYER_PARAMS[l] * 4);
     }
-    if (e != cudaSuccess) return EKL_ERR_ALLOC;
-    W.cap = N;
+    const size_t oe = carve(extra);
+    if (cudaMalloc(&W.arena, off) != cudaSuccess) {
+        cudaGetLastError();
+        W.arena = nullptr;
+        return EKL_ERR_ALLOC;
+    }
+    char *b = (char *)W.arena;
+    W.x = (float *)(b + ox);
+    W.a1 = (__nv_bfloat16 *)(b + o1);
+    W.a2 = (__nv_bfloat16 *)(b + o2);
+    W.a3 = (__nv_bfloat16 *)(b + o3);
+    W.y = (float *)(b + oy);
+    W.w = (float *)(b + ow);
+    W.W2f = (__nv_bfloat16 *)(b + of2);
+    W.W2b = (__nv_bfloat16 *)(b + ob2);
+    W.W3f = (__nv_bfloat16 *)(b + of3);
+    W.W3b = (__nv_bfloat16 *)(b + ob3);
+    if (train) {
+        W.dz = (__nv_bfloat16 *)(b + od);
+        W.dz2 = (__nv_bfloat16 *)(b + od2);
+        W.gy = (float *)(b + og);
+        W.grad = (float *)(b + ogr);
+        W.lpart = (double *)(b + ol);
+        W.loss = (double *)(b + oloss);
+        for (int l = 0; l < 4; l++) W.part[l] = (float *)(b + op[l]);
+    }
+    if (extra_out) *extra_out = b + oe;
     return EKL_OK;
 }
 
 void work_free(NetWork &W)
 {
-    cudaFree(W.x); cudaFree(W.a1); cudaFree(W.a2); cudaFree(W.a3); cudaFree(W.dz); cudaFree(W.dz2);
-    cudaFree(W.y); cudaFree(W.gy); cudaFree(W.part); cudaFree(W.lpart); cudaFree(W.w); cudaFree(W.grad);
-    cudaFree(W.W2f); cudaFree(W.W2b); cudaFree(W.W3f); cudaFree(W.W3b);
+    cudaFree(W.arena);
     W = NetWork();
 }
 
-// forward pass on W.x with the parameters in W.w; output in W.y
-void net_forward(NetWork &W, cudaStream_t s)
+// BF16 copies of the 16 -> 16 layers' parameters in W.w
+void net_prepare(NetWork &W, cudaStream_t s)
 {
-    const NetGrid &g = W.g;
-    prep_w16<<<27, 256, 0, s>>>(W.w, OW2, W.W2f, W.W2b);
-    prep_w16<<<27, 256, 0, s>>>(W.w, OW3, W.W3f, W.W3b);
-    const int bn = (g.N + NT - 1) / NT;
-    l1_fwd<<<bn, NT, 0, s>>>(g, W.x, W.w, W.a1);
-    conv16<true>(g, W.a1, W.W2f, W.w + OB2, 0, W.a2, nullptr, s);
-    conv16<true>(g, W.a2, W.W3f, W.w + OB3, 0, W.a3, nullptr, s);
-    l4_fwd<<<bn, NT, 0, s>>>(g, W.a3, W.w, W.y);
+    prep_w16<<<54, 256, 0, s>>>(W.w, W.W2f, W.W2b, W.W3f, W.W3b);
 }
 
-// loss and gradient (W.grad) for target t and mask on W.x
-int net_backward(NetWork &W, const float *d_t, const uint8_t *d_mask, float inv_cnt, double *loss, cudaStream_t s)
+// forward pass over ns samples of `in` with the parameters in W.w (prepared);
+// output in W.y
+void net_forward(NetWork &W, const NetInput &in, int ns, cudaStream_t s)
+{
+    NetGrid &g = W.g;
+    g.total = ns * g.N;
+    const int bn = (g.total + NT - 1) / NT;
+    l1_fwd<<<bn, NT, 0, s>>>(g, in, W.w, W.a1);
+    conv16<true>(g, W.a1, W.W2f, W.w + OB2, 0, W.a2, nullptr, s);
+    conv16<true>(g, W.a2, W.W3f, W.w + OB3, 0, W.a3, nullptr, s);
+    const NetTile T = make_tile(g);
+    static std::once_flag attr;
+    std::call_once(attr, [] { cudaFuncSetAttribute(l4_fwd, cudaFuncAttributeMaxDynamicSharedMemorySize, TC_SMEM_MOST); });
+    l4_fwd<<<T.ntx * T.nty * T.ntz * ns, TL_T, tc_smem(T), s>>>(g, T, W.a3, W.w, W.y);
+}
+
+template <int CI, int CO>
+void wgrad(const NetGrid &g, const NetInput &in, const __nv_bfloat16 *a, const void *dz, float *part, cudaStream_t s)
+{
+    static std::once_flag attr;
+    std::call_once(attr, [] {
+        cudaFuncSetAttribute(wgrad_k<CI, CO>, cudaFuncAttributeMaxDynamicSharedMemorySize, wg_smem<CI, CO>());
+    });
+    const int blocks = (g.N + WG_NODES - 1) / WG_NODES * (g.total / g.N);
+    wgrad_k<CI, CO><<<blocks, WG_T, wg_smem<CI, CO>(), s>>>(g, in, a, dz, part);
+}
+
+// gradient of the loss over the ns samples of the last forward pass, into (or
+// added to) W.grad; *loss (device) (+)= loss_scale times their summed squared
+// error
+void net_backward(NetWork &W, const NetInput &in, int ns, const float *d_t, const uint8_t *d_mask, float inv_cnt,
+                  bool add, double loss_scale, double *d_loss, cudaStream_t s)
 {
     const NetGrid &g = W.g;
-    const int bn = (g.N + NT - 1) / NT;
-    const int bw = (g.N + 511) / 512;
-    loss_grad_k<<<bn, NT, 0, s>>>(g.N, W.y, d_t, d_mask, inv_cnt, W.gy, W.lpart);
-    // layer 4
-    wgrad_partial<16, 1><<<bw, NT, 0, s>>>(g, W.a3, 1, W.gy, 0, W.part);
-    reduce_partials<<<(16 * 27 + 1 + 255) / 256, 256, 0, s>>>(W.part, bw, 16 * 27 + 1, W.grad, OW4);
+    const int bn = (g.total + NT - 1) / NT;
+    const int per = (g.N + WG_NODES - 1) / WG_NODES;
+    loss_grad_k<<<bn, NT, 0, s>>>(g, W.y, d_t, in.smp, d_mask, inv_cnt, W.gy, W.lpart);
+    loss_sum_k<<<1, NT, 0, s>>>(W.lpart, bn, loss_scale, add ? 1 : 0, d_loss);
+    wgrad<16, 1>(g, in, W.a3, W.gy, W.part[3], s);
     l4_bwd_data<<<bn, NT, 0, s>>>(g, W.gy, W.w, W.a3, W.dz);
-    // layer 3: dz holds d z3 (through relu of a3)
-    wgrad_partial<16, 16><<<bw, NT, 0, s>>>(g, W.a2, 1, W.dz, 1, W.part);
-    reduce_partials<<<(16 * 16 * 27 + 16 + 255) / 256, 256, 0, s>>>(W.part, bw, 16 * 16 * 27 + 16, W.grad, OW3);
+    // dz holds d z3 (through relu of a3)
+    wgrad<16, 16>(g, in, W.a2, W.dz, W.part[2], s);
     conv16<false>(g, W.dz, W.W3b, nullptr, 1, W.dz2, W.a2, s);
-    // layer 2
-    wgrad_partial<16, 16><<<bw, NT, 0, s>>>(g, W.a1, 1, W.dz2, 1, W.part);
-    reduce_partials<<<(16 * 16 * 27 + 16 + 255) / 256, 256, 0, s>>>(W.part, bw, 16 * 16 * 27 + 16, W.grad, OW2);
+    wgrad<16, 16>(g, in, W.a1, W.dz2, W.part[1], s);
     conv16<false>(g, W.dz2, W.W2b, nullptr, 1, W.dz, W.a1, s);
-    // layer 1
-    wgrad_partial<2, 16><<<bw, NT, 0, s>>>(g, W.x, 0, W.dz, 1, W.part);
-    reduce_partials<<<(16 * 2 * 27 + 16 + 255) / 256, 256, 0, s>>>(W.part, bw, 16 * 2 * 27 + 16, W.grad, OW1);
-    if (loss) {
-        std::vector<double> lp(bn);
-        cudaError_t e = cudaMemcpyAsync(lp.data(), W.lpart, bn * sizeof(double), cudaMemcpyDeviceToHost, s);
-        if (e == cudaSuccess) e = cudaStreamSynchronize(s);
-        if (e != cudaSuccess) return EKL_ERR_CUDA;
-        double t = 0;
-        for (int b = 0; b < bn; b++) t += lp[b];
-        *loss = t * inv_cnt;
-    }
-    return cuda_err(cudaGetLastError());
+    wgrad<2, 16>(g, in, nullptr, W.dz, W.part[0], s);
+    grad_reduce<<<(NPARAM + 63) / 64, 64, 0, s>>>(W.part[0], W.part[1], W.part[2], W.part[3], per, ns, add ? 1 : 0,
+                                                  W.grad);
 }
 
 NetGrid make_grid(const int32_t dims[3], const int32_t periodic[3])
@@ -628,6 +966,7 @@ NetGrid make_grid(const int32_t dims[3], const int32_t periodic[3])
     g.nz = dims[2];
     for (int a = 0; a < 3; a++) g.per[a] = periodic ? (periodic[a] ? 1 : 0) : 0;
     g.N = g.nx * g.ny * g.nz;
+    g.total = g.N;
     return g;
 }
 
@@ -832,7 +1171,7 @@ int warmstart_before_poisson(Ctx &c)
         c.launches++;
     }
     if (ws.enabled && have) {
-        net_forward(ws.W, c.stream);
+        net_forward(ws.W, NetInput{ws.W.x, nullptr}, 1, c.stream);
         if (L) {
             if (c.prec == EKL_F64)
                 ws_apply_coarse<double><<<bn, 256, 0, c.stream>>>(ws.fine, ws.W.g, L, c.mask, ws.W.y, ws.s_out,
@@ -844,7 +1183,7 @@ int warmstart_before_poisson(Ctx &c)
             if (c.prec == EKL_F64) ws_apply<double><<<bn, 256, 0, c.stream>>>(N, c.mask, ws.W.y, ws.s_out, (double *)c.phi);
             else ws_apply<long long><<<bn, 256, 0, c.stream>>>(N, c.mask, ws.W.y, ws.s_out, (long long *)c.phi);
         }
-        c.launches += 7;
+        c.launches += 5;
     }
     std::swap(ws.bprev, ws.bcur);
     ws.have_prev = 1;
@@ -916,7 +1255,7 @@ static int warmstart_ensure(Ctx &c, int level = -1)
     const int32_t cdims[3] = {c.nx >> level, c.ny >> level, c.nz >> level};
     ws->W.g = make_grid(cdims, c.per);
     const int N = (int)c.N;
-    int rc = work_alloc(ws->W, ws->W.g.N);
+    int rc = work_alloc(ws->W, 1, false);
     cudaError_t e = rc == EKL_OK ? cudaSuccess : cudaErrorMemoryAllocation;
     if (e == cudaSuccess) e = cudaMalloc(&ws->bprev, (size_t)N * 4);
     if (e == cudaSuccess) e = cudaMalloc(&ws->bcur, (size_t)N * 4);
@@ -960,17 +1299,28 @@ int ekl_net_eval(const int32_t dims[3], const int32_t periodic[3], const float *
     if (!dims || !x || !w || !y || dims[0] < 1 || dims[1] < 1 || dims[2] < 1) return EKL_ERR_ARG;
     NetWork W;
     W.g = make_grid(dims, periodic);
-    int rc = work_alloc(W, W.g.N);
-    if (rc != EKL_OK) { work_free(W); return rc; }
+    int rc = work_alloc(W, 1, false);
+    if (rc != EKL_OK) return rc;
     cudaError_t e = cudaMemcpy(W.x, x, 2 * (size_t)W.g.N * 4, cudaMemcpyHostToDevice);
     if (e == cudaSuccess) e = cudaMemcpy(W.w, w, NPARAM * 4, cudaMemcpyHostToDevice);
     if (e == cudaSuccess) {
-        net_forward(W, 0);
+        net_prepare(W, 0);
+        net_forward(W, NetInput{W.x, nullptr}, 1, 0);
         e = cudaMemcpy(y, W.y, (size_t)W.g.N * 4, cudaMemcpyDeviceToHost);
     }
     work_free(W);
     if (e == cudaSuccess) return tc_check();
     return cuda_err(e);
+}
+
+static long long mask_count(const uint8_t *mask, int N)
+{
+    long long cnt = N;
+    if (mask) {
+        cnt = 0;
+        for (int i = 0; i < N; i++) cnt += mask[i] ? 1 : 0;
+    }
+    return cnt;
 }
 
 int ekl_net_loss_grad(const int32_t dims[3], const int32_t periodic[3], const float *x, const float *target,
@@ -980,34 +1330,36 @@ int ekl_net_loss_grad(const int32_t dims[3], const int32_t periodic[3], const fl
     NetWork W;
     W.g = make_grid(dims, periodic);
     const int N = W.g.N;
-    int rc = work_alloc(W, N);
-    if (rc != EKL_OK) { work_free(W); return rc; }
-    float *dt = nullptr;
-    uint8_t *dm = nullptr;
-    long long cnt = N;
-    if (mask) {
-        cnt = 0;
-        for (int i = 0; i < N; i++) cnt += mask[i] ? 1 : 0;
-    }
-    cudaError_t e = cudaMalloc(&dt, (size_t)N * 4);
-    if (e == cudaSuccess && mask) e = cudaMalloc(&dm, N);
-    if (e == cudaSuccess) e = cudaMemcpy(W.x, x, 2 * (size_t)N * 4, cudaMemcpyHostToDevice);
+    char *extra = nullptr;
+    const size_t tb = ((size_t)N * 4 + 255) & ~(size_t)255;
+    int rc = work_alloc(W, 1, true, tb + (size_t)N, &extra);
+    if (rc != EKL_OK) return rc;
+    float *dt = (float *)extra;
+    uint8_t *dm = mask ? (uint8_t *)(extra + tb) : nullptr;
+    const long long cnt = mask_count(mask, N);
+    const float inv_cnt = 1.f / (float)(cnt > 0 ? cnt : 1);
+    cudaError_t e = cudaMemcpy(W.x, x, 2 * (size_t)N * 4, cudaMemcpyHostToDevice);
     if (e == cudaSuccess) e = cudaMemcpy(W.w, w, NPARAM * 4, cudaMemcpyHostToDevice);
     if (e == cudaSuccess) e = cudaMemcpy(dt, target, (size_t)N * 4, cudaMemcpyHostToDevice);
     if (e == cudaSuccess && mask) e = cudaMemcpy(dm, mask, N, cudaMemcpyHostToDevice);
-    if (e == cudaSuccess) e = cudaMemset(W.grad, 0, NPARAM * 4);
     if (e == cudaSuccess) {
-        net_forward(W, 0);
-        rc = net_backward(W, dt, dm, 1.f / (float)(cnt > 0 ? cnt : 1), loss, 0);
-        if (rc == EKL_OK) e = cudaMemcpy(grad, W.grad, NPARAM * 4, cudaMemcpyDeviceToHost);
+        const NetInput in{W.x, nullptr};
+        net_prepare(W, 0);
+        net_forward(W, in, 1, 0);
+        net_backward(W, in, 1, dt, dm, inv_cnt, false, (double)inv_cnt, W.loss, 0);
+        e = cudaGetLastError();
+        if (e == cudaSuccess && loss) e = cudaMemcpy(loss, W.loss, sizeof(double), cudaMemcpyDeviceToHost);
+        if (e == cudaSuccess) e = cudaMemcpy(grad, W.grad, NPARAM * 4, cudaMemcpyDeviceToHost);
     }
-    cudaFree(dt);
-    cudaFree(dm);
     work_free(W);
-    if (rc != EKL_OK) return rc;
     if (e == cudaSuccess) return tc_check();
     return cuda_err(e);
 }
+
+// Nodes of one training pass: the samples of a batch go through the network
+// together as long as their buffers stay under about 4 GB (250 bytes a
+// node), else in several passes whose gradients add up.
+static constexpr long long NET_PASS_NODES = 16ll << 20;
 
 int ekl_net_train_grid(int32_t nsamples, const int32_t dims[3], const int32_t periodic[3], const float *x,
                        const float *target, const uint8_t *mask, float *w, int32_t iters, int32_t batch, float lr,
@@ -1017,26 +1369,25 @@ int ekl_net_train_grid(int32_t nsamples, const int32_t dims[3], const int32_t pe
     NetWork W;
     W.g = make_grid(dims, periodic);
     const int N = W.g.N;
-    int rc = work_alloc(W, N);
-    if (rc != EKL_OK) { work_free(W); return rc; }
-    float *dx = nullptr, *dt = nullptr, *m1 = nullptr, *m2 = nullptr;
-    uint8_t *dm = nullptr;
-    long long cnt = N;
-    if (mask) {
-        cnt = 0;
-        for (int i = 0; i < N; i++) cnt += mask[i] ? 1 : 0;
-    }
-    cudaError_t e = cudaMalloc(&dx, (size_t)nsamples * 2 * N * 4);
-    if (e == cudaSuccess) e = cudaMalloc(&dt, (size_t)nsamples * N * 4);
-    if (e == cudaSuccess) e = cudaMalloc(&m1, NPARAM * 4);
-    if (e == cudaSuccess) e = cudaMalloc(&m2, NPARAM * 4);
-    if (e == cudaSuccess && mask) e = cudaMalloc(&dm, N);
-    if (e == cudaSuccess) e = cudaMemcpy(dx, x, (size_t)nsamples * 2 * N * 4, cudaMemcpyHostToDevice);
-    if (e == cudaSuccess) e = cudaMemcpy(dt, target, (size_t)nsamples * N * 4, cudaMemcpyHostToDevice);
-    if (e == cudaSuccess && mask) e = cudaMemcpy(dm, mask, N, cudaMemcpyHostToDevice);
-    if (e == cudaSuccess) e = cudaMemcpy(W.w, w, NPARAM * 4, cudaMemcpyHostToDevice);
-    if (e == cudaSuccess) e = cudaMemset(m1, 0, NPARAM * 4);
-    if (e == cudaSuccess) e = cudaMemset(m2, 0, NPARAM * 4);
+    const long long fit = N > 0 ? NET_PASS_NODES / N : 1;
+    const int group = (int)(fit < 1 ? 1 : fit < batch ? fit : batch);
+    size_t off = 0;
+    auto carve = [&](size_t bytes) {
+        const size_t at = off;
+        off += (bytes + 255) & ~(size_t)255;
+        return at;
+    };
+    const size_t ox = carve((size_t)nsamples * 2 * N * 4), ot = carve((size_t)nsamples * N * 4), o1 = carve(NPARAM * 4),
+                 o2 = carve(NPARAM * 4), om = carve((size_t)N), os = carve((size_t)iters * batch * sizeof(int)),
+                 ol = carve((size_t)iters * sizeof(double));
+    char *ex = nullptr;
+    int rc = work_alloc(W, group, true, off, &ex);
+    if (rc != EKL_OK) return rc;
+    float *dx = (float *)(ex + ox), *dt = (float *)(ex + ot), *m1 = (float *)(ex + o1), *m2 = (float *)(ex + o2);
+    uint8_t *dm = mask ? (uint8_t *)(ex + om) : nullptr;
+    int *dsmp = (int *)(ex + os);
+    double *dloss = (double *)(ex + ol);
+    const long long cnt = mask_count(mask, N);
     // seeded sample order (splitmix64)
     uint64_t st = seed;
     auto next = [&]() {
@@ -1046,29 +1397,37 @@ int ekl_net_train_grid(int32_t nsamples, const int32_t dims[3], const int32_t pe
         z = (z ^ (z >> 27)) * 0x94D049BB133111EBull;
         return z ^ (z >> 31);
     };
+    std::vector<int> smp((size_t)iters * batch);
+    for (auto &v : smp) v = (int)(next() % (uint64_t)nsamples);
+    cudaError_t e = cudaMemcpy(dx, x, (size_t)nsamples * 2 * N * 4, cudaMemcpyHostToDevice);
+    if (e == cudaSuccess) e = cudaMemcpy(dt, target, (size_t)nsamples * N * 4, cudaMemcpyHostToDevice);
+    if (e == cudaSuccess && mask) e = cudaMemcpy(dm, mask, N, cudaMemcpyHostToDevice);
+    if (e == cudaSuccess) e = cudaMemcpy(W.w, w, NPARAM * 4, cudaMemcpyHostToDevice);
+    if (e == cudaSuccess && !smp.empty())
+        e = cudaMemcpy(dsmp, smp.data(), smp.size() * sizeof(int), cudaMemcpyHostToDevice);
+    if (e == cudaSuccess) e = cudaMemset(m1, 0, NPARAM * 4);
+    if (e == cudaSuccess) e = cudaMemset(m2, 0, NPARAM * 4);
     const float b1 = 0.9f, b2 = 0.999f, eps = 1e-8f;
-    for (int it = 0; it < iters && e == cudaSuccess && rc == EKL_OK; it++) {
-        cudaMemsetAsync(W.grad, 0, NPARAM * 4, 0);
-        double lsum = 0.0;
-        for (int bidx = 0; bidx < batch; bidx++) {
-            const int smp = (int)(next() % (uint64_t)nsamples);
-            e = cudaMemcpyAsync(W.x, dx + (size_t)smp * 2 * N, 2 * (size_t)N * 4, cudaMemcpyDeviceToDevice, 0);
-            if (e != cudaSuccess) break;
-            net_forward(W, 0);
-            double l = 0.0;
-            rc = net_backward(W, dt + (size_t)smp * N, dm, 1.f / (float)(cnt * batch), &l, 0);
-            lsum += l * batch;
-            if (rc != EKL_OK) break;
+    const float inv_cnt = 1.f / (float)(cnt * batch);
+    for (int it = 0; it < iters && e == cudaSuccess; it++) {
+        net_prepare(W, 0);
+        for (int k = 0; k < batch; k += group) {
+            const int ns = batch - k < group ? batch - k : group;
+            const NetInput in{dx, dsmp + (size_t)it * batch + k};
+            net_forward(W, in, ns, 0);
+            net_backward(W, in, ns, dt, dm, inv_cnt, k > 0, (double)inv_cnt, dloss + it, 0);
         }
         const float c1 = 1.f - powf(b1, (float)(it + 1)), c2 = 1.f - powf(b2, (float)(it + 1));
         adam_k<<<(NPARAM + 255) / 256, 256>>>(NPARAM, W.w, W.grad, m1, m2, lr, b1, b2, eps, c1, c2);
-        if (loss_out) loss_out[it] = (float)(lsum / batch);
         e = cudaGetLastError();
     }
-    if (e == cudaSuccess && rc == EKL_OK) e = cudaMemcpy(w, W.w, NPARAM * 4, cudaMemcpyDeviceToHost);
-    cudaFree(dx); cudaFree(dt); cudaFree(m1); cudaFree(m2); cudaFree(dm);
+    if (e == cudaSuccess) e = cudaMemcpy(w, W.w, NPARAM * 4, cudaMemcpyDeviceToHost);
+    if (e == cudaSuccess && loss_out && iters > 0) {
+        std::vector<double> l(iters);
+        e = cudaMemcpy(l.data(), dloss, (size_t)iters * sizeof(double), cudaMemcpyDeviceToHost);
+        for (int it = 0; it < iters; it++) loss_out[it] = (float)l[it];
+    }
     work_free(W);
-    if (rc != EKL_OK) return rc;
     if (e == cudaSuccess) return tc_check();
     return cuda_err(e);
 }
@@ -1118,7 +1477,12 @@ int ekl_set_warmstart(ekl_handle *h, const float *w, const float scales[3])
     int rc = ekl::warmstart_ensure(c);
     if (rc != EKL_OK) return rc;
     WarmStart &ws = *(WarmStart *)c.net;
-    if (cudaMemcpy(ws.W.w, w, NPARAM * 4, cudaMemcpyHostToDevice) != cudaSuccess) return EKL_ERR_CUDA;
+    // ordered on the handle's stream: earlier steps still read the old parameters
+    if (cudaStreamSynchronize(c.stream) != cudaSuccess ||
+        cudaMemcpy(ws.W.w, w, NPARAM * 4, cudaMemcpyHostToDevice) != cudaSuccess)
+        return EKL_ERR_CUDA;
+    net_prepare(ws.W, c.stream);
+    if (cudaGetLastError() != cudaSuccess) return EKL_ERR_CUDA;
     if (scales) {
         ws.s_db = scales[0];
         ws.s_phi = scales[1];
