@@ -18,7 +18,7 @@ constexpr int MG_THREADS = 512;     // multigrid launch: one block per SM (laten
 constexpr int MG_WIDE_THREADS = 1024;  // the same for lattices of at least MG_WIDE_NODES_PER_SM nodes per SM
 constexpr int MG_WIDE_NODES_PER_SM = 16384;
 constexpr int MG_BATCH_THREADS = 1024;  // batched multigrid: each block sweeps large replica volumes
-constexpr int BEAD_THREADS = 256;
+constexpr int BEAD_THREADS = 1024;
 // fixed-point scale of the potential in the reduced-precision paths: 2^40
 constexpr double PHI_SCALE = 1099511627776.0;
 constexpr double PHI_INV = 1.0 / 1099511627776.0;

@@ -76,6 +76,16 @@ template <typename S, typename R, typename PhiT> struct StepArgs {
     long long step;
 };
 
+// x / b rounded to nearest from y = 1 / b rounded to nearest: Markstein's
+// correction of the product x y (IBM J. Res. Dev. 34, 1990), exact for
+// quotients in the normal range; three operations where a division takes
+// about ten
+template <typename R> __device__ __forceinline__ R quot(R x, R b, R y)
+{
+    const R q = x * y;
+    return fma(fma(-q, b, x), y, q);
+}
+
 // pull of the 19 populations of species s at node i (bounce-back on set bits)
 template <typename S, typename R>
 __device__ __forceinline__ void pull19(const S *__restrict__ f, long long N, int s, long long i,
@@ -979,188 +989,195 @@ template <typename R> struct BeadArgs {
     int *status;
 };
 
-// Trilinear weights of the 8 nodes around a bead, wall nodes weighted zero
-// and the rest renormalised (the interpolation kernel of Sec. II.C).
-// Slot order k = ox + 2 oy + 4 oz.  Returns false when all 8 are wall.
+// Corner k (x fastest) of the trilinear stencil of a bead at Rb: its node (-1
+// beyond a closed face), whether it is fluid, and its weight before
+// renormalisation (0 on walls).  False when the position is absurd.
 template <typename R>
-__device__ bool bead_stencil(const Grid3 &g, const int per[3], const uint32_t *mask, const double Rb[3],
-                             long long nodes[8], R w[8])
+__device__ __forceinline__ bool bead_corner(const Grid3 &g, const int per[3], const uint32_t *mask, const double Rb[3],
+                                            int k, long long &node, bool &fluid, R &w)
 {
-    int base[3];
-    R fr[3];
-    int dims[3] = {g.nx, g.ny, g.nz};
+    const int dims[3] = {g.nx, g.ny, g.nz};
+    node = -1;
+    fluid = false;
+    w = R(0);
     for (int c = 0; c < 3; c++)
         if (!(fabs(Rb[c]) < 1e6)) return false;  // non-finite or absurd position
+    int q[3];
+    bool in = true;
+    R wk = R(1);
     for (int c = 0; c < 3; c++) {
-        double fl = floor(Rb[c]);
-        base[c] = (int)fl;
-        fr[c] = (R)(Rb[c] - fl);
-    }
-    // node ids first (a position in [0, L) on a periodic axis puts every
-    // corner within one period, so a single add or subtract wraps it), then
-    // all eight link words are loaded together
-    uint32_t mk[8];
-#pragma unroll
-    for (int k = 0; k < 8; k++) {
-        const int o[3] = {k & 1, (k >> 1) & 1, (k >> 2) & 1};
-        int q[3];
-        bool in = true;
-        for (int c = 0; c < 3; c++) {
-            int v = base[c] + o[c];
-            if (per[c]) {
-                if (v >= dims[c]) v -= dims[c];
-                else if (v < 0) v += dims[c];
-                if (v < 0 || v >= dims[c]) {  // far outside the box: the general wrap
-                    v %= dims[c];
-                    if (v < 0) v += dims[c];
-                }
-            } else if (v < 0 || v >= dims[c]) {
-                in = false;
+        const double fl = floor(Rb[c]);
+        const R fr = (R)(Rb[c] - fl);
+        const int o = (k >> c) & 1;
+        wk *= o ? fr : R(1) - fr;
+        // a position in [0, L) on a periodic axis puts every corner within
+        // one period, so a single add or subtract wraps it
+        int v = (int)fl + o;
+        if (per[c]) {
+            if (v >= dims[c]) v -= dims[c];
+            else if (v < 0) v += dims[c];
+            if (v < 0 || v >= dims[c]) {  // far outside the box: the general wrap
+                v %= dims[c];
+                if (v < 0) v += dims[c];
             }
-            q[c] = v;
+        } else if (v < 0 || v >= dims[c]) {
+            in = false;
         }
-        nodes[k] = in ? (long long)q[0] + (long long)g.nx * (q[1] + (long long)g.ny * q[2]) : -1;
+        q[c] = v;
     }
-#pragma unroll
-    for (int k = 0; k < 8; k++) mk[k] = nodes[k] >= 0 ? mask[nodes[k]] : SOLID_BIT;
-    R W = R(0);
-#pragma unroll
-    for (int k = 0; k < 8; k++) {
-        const int o[3] = {k & 1, (k >> 1) & 1, (k >> 2) & 1};
-        R wk = R(1);
-        for (int c = 0; c < 3; c++) wk *= o[c] ? fr[c] : R(1) - fr[c];
-        w[k] = (mk[k] & SOLID_BIT) ? R(0) : wk;
-        W += w[k];
-    }
-    if (!(W > R(0))) return false;
-    for (int k = 0; k < 8; k++) w[k] = w[k] / W;
+    if (!in) return true;
+    node = (long long)q[0] + (long long)g.nx * (q[1] + (long long)g.ny * q[2]);
+    fluid = !(mask[node] & SOLID_BIT);
+    if (fluid) w = wk;
     return true;
 }
 
-// One block: stencils of all beads, entries sorted by (node, bead) with a
-// bitonic sort in shared memory, unique nodes -> patch slots (ascending node
-// id), the sorted entry list with each slot's first position, and the bead
-// charge per slot summed in bead order.
+// One block: stencils of all beads (eight lanes per bead, a corner each),
+// entries sorted by (node, bead) in shared memory, unique nodes -> patch slots
+// (ascending node id), the sorted entry list with each slot's first position,
+// and the bead charge per slot summed in bead order.  Up to RANK_ENTRIES
+// entries are sorted by counting the smaller keys of each (no barrier between
+// its steps), more by a bitonic network.  What bounds it: latency, one block;
+// 32 beads 18 -> 13 us, 100 beads 38 -> 22 us (one thread per bead, 256
+// threads and 36 to 55 barriers of the network before).
+constexpr int RANK_ENTRIES = 512;
 template <typename R> __device__ void bead_bin_body(const BeadArgs<R> &a)
 {
     __shared__ unsigned long long key[MAX_ENTRIES];
-    __shared__ int flag[MAX_ENTRIES];
-    const int ne = a.nb * 8;
-    int npow = 1;
+    __shared__ R wt[MAX_ENTRIES];
+    __shared__ int wtot[BEAD_THREADS / 32];
+    __shared__ int s_nvalid, s_slots;
+    const int ne = a.nb * 8, tid = threadIdx.x;
+    int npow = 32;
     while (npow < ne) npow <<= 1;
     // clear the previous step's patch bits (the list is rewritten below,
     // after several block barriers)
     {
         const int old = *a.patch_count;
-        for (int k = threadIdx.x; k < old; k += blockDim.x) {
+        for (int k = tid; k < old; k += blockDim.x) {
             const int nd = a.patch_node[k];
             atomicAnd(a.patch_bits + (nd >> 5), ~(1u << (nd & 31)));
         }
     }
-    for (int b = threadIdx.x; b < a.nb; b += blockDim.x) {
-        double Rb[3] = {a.Rb[3 * b], a.Rb[3 * b + 1], a.Rb[3 * b + 2]};
-        long long nd[8];
-        R w[8];
-        bool ok = bead_stencil<R>(a.g, a.per, a.mask, Rb, nd, w);
-        if (!ok) atomicOr(a.status, ST_BEAD);
-        for (int k = 0; k < 8; k++) {
-            int e = b * 8 + k;
-            a.entry_w[e] = ok ? w[k] : R(0);
-            bool use = ok && nd[k] >= 0 && !(a.mask[nd[k]] & SOLID_BIT);
-            key[e] = use ? (((unsigned long long)nd[k] << 20) | (unsigned)e) : ~0ull;
+    if (tid == 0) s_nvalid = 0;
+    for (int e = tid; e < npow; e += blockDim.x) {  // whole warps
+        const int b = e >> 3, k = e & 7;
+        long long node = -1;
+        bool fluid = false, ok = false;
+        R w = R(0);
+        if (e < ne) {
+            const double Rb[3] = {a.Rb[3 * b], a.Rb[3 * b + 1], a.Rb[3 * b + 2]};
+            ok = bead_corner<R>(a.g, a.per, a.mask, Rb, k, node, fluid, w);
+        }
+        // the eight weights added in corner order
+        R W = R(0);
+#pragma unroll
+        for (int c = 0; c < 8; c++) W += __shfl_sync(0xffffffffu, w, (tid & 24) + c);
+        ok = ok && W > R(0);
+        w = ok ? w / W : R(0);
+        key[e] = ok && fluid ? (((unsigned long long)node << 20) | (unsigned)e) : ~0ull;
+        wt[e] = w;
+        if (e < ne) {
+            a.entry_w[e] = w;
+            a.entry_slot[e] = -1;
+            if (!ok && k == 0) atomicOr(a.status, ST_BEAD);
         }
     }
-    for (int e = ne + threadIdx.x; e < npow; e += blockDim.x) key[e] = ~0ull;
     __syncthreads();
-    for (int k = 2; k <= npow; k <<= 1) {
-        for (int j = k >> 1; j > 0; j >>= 1) {
-            for (int t = threadIdx.x; t < npow; t += blockDim.x) {
-                int ixj = t ^ j;
-                if (ixj > t) {
-                    unsigned long long u = key[t], v = key[ixj];
-                    bool up = (t & k) == 0;
-                    if ((u > v) == up) {
-                        key[t] = v;
-                        key[ixj] = u;
+    if (npow <= RANK_ENTRIES) {
+        // `split` neighbouring threads count for one entry
+        const int split = min(32, (int)blockDim.x / npow), e = tid / split, part = tid - e * split;
+        unsigned long long mine = ~0ull;
+        int rank = 0;
+        if (e < npow) {
+            mine = key[e];
+            for (int t = part; t < ne; t += split) rank += key[t] < mine;
+        }
+        for (int o = 1; o < split; o <<= 1) rank += __shfl_xor_sync(0xffffffffu, rank, o);
+        const bool valid = e < npow && part == 0 && mine != ~0ull;
+        if (valid) atomicAdd(&s_nvalid, 1);
+        __syncthreads();
+        const int nv = s_nvalid;
+        if (valid) key[rank] = mine;
+        if (e < npow && part == 0 && e >= nv) {
+            // positions past the valid keys (their old keys have been read)
+            key[e] = ~0ull;
+        }
+        __syncthreads();
+    } else {
+        for (int k = 2; k <= npow; k <<= 1) {
+            for (int j = k >> 1; j > 0; j >>= 1) {
+                for (int t = tid; t < npow; t += blockDim.x) {
+                    int ixj = t ^ j;
+                    if (ixj > t) {
+                        unsigned long long u = key[t], v = key[ixj];
+                        bool up = (t & k) == 0;
+                        if ((u > v) == up) {
+                            key[t] = v;
+                            key[ixj] = u;
+                        }
                     }
                 }
+                __syncthreads();
             }
-            __syncthreads();
         }
     }
     // slots: an entry starts a slot when its node differs from the previous
-    // entry's; slot index = inclusive prefix count of starts - 1 (block scan:
-    // each thread takes a contiguous chunk, warps scan their chunk totals by
-    // shuffles, warp totals are scanned once); unused keys (~0) sort last
-    {
-        __shared__ int wtot[BEAD_THREADS / 32];
-        __shared__ int s_nvalid;
-        const int per = (npow + blockDim.x - 1) / blockDim.x;
-        const int t0 = threadIdx.x * per, t1 = min(t0 + per, npow);
-        int local = 0;
-        for (int t = t0; t < t1; t++) {
-            const unsigned long long u = key[t];
-            local += (u != ~0ull) && (t == 0 || (key[t - 1] >> 20) != (u >> 20));
-        }
-        const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
-        int incl = local;
+    // entry's; slot index = inclusive prefix count of starts - 1 (each thread
+    // takes a contiguous chunk, warps scan their chunk totals by shuffles, a
+    // thread adds the totals of the warps before its own); unused keys (~0)
+    // sort last
+    const int per = (npow + blockDim.x - 1) / blockDim.x;
+    const int t0 = tid * per, t1 = min(t0 + per, npow);
+    auto starts = [&](int t) {
+        const unsigned long long u = key[t];
+        return u != ~0ull && (t == 0 || (key[t - 1] >> 20) != (u >> 20));
+    };
+    int local = 0, used = 0;
+    for (int t = t0; t < t1; t++) {
+        local += starts(t);
+        used += key[t] != ~0ull;
+    }
+    const int lane = tid & 31, wid = tid >> 5;
+    int incl = local;
 #pragma unroll
-        for (int o = 1; o < 32; o <<= 1) {
-            const int v = __shfl_up_sync(0xffffffffu, incl, o);
-            if (lane >= o) incl += v;
-        }
-        if (lane == 31) wtot[wid] = incl;
-        if (threadIdx.x == 0) s_nvalid = npow;
-        __syncthreads();
-        int before = 0;
-        for (int w = 0; w < wid; w++) before += wtot[w];
-        int run = before + incl - local;  // starts before this thread's chunk
-        for (int t = t0; t < t1; t++) {
-            const unsigned long long u = key[t];
-            if (u == ~0ull) {
-                flag[t] = -1;
-                if (t == 0 || key[t - 1] != ~0ull) s_nvalid = t;  // first unused key
-                continue;
-            }
-            if (t == 0 || (key[t - 1] >> 20) != (u >> 20)) {
-                a.slot_first[run] = t;
-                run++;
-            }
-            flag[t] = run - 1;
-        }
-        __syncthreads();
-        if (threadIdx.x == blockDim.x - 1) {
-            int c = 0;
-            for (int w = 0; w < (int)(blockDim.x >> 5); w++) c += wtot[w];
-            a.slot_first[c] = s_nvalid;
-            *a.patch_count = c;
-        }
+    for (int o = 1; o < 32; o <<= 1) {
+        const int v = __shfl_up_sync(0xffffffffu, incl, o);
+        if (lane >= o) incl += v;
     }
+    if (lane == 31) wtot[wid] = incl;
+    if (npow > RANK_ENTRIES && used) atomicAdd(&s_nvalid, used);
     __syncthreads();
-    for (int t = threadIdx.x; t < ne; t += blockDim.x) a.entry_slot[t] = -1;
-    __syncthreads();
-    for (int t = threadIdx.x; t < npow; t += blockDim.x) {
-        unsigned long long u = key[t];
+    int before = 0;
+    for (int w = 0; w < wid; w++) before += wtot[w];
+    int run = before + incl - local;  // starts before this thread's chunk
+    for (int t = t0; t < t1; t++) {
+        const unsigned long long u = key[t];
         if (u == ~0ull) continue;
-        int e = (int)(u & 0xFFFFFu);
-        a.entry_slot[e] = flag[t];
-        a.sorted_entry[t] = e;
-        if (t == 0 || (key[t - 1] >> 20) != (u >> 20)) {
+        const int e = (int)(u & 0xFFFFFu);
+        if (starts(t)) {
             const int nd = (int)(u >> 20);
-            a.patch_node[flag[t]] = nd;
+            a.slot_first[run] = t;
+            a.patch_node[run] = nd;
             atomicOr(a.patch_bits + (nd >> 5), 1u << (nd & 31));
+            // the slot's charge: its entries in order
+            R acc = R(0);
+            for (int v = t; v < npow && key[v] != ~0ull && (key[v] >> 20) == (u >> 20); v++) {
+                const int f = (int)(key[v] & 0xFFFFFu);
+                const R w = wt[f];
+                if (w != R(0)) acc += a.qb[f >> 3] * w;
+            }
+            a.patch_q[run] = acc;
+            run++;
         }
+        a.entry_slot[e] = run - 1;
+        a.sorted_entry[t] = e;
     }
+    if (tid == (int)blockDim.x - 1) s_slots = before + incl;
     __syncthreads();
-    const int pc = *a.patch_count;
-    for (int k = threadIdx.x; k < pc; k += blockDim.x) {
-        R acc = R(0);
-        for (int t = a.slot_first[k]; t < a.slot_first[k + 1]; t++) {
-            int e = a.sorted_entry[t];
-            R w = a.entry_w[e];
-            if (w != R(0)) acc += a.qb[e >> 3] * w;
-        }
-        a.patch_q[k] = acc;
+    if (tid == 0) {
+        a.slot_first[s_slots] = s_nvalid;
+        *a.patch_count = s_slots;
     }
 }
 
@@ -1304,132 +1321,134 @@ __device__ __forceinline__ bool bond_add(const MdArgs<S, R, PhiT, DEV> &A, const
     return ok;
 }
 
-// Conservative force on bead b, summed serially in the oracle's order: bond
-// with b-1, bond with b+1 (Eq. 9c, FENE option), WCA with every other bead in
-// index order except bonded neighbours when the bond is harmonic (Eq. 9a),
-// WCA against wall nodes in z, y, x order.
-template <typename S, typename R, typename PhiT, bool DEV>
-__device__ bool bead_force_serial(const MdArgs<S, R, PhiT, DEV> &A, const double *Rs, int b, R F[3],
-                                  const int *org, const uint32_t *bits)
+// Conservative force on bead b with the 32 lanes of a warp sharing the partner
+// and wall loops: bond with b - 1 in lane 0, bond with b + 1 in lane 1 (Eq. 9c,
+// FENE option), WCA with every other bead except bonded neighbours when the
+// bond is harmonic (Eq. 9a), WCA against wall nodes.  Valid in every lane.
+// FP32: each lane adds its own terms, then a fixed xor tree.  FP64: the terms
+// that are not zero (a handful) are added one by one in the oracle's order,
+// bonds, partners by index, wall nodes by z, y, x.  Rq, Rf: positions of all
+// beads (P: double, or fixed point in the reduced-precision paths) and their
+// FP32 copies; wlo, wn, org, bits: this bead's wall scan box and cached
+// block; rloc: its position relative to the block's origin.
+template <typename S, typename R, typename PhiT, bool DEV, typename P>
+__device__ bool bead_force_warp(const MdArgs<S, R, PhiT, DEV> &A, const P *Rq, const float *Rf, const R *rloc,
+                                const int *wlo, const int *wn, const int *chain, int b, R F[3], const int *org,
+                                const uint32_t *bits)
 {
-    const Grid3 &g = A.b.g;
-    const int nb = A.b.nb;
-    F[0] = F[1] = F[2] = R(0);
-    bool ok = bond_add(A, Rs, A.b.chain, b, 0, F);
-    ok = bond_add(A, Rs, A.b.chain, b, 1, F) && ok;
-    for (int c2 = 0; c2 < nb; c2++) {
-        if (c2 == b) continue;
-        int lo = c2 < b ? c2 : b, hi = c2 < b ? b : c2;
-        if (A.bond_kind == EKL_BOND_HARMONIC && A.b.chain[lo] == A.b.chain[hi] && hi - lo <= 1)
-            continue;
-        R d[3];
-        separation(g, A.b.per, &Rs[3 * lo], &Rs[3 * hi], d);
-        R Fp[3] = {R(0), R(0), R(0)};
-        wca_add<R>(A.wca_eps, A.wca_sigma, d, Fp);
-        for (int c = 0; c < 3; c++) {
-            if (c2 < b) F[c] -= Fp[c];
-            else F[c] += Fp[c];
-        }
-    }
-    const double rc = 1.122462048309373 * (double)A.wall_sigma;  // 2^(1/6) sigma
-    for (int c = 0; c < 3; c++)
-        if (!(fabs(Rs[3 * b + c]) < 1e6) || !(rc < 16.0)) return false;  // keeps the scan bounded
-    int lo[3], hi[3];
-    for (int c = 0; c < 3; c++) {
-        lo[c] = (int)floor(Rs[3 * b + c] - rc);
-        hi[c] = (int)floor(Rs[3 * b + c] + rc) + 1;
-    }
-    for (int z = lo[2]; z <= hi[2]; z++)
-        for (int y = lo[1]; y <= hi[1]; y++)
-            for (int x = lo[0]; x <= hi[0]; x++) {
-                bool in;
-                if (!wall_solid(g, A.b.per, A.b.mask, x, y, z, org, bits, in)) continue;
-                R d[3] = {(R)(Rs[3 * b] - x), (R)(Rs[3 * b + 1] - y), (R)(Rs[3 * b + 2] - z)};
-                wca_add<R>(A.wall_eps, A.wall_sigma, d, F);
-            }
-    return ok;
-}
-
-// Same forces with the 32 lanes of a warp sharing the partner and wall loops
-// (reduced-precision paths); the result is reduced with a fixed xor tree and
-// is valid in every lane.
-template <typename S, typename R, typename PhiT, bool DEV>
-__device__ bool bead_force_warp(const MdArgs<S, R, PhiT, DEV> &A, const long long *Rq, const float *Rf,
-                                const float *Rloc, const int *wlo, const int *wn, const int *chain, int b, R F[3],
-                                const int *org, const uint32_t *bits)
-{
+    constexpr bool ORDERED = sizeof(R) == 8;
     const Grid3 &g = A.b.g;
     const int nb = A.b.nb;
     const int lane = threadIdx.x & 31;
-    R f[3] = {R(0), R(0), R(0)};
+    R f[3] = {R(0), R(0), R(0)};  // ORDERED: the running sum, the same in every lane
+    // one term of each lane (zero in lanes without one)
+    auto add = [&](const R t[3]) {
+        if constexpr (ORDERED) {
+            unsigned m = __ballot_sync(0xffffffffu, t[0] != R(0) || t[1] != R(0) || t[2] != R(0));
+            while (m) {
+                const int src = __ffs(m) - 1;
+                m &= m - 1;
+                for (int c = 0; c < 3; c++) f[c] += __shfl_sync(0xffffffffu, t[c], src);
+            }
+        } else {
+            for (int c = 0; c < 3; c++) f[c] += t[c];
+        }
+    };
     bool ok = true;
-    // the bond with b - 1 in lane 0, with b + 1 in lane 1 (one pass)
-    if (lane < 2) ok = bond_add(A, Rq, chain, b, lane, f);
+    {
+        R t[3] = {R(0), R(0), R(0)};
+        if (lane < 2) ok = bond_add(A, Rq, chain, b, lane, t);
+        add(t);
+    }
     const float Lf[3] = {(float)g.nx, (float)g.ny, (float)g.nz};
     const float cut2 = 1.2599210498948732f * (float)A.wca_sigma * (float)A.wca_sigma;
-    for (int c2 = lane; c2 < nb; c2 += 32) {
-        if (c2 == b) continue;
-        int lo = c2 < b ? c2 : b, hi = c2 < b ? b : c2;
-        if (A.bond_kind == EKL_BOND_HARMONIC && chain[lo] == chain[hi] && hi - lo <= 1) continue;
-        // float screen, FP64 separation only for pairs near the cut-off
-        float q2 = 0.f;
-        for (int c = 0; c < 3; c++) {
-            float v = Rf[3 * b + c] - Rf[3 * c2 + c];
-            if (A.b.per[c]) {
-                if (v > 0.5f * Lf[c]) v -= Lf[c];
-                else if (v < -0.5f * Lf[c]) v += Lf[c];
+    for (int c0 = 0; c0 < nb; c0 += 32) {
+        const int c2 = c0 + lane;
+        R t[3] = {R(0), R(0), R(0)};
+        const int lo = c2 < b ? c2 : b, hi = c2 < b ? b : c2;
+        if (c2 < nb && c2 != b &&
+            !(A.bond_kind == EKL_BOND_HARMONIC && chain[lo] == chain[hi] && hi - lo <= 1)) {
+            // float screen, exact separation only for pairs near the cut-off
+            float q2 = 0.f;
+            for (int c = 0; c < 3; c++) {
+                float v = Rf[3 * b + c] - Rf[3 * c2 + c];
+                if (A.b.per[c]) {
+                    if (v > 0.5f * Lf[c]) v -= Lf[c];
+                    else if (v < -0.5f * Lf[c]) v += Lf[c];
+                }
+                q2 += v * v;
             }
-            q2 += v * v;
+            if (!(q2 > 1.1f * cut2 + 0.01f)) {
+                R d[3];
+                separation(g, A.b.per, &Rq[3 * lo], &Rq[3 * hi], d);
+                wca_add<R>(A.wca_eps, A.wca_sigma, d, t);
+                if (c2 < b)
+                    for (int c = 0; c < 3; c++) t[c] = -t[c];
+            }
         }
-        if (q2 > 1.1f * cut2 + 0.01f) continue;
-        R d[3];
-        separation(g, A.b.per, &Rq[3 * lo], &Rq[3 * hi], d);
-        R Fp[3] = {R(0), R(0), R(0)};
-        wca_add<R>(A.wca_eps, A.wca_sigma, d, Fp);
-        for (int c = 0; c < 3; c++) {
-            if (c2 < b) f[c] -= Fp[c];
-            else f[c] += Fp[c];
-        }
+        add(t);
     }
-    // wall nodes in the scan box; coordinates relative to the cached box origin
-    const int n0 = wn[3 * b], n1 = wn[3 * b + 1], n2 = wn[3 * b + 2];
-    const int cells = n0 * n1 * n2;
-    const float i0 = 1.f / (float)n0, i1 = 1.f / (float)n1;
-    for (int t = lane; t < cells; t += 32) {
-        const int r = tdiv(t, i0), zz = tdiv(r, i1);
-        const int x = wlo[3 * b] + t - r * n0, y = wlo[3 * b + 1] + r - zz * n1, z = wlo[3 * b + 2] + zz;
-        bool in;
-        if (!wall_solid(g, A.b.per, A.b.mask, x, y, z, org, bits, in)) continue;
-        R d[3] = {(R)(Rloc[3 * b] - (float)(x - org[0])), (R)(Rloc[3 * b + 1] - (float)(y - org[1])),
-                  (R)(Rloc[3 * b + 2] - (float)(z - org[2]))};
-        wca_add<R>(A.wall_eps, A.wall_sigma, d, f);
-    }
+    // wall nodes in the scan box; coordinates relative to the cached box
+    // origin.  Away from walls (no flag set in a block that covers the box)
+    // there is nothing to scan.
+    const int n0 = wn[0], n1 = wn[1], n2 = wn[2];
+    uint32_t any = 0;
 #pragma unroll
-    for (int o = 16; o > 0; o >>= 1)
-        for (int c = 0; c < 3; c++) f[c] += __shfl_xor_sync(0xffffffffu, f[c], o);
+    for (int w = 0; w < WALL_WORDS; w++) any |= bits[w];
+    bool covered = true;
+    for (int c = 0; c < 3; c++) covered = covered && wlo[c] >= org[c] && wlo[c] + wn[c] <= org[c] + WALL_BOX;
+    const int cells = (covered && any == 0) ? 0 : n0 * n1 * n2;
+    const float i0 = 1.f / (float)n0, i1 = 1.f / (float)n1;
+    for (int t0 = 0; t0 < cells; t0 += 32) {
+        const int k = t0 + lane;
+        R t[3] = {R(0), R(0), R(0)};
+        if (k < cells) {
+            const int r = tdiv(k, i0), zz = tdiv(r, i1);
+            const int x = wlo[0] + k - r * n0, y = wlo[1] + r - zz * n1, z = wlo[2] + zz;
+            bool in;
+            if (wall_solid(g, A.b.per, A.b.mask, x, y, z, org, bits, in)) {
+                R d[3];
+                if constexpr (ORDERED) {
+                    d[0] = (R)Rq[3 * b] - (R)x;
+                    d[1] = (R)Rq[3 * b + 1] - (R)y;
+                    d[2] = (R)Rq[3 * b + 2] - (R)z;
+                } else {
+                    d[0] = rloc[0] - (R)(x - org[0]);
+                    d[1] = rloc[1] - (R)(y - org[1]);
+                    d[2] = rloc[2] - (R)(z - org[2]);
+                }
+                wca_add<R>(A.wall_eps, A.wall_sigma, d, t);
+            }
+        }
+        add(t);
+    }
+    if constexpr (!ORDERED) {
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1)
+            for (int c = 0; c < 3; c++) f[c] += __shfl_xor_sync(0xffffffffu, f[c], o);
+    }
     for (int c = 0; c < 3; c++) F[c] = f[c];
     return __all_sync(0xffffffffu, ok);
 }
 
-// Per-bead wall scan box [floor(R - rc), floor(R + rc) + 1] and coordinates
-// local to the cached block (one thread per coordinate, FP64 once per sub-step)
-__device__ __forceinline__ void scan_bounds(double r, double rc, int org, int &lo, int &n, float &loc,
-                                            int &bad)
+// One coordinate of a bead's wall scan box [floor(R - rc), floor(R + rc) + 1]
+// (lo, n) and its coordinate relative to the cached block's origin, from an
+// FP64 position, or from a fixed-point one and cut-off (40 fractional bits)
+__device__ __forceinline__ void scan_bounds(double r, double rc, int org, int &lo, int &n, double &loc, int &bad)
 {
     if (!(fabs(r) < 1e6) || !(rc < 16.0)) {
         bad = 1;
         lo = 0;
         n = 0;
-        loc = 0.f;
+        loc = 0.0;
         return;
     }
     lo = (int)floor(r - rc);
     n = (int)floor(r + rc) + 2 - lo;
-    loc = (float)(r - (double)org);
+    loc = r - (double)org;
 }
-// the same from a fixed-point position rq and cut-off rcq (40 fractional bits)
-__device__ __forceinline__ void scan_bounds_q(long long rq, long long rcq, int org, int &lo, int &n, float &loc,
-                                              int &bad)
+__device__ __forceinline__ void scan_bounds(long long rq, long long rcq, int org, int &lo, int &n, float &loc,
+                                            int &bad)
 {
     if (!(rq < (1ll << 60) && rq > -(1ll << 60)) || !(rcq < (16ll << 40))) {
         bad = 1;
@@ -1443,53 +1462,111 @@ __device__ __forceinline__ void scan_bounds_q(long long rq, long long rcq, int o
     loc = ll_to_float(rq - ((long long)org << 40)) * (float)PHI_INV;
 }
 
-// One block: moments and field at the patch nodes, interpolation to beads,
-// md_substeps Langevin sub-steps with implicit friction, spreading of the
-// sub-step-averaged drag g^a_i = -gamma^a (u^a(R_i) - V_i) as a force per
-// particle on the patch nodes.  Readings as in the oracle: gamma^a = xi n^a/n
-// (or xi), fluid/field held at R(t) over the sub-steps, R(t) weights both ways.
-// FP64 instantiation: one thread per bead, serial sums in the oracle's order.
-// Reduced-precision instantiations: one warp per bead.
+// One cluster of MD_BLOCKS blocks: moments and field at the patch nodes,
+// interpolation to the beads, md_substeps Langevin sub-steps with implicit
+// friction, spreading of the sub-step-averaged drag g^a_i = -gamma^a (u^a(R_i)
+// - V_i) as a force per particle on the patch nodes.  Readings as in the
+// oracle: gamma^a = xi n^a/n (or xi), fluid/field held at R(t) over the
+// sub-steps, R(t) weights both ways.
+//
+// Block k takes the beads from k per to (k + 1) per, one warp per bead, and
+// every block holds all positions in shared memory, twice: a sub-step reads
+// one copy and writes its beads' new positions into the other copy of every
+// block (distributed shared memory), with one cluster barrier per sub-step.
+// The patch nodes (moments before, drag after) are shared out in the same
+// way.  What bounds it: the chain of sub-steps, each a force evaluation of
+// about a thousand dependent instructions; on one SM the 32 to 128 warps of a
+// chain shared its four schedulers, over eight SMs a warp mostly has its own.
+// 64x64x128 pore, 32 beads: 61 -> 46 us; 100 beads: 195 -> 59 us; FP64, one
+// thread per bead before: 847 -> 140 us, with the same sums bit for bit.
+constexpr int MD_BLOCKS = 8;
+constexpr int MD_THREADS = 512;
+static_assert(3 * MD_BLOCKS <= 32, "a warp hands a position to every block at once");
+
+// positions inside the sub-steps
+template <typename R> struct MdPos { typedef long long type; };
+template <> struct MdPos<double> { typedef double type; };
+
+__host__ __device__ inline int md_per_block(int nb) { return (nb + MD_BLOCKS - 1) / MD_BLOCKS; }
+
+// per bead of the chain: two copies of its position in P and in FP32, its
+// chain id, its two-step drag; per bead of the block: velocity, u^a, grad phi,
+// gamma, local position, block origin, scan box, wall flags
 template <typename R> inline size_t md_smem_bytes(int nb)
 {
-    return (size_t)nb * (3 * sizeof(double) + 27 * sizeof(R) + 6 * sizeof(float) + 10 * sizeof(int) +
-                         WALL_WORDS * sizeof(uint32_t));
+    const size_t all = (size_t)nb * (6 * sizeof(double) + 6 * sizeof(float) + sizeof(int));
+    const size_t own = (size_t)md_per_block(nb) * (29 * sizeof(R) + 9 * sizeof(int) + WALL_WORDS * sizeof(uint32_t));
+    return all + own + 64;
 }
 
-template <typename R> struct MdThreads {
-    static constexpr int value = sizeof(R) == 8 ? BEAD_THREADS : 1024;
-};
+__device__ __forceinline__ unsigned cluster_map(const void *p, int rank)
+{
+    unsigned a = (unsigned)__cvta_generic_to_shared(p), r;
+    asm("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(r) : "r"(a), "r"(rank));
+    return r;
+}
+__device__ __forceinline__ void cluster_st(unsigned a, float v)
+{
+    asm volatile("st.shared::cluster.f32 [%0], %1;" ::"r"(a), "f"(v) : "memory");
+}
+__device__ __forceinline__ void cluster_st(unsigned a, double v)
+{
+    asm volatile("st.shared::cluster.f64 [%0], %1;" ::"r"(a), "d"(v) : "memory");
+}
+__device__ __forceinline__ void cluster_st(unsigned a, long long v)
+{
+    asm volatile("st.shared::cluster.s64 [%0], %1;" ::"r"(a), "l"(v) : "memory");
+}
+__device__ __forceinline__ float cluster_ld(unsigned a, float)
+{
+    float v;
+    asm volatile("ld.shared::cluster.f32 %0, [%1];" : "=f"(v) : "r"(a) : "memory");
+    return v;
+}
+__device__ __forceinline__ double cluster_ld(unsigned a, double)
+{
+    double v;
+    asm volatile("ld.shared::cluster.f64 %0, [%1];" : "=d"(v) : "r"(a) : "memory");
+    return v;
+}
+// every thread of every block of the cluster; orders shared and global memory
+__device__ __forceinline__ void cluster_barrier()
+{
+    asm volatile("barrier.cluster.arrive.release.aligned;\n barrier.cluster.wait.acquire.aligned;" ::: "memory");
+}
 
 template <typename S, typename R, typename PhiT, bool DEV>
 __device__ void bead_md_body(const MdArgs<S, R, PhiT, DEV> &A)
 {
-    constexpr bool SERIAL = sizeof(R) == 8;
+    constexpr bool F64 = sizeof(R) == 8;
+    typedef typename MdPos<R>::type P;
     const StepArgs<S, R, PhiT> &a = A.s;
     const BeadArgs<R> &B = A.b;
     const Grid3 g = a.g;
     const int nb = B.nb;
     const int pc = *B.patch_count;
-    // dynamic shared memory, sized for nb beads (md_smem_bytes)
+    const int rank = blockIdx.x;  // cluster = the blocks of one grid row
+    const int per = md_per_block(nb), b0 = rank * per, own = max(0, min(per, nb - b0));
+    // dynamic shared memory (md_smem_bytes)
     extern __shared__ __align__(16) unsigned char md_smem[];
-    double *Rs = (double *)md_smem;              // positions, FP64 path
-    long long *Rq = (long long *)md_smem;        // positions, fixed point (other paths)
-    R *sV = (R *)(Rs + 3 * nb);
-    R *sU = sV + 3 * nb;
-    R *sG = sU + 9 * nb;
-    R *sGam = sG + 3 * nb;
-    R *sAcc = sGam + 3 * nb;
-    float *Rf = (float *)(sAcc + 9 * nb);
-    float *Rloc = Rf + 3 * nb;
-    int *worg = (int *)(Rloc + 3 * nb);
-    int *wlo = worg + 3 * nb;
-    int *wn = wlo + 3 * nb;
-    int *sChain = wn + 3 * nb;  // chain ids (read every sub-step)
+    P *pos = (P *)md_smem;                       // [2][3 nb]
+    R *sV = (R *)(pos + 6 * nb);                 // [3 per]
+    R *sU = sV + 3 * per;
+    R *sG = sU + 9 * per;
+    R *sGam = sG + 3 * per;
+    R *sAcc = sGam + 3 * per;
+    R *sQ = sAcc + 9 * per;                      // charge, thermal amplitude
+    float *Rf = (float *)(sQ + 2 * per);         // [2][3 nb]
+    int *worg = (int *)(Rf + 6 * nb);            // [3 per]
+    int *wlo = worg + 3 * per;
+    int *wn = wlo + 3 * per;
+    int *sChain = wn + 3 * per;                  // chain ids (read every sub-step)
     uint32_t *wbits = (uint32_t *)(sChain + nb);
     __shared__ int sBad;
     if (threadIdx.x == 0) sBad = 0;
     // moments at the patch nodes: thread (k, s) takes species s of node k,
     // thread (k, 3) the potential gradient (one memory round trip each)
-    for (int t = threadIdx.x; t < 4 * pc; t += blockDim.x) {
+    for (int t = rank * blockDim.x + threadIdx.x; t < 4 * pc; t += MD_BLOCKS * blockDim.x) {
         const int k = t >> 2, s = t & 3;
         long long i = B.patch_node[k];
         uint32_t m = a.mask[i];
@@ -1512,48 +1589,45 @@ __device__ void bead_md_body(const MdArgs<S, R, PhiT, DEV> &A)
                 if (cz_(p) == -1) jz -= v[p];
             }
             if (DEV) n = a.n_ref[s] + n;
-            out[s] = n;
-            out[3 + 3 * s + 0] = jx / n;
-            out[3 + 3 * s + 1] = jy / n;
-            out[3 + 3 * s + 2] = jz / n;
+            __stcg(out + s, n);
+            __stcg(out + 3 + 3 * s + 0, jx / n);
+            __stcg(out + 3 + 3 * s + 1, jy / n);
+            __stcg(out + 3 + 3 * s + 2, jz / n);
         } else {
             R gr[3];
             int olo[3], ohi[3];
             closed_faces(g, a.per, x, y, z, olo, ohi);
             node_gradient<R, PhiT>(a.phi, a.wall_share, a.c4, i, m, nbr, olo, ohi, gr);
-            out[12] = gr[0];
-            out[13] = gr[1];
-            out[14] = gr[2];
+            __stcg(out + 12, gr[0]);
+            __stcg(out + 13, gr[1]);
+            __stcg(out + 14, gr[2]);
         }
     }
+    const double rcd = 1.122462048309373 * (double)A.wall_sigma;  // 2^(1/6) sigma
+    P rcw;
+    if constexpr (F64) rcw = rcd;
+    else rcw = rcd < 16.0 ? __double2ll_rn(rcd * PHI_SCALE) : (16ll << 40);
     for (int t = threadIdx.x; t < 3 * nb; t += blockDim.x) {
         const double r = B.Rb[t];
-        if constexpr (SERIAL) Rs[t] = r;
-        else Rq[t] = __double2ll_rn(r * PHI_SCALE);
+        if constexpr (F64) pos[t] = r;
+        else pos[t] = __double2ll_rn(r * PHI_SCALE);
         Rf[t] = (float)r;
-        sV[t] = B.Vb[t];
     }
     for (int t = threadIdx.x; t < nb; t += blockDim.x) sChain[t] = B.chain[t];
-    for (int t = threadIdx.x; t < 9 * nb; t += blockDim.x) sAcc[t] = R(0);
-    const double rcw = 1.122462048309373 * (double)A.wall_sigma;  // 2^(1/6) sigma
-    const long long rcq = rcw < 16.0 ? __double2ll_rn(rcw * PHI_SCALE) : (16ll << 40);
-    int bad0 = 0;  // raised into sBad after the barrier that orders its reset
-    for (int t = threadIdx.x; t < 3 * nb; t += blockDim.x) {
-        const double r = B.Rb[t];
+    for (int t = threadIdx.x; t < 9 * own; t += blockDim.x) sAcc[t] = R(0);
+    for (int t = threadIdx.x; t < 3 * own; t += blockDim.x) {
+        const double r = B.Rb[3 * b0 + t];
         worg[t] = fabs(r) < 1e6 ? (int)floor(r) - WALL_BOX / 2 + 1 : 0;
-        int bad = 0;
-        scan_bounds(r, rcw, worg[t], wlo[t], wn[t], Rloc[t], bad);
-        bad0 |= bad;
+        sV[t] = B.Vb[3 * b0 + t];
     }
     __syncthreads();
-    if (bad0) sBad = 1;
     {
         // one word (32 cells of one bead's block) per warp and round, built by
         // a ballot; WALL_ROUNDS rounds' link words are loaded before any is used
         constexpr int WALL_ROUNDS = 8;
         const int dims[3] = {g.nx, g.ny, g.nz};
         const int cells = WALL_BOX * WALL_BOX * WALL_BOX;
-        const int words = nb * WALL_WORDS;
+        const int words = own * WALL_WORDS;
         const int wid = threadIdx.x >> 5, ln = threadIdx.x & 31, nw = blockDim.x >> 5;
         for (int w0 = wid; w0 < words; w0 += WALL_ROUNDS * nw) {
             bool solid[WALL_ROUNDS];
@@ -1589,54 +1663,54 @@ __device__ void bead_md_body(const MdArgs<S, R, PhiT, DEV> &A)
             }
         }
     }
-    // interpolation.  FP64: one thread per bead, entries in slot order k (the
-    // oracle's order).  Reduced precision: eight lanes per bead, one entry
-    // each (all loads in flight at once), summed over the lanes by shuffles.
-    auto interp_out = [&](int b, const R *v) {  // v: n^a (3), u^a (9), grad phi (3)
-        const R ntot = v[0] + v[1] + v[2];
-        for (int s = 0; s < NS; s++) {
-            sGam[3 * b + s] = (a.flags & EKL_GAMMA_LITERAL) ? A.xi : A.xi * v[s] / ntot;
-            for (int c = 0; c < 3; c++) sU[9 * b + 3 * s + c] = v[3 + 3 * s + c];
-        }
-        const R qb = B.qb[b];
-        for (int c = 0; c < 3; c++) {
-            sG[3 * b + c] = v[12 + c];
-            if (fabs(qb * v[12 + c]) >= R(1)) atomicOr(a.status, ST_CFL);
-        }
-    };
-    if constexpr (SERIAL) {
-        for (int b = threadIdx.x; b < nb; b += blockDim.x) {
-            R v[15];
-            for (int j = 0; j < 15; j++) v[j] = R(0);
-            for (int k = 0; k < 8; k++) {
-                R w = B.entry_w[b * 8 + k];
-                if (w == R(0)) continue;
-                int slot = B.entry_slot[b * 8 + k];
-                const R *mo = B.patch_mom + (long long)slot * 15;
-                for (int j = 0; j < 15; j++) v[j] += w * mo[j];
-            }
-            interp_out(b, v);
-        }
-    } else {
-        const int total = (8 * nb + 31) & ~31;  // whole warps: the shuffles below are warp-wide
+    // the patch moments of every block are complete after this
+    cluster_barrier();
+    // interpolation: eight lanes per bead, one entry each (all loads in
+    // flight at once), summed over the lanes by shuffles
+    {
+        const int total = (8 * own + 31) & ~31;  // whole warps: the shuffles below are warp-wide
         for (int t = threadIdx.x; t < total; t += blockDim.x) {
-            const int b = t >> 3, k = t & 7;
-            R v[15];
+            const int lb = t >> 3, k = t & 7, b = b0 + lb;
+            R v[15];  // n^a (3), u^a (9), grad phi (3)
 #pragma unroll
             for (int j = 0; j < 15; j++) v[j] = R(0);
-            if (b < nb) {
+            if (lb < own) {
                 const R w = B.entry_w[b * 8 + k];
                 if (w != R(0)) {
                     const R *mo = B.patch_mom + (long long)B.entry_slot[b * 8 + k] * 15;
 #pragma unroll
-                    for (int j = 0; j < 15; j++) v[j] = w * mo[j];
+                    for (int j = 0; j < 15; j++) v[j] = w * __ldcg(mo + j);
                 }
             }
+            if constexpr (F64) {  // in corner order, as the oracle
 #pragma unroll
-            for (int j = 0; j < 15; j++)
+                for (int j = 0; j < 15; j++) {
+                    R t = R(0);
 #pragma unroll
-                for (int o = 1; o < 8; o <<= 1) v[j] += __shfl_xor_sync(0xffffffffu, v[j], o);
-            if (k == 0 && b < nb) interp_out(b, v);
+                    for (int o = 0; o < 8; o++) t += __shfl_sync(0xffffffffu, v[j], (threadIdx.x & 24) + o);
+                    v[j] = t;
+                }
+            } else {
+#pragma unroll
+                for (int j = 0; j < 15; j++)
+#pragma unroll
+                    for (int o = 1; o < 8; o <<= 1) v[j] += __shfl_xor_sync(0xffffffffu, v[j], o);
+            }
+            if (k == 0 && lb < own) {
+                const R ntot = v[0] + v[1] + v[2];
+                for (int s = 0; s < NS; s++) {
+                    sGam[3 * lb + s] = (a.flags & EKL_GAMMA_LITERAL) ? A.xi : A.xi * v[s] / ntot;
+                    for (int c = 0; c < 3; c++) sU[9 * lb + 3 * s + c] = v[3 + 3 * s + c];
+                }
+                const R qb = B.qb[b], dt = R(1) / (R)A.md_substeps;
+                const R gtot = sGam[3 * lb] + sGam[3 * lb + 1] + sGam[3 * lb + 2];
+                sQ[2 * lb] = qb;
+                sQ[2 * lb + 1] = A.bead_kT > R(0) ? sqrt(R(2) * gtot * A.bead_kT / dt) : R(0);
+                for (int c = 0; c < 3; c++) {
+                    sG[3 * lb + c] = v[12 + c];
+                    if (fabs(qb * v[12 + c]) >= R(1)) atomicOr(a.status, ST_CFL);
+                }
+            }
         }
     }
     __syncthreads();
@@ -1644,102 +1718,117 @@ __device__ void bead_md_body(const MdArgs<S, R, PhiT, DEV> &A)
     const R dt = R(1) / (R)nsub;
     const bool noise = A.bead_kT > R(0) && !(a.flags & EKL_NO_BEAD_NOISE);
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, nwarps = blockDim.x >> 5;
-    // Reduced-precision instantiations: with one bead per warp and at most
-    // 32 sub-steps, lane s draws the sub-step-s noise of its warp's bead up
-    // front (the draws are independent of the dynamics)
-    const bool pre = !SERIAL && noise && nb <= nwarps && nsub <= 32;
-    float xpre[3] = {0.f, 0.f, 0.f};
-    if (pre && warp < nb && lane < nsub) {
-        uint32_t ctr[4] = {(uint32_t)warp, (uint32_t)lane | (1u << 24), (uint32_t)A.step,
+    // with one bead per warp and at most 32 sub-steps, lane s draws the
+    // sub-step-s noise of its warp's bead up front (the draws are
+    // independent of the dynamics)
+    auto draw = [&](int b, int sub, R x[3]) {
+        uint32_t ctr[4] = {(uint32_t)b, (uint32_t)sub | (1u << 24), (uint32_t)A.step,
                            (uint32_t)((uint64_t)A.step >> 32)};
         philox4x32_10(ctr, A.key0, A.key1);
-        for (int c = 0; c < 3; c++) xpre[c] = unit_variate_f32(ctr[c]);
-    }
+        for (int c = 0; c < 3; c++) {
+            if constexpr (F64) x[c] = unit_variate<R>(ctr[c]);
+            else x[c] = unit_variate_f32(ctr[c]);
+        }
+    };
+    const bool pre = noise && own <= nwarps && nsub <= 32;
+    R xpre[3] = {R(0), R(0), R(0)};
+    if (pre && warp < own && lane < nsub) draw(b0 + warp, lane, xpre);
+    int bad = 0;
     for (int sub = 0; sub < nsub; sub++) {
-        // force from the positions at the start of the sub-step, then the
-        // bead's own velocity and drag update (positions move after the barrier)
-        const int first = SERIAL ? (int)threadIdx.x : warp;
-        const int stride = SERIAL ? (int)blockDim.x : nwarps;
-        for (int b = first; b < nb; b += stride) {
+        const P *cur = pos + (sub & 1) * 3 * nb;
+        P *nxt = pos + ((sub & 1) ^ 1) * 3 * nb;
+        const float *curf = Rf + (sub & 1) * 3 * nb;
+        float *nxtf = Rf + ((sub & 1) ^ 1) * 3 * nb;
+        for (int lb = warp; lb < own; lb += nwarps) {
+            const int b = b0 + lb;
+            // the bead's wall scan box at the present position (lane c: coordinate c)
+            R loc = R(0);
+            if (lane < 3) {
+                int lo, n;
+                scan_bounds(cur[3 * b + lane], rcw, worg[3 * lb + lane], lo, n, loc, bad);
+                wlo[3 * lb + lane] = lo;
+                wn[3 * lb + lane] = n;
+            }
+            __syncwarp();
+            R rloc[3];
+            for (int c = 0; c < 3; c++) rloc[c] = __shfl_sync(0xffffffffu, loc, c);
             R F[3];
-            bool okf;
-            if constexpr (SERIAL) okf = bead_force_serial(A, Rs, b, F, &worg[3 * b], &wbits[b * WALL_WORDS]);
-            else okf = bead_force_warp(A, Rq, Rf, Rloc, wlo, wn, sChain, b, F, &worg[3 * b], &wbits[b * WALL_WORDS]);
-            if (!okf) sBad = 1;
+            if (!bead_force_warp(A, cur, curf, rloc, wlo + 3 * lb, wn + 3 * lb, sChain, b, F, worg + 3 * lb,
+                                 wbits + lb * WALL_WORDS))
+                bad = 1;
             R xi_[3] = {R(0), R(0), R(0)};
             if (noise) {
                 if (pre) {
                     for (int c = 0; c < 3; c++) xi_[c] = __shfl_sync(0xffffffffu, xpre[c], sub);
                 } else {
-                    uint32_t ctr[4] = {(uint32_t)b, (uint32_t)sub | (1u << 24), (uint32_t)A.step,
-                                       (uint32_t)((uint64_t)A.step >> 32)};
-                    philox4x32_10(ctr, A.key0, A.key1);
-                    for (int c = 0; c < 3; c++) {
-                        if constexpr (SERIAL) xi_[c] = unit_variate<R>(ctr[c]);
-                        else xi_[c] = unit_variate_f32(ctr[c]);
-                    }
+                    draw(b, sub, xi_);
                 }
             }
-            // the serial instantiation updates the three components in turn;
-            // the warp instantiation updates component `lane` in lanes 0-2
-            const int c0 = SERIAL ? 0 : lane, c1 = SERIAL ? 3 : lane + 1;
-            if (c0 >= 3) continue;
-            const R *gam = &sGam[3 * b];
-            R gtot = gam[0] + gam[1] + gam[2];
-            R amp = noise ? sqrt(R(2) * gtot * A.bead_kT / dt) : R(0);
-            R qb = B.qb[b];
-            for (int c = c0; c < c1; c++) {
+            // component `lane` in lanes 0-2: velocity and drag, then the new
+            // position, wrapped into [0, L) on periodic axes
+            P r = P(0);
+            float rf = 0.f;
+            if (lane < 3) {
+                const int c = lane;
+                const R *gam = &sGam[3 * lb];
+                R gtot = gam[0] + gam[1] + gam[2];
+                R amp = noise ? sQ[2 * lb + 1] : R(0);
+                R qb = sQ[2 * lb];
                 const R Fc = c == 0 ? F[0] : c == 1 ? F[1] : F[2];
                 const R xc = c == 0 ? xi_[0] : c == 1 ? xi_[1] : xi_[2];
-                R Fe = -qb * Consts<R>::KT * sG[3 * b + c] + qb * Consts<R>::KT * a.E[c];
-                R num = A.mass * sV[3 * b + c] / dt;
-                for (int s2 = 0; s2 < NS; s2++) num += gam[s2] * sU[9 * b + 3 * s2 + c];
+                R Fe = -qb * Consts<R>::KT * sG[3 * lb + c] + qb * Consts<R>::KT * a.E[c];
+                R num = A.mass * sV[3 * lb + c] / dt;
+                for (int s2 = 0; s2 < NS; s2++) num += gam[s2] * sU[9 * lb + 3 * s2 + c];
                 num += Fc + Fe + amp * xc;
                 R Vn = num / (A.mass / dt + gtot);
                 for (int s2 = 0; s2 < NS; s2++)
-                    sAcc[9 * b + 3 * s2 + c] += dt * (-gam[s2] * (sU[9 * b + 3 * s2 + c] - Vn));
-                sV[3 * b + c] = Vn;
-            }
-        }
-        __syncthreads();
-        // positions, wrapped into [0, L) on periodic axes
-        for (int t = threadIdx.x; t < 3 * nb; t += blockDim.x) {
-            const int c = t % 3;
-            const int Li = c == 0 ? g.nx : (c == 1 ? g.ny : g.nz);
-            int bad = 0;
-            if constexpr (SERIAL) {
-                const double L = Li;
-                double r = Rs[t] + (double)(dt * sV[t]);
-                if (B.per[c]) {
-                    if (r < 0.0) r += L;
-                    else if (r >= L) r -= L;
+                    sAcc[9 * lb + 3 * s2 + c] += dt * (-gam[s2] * (sU[9 * lb + 3 * s2 + c] - Vn));
+                sV[3 * lb + c] = Vn;
+                const int Li = c == 0 ? g.nx : (c == 1 ? g.ny : g.nz);
+                if constexpr (F64) {
+                    const double L = Li;
+                    r = cur[3 * b + c] + (double)(dt * Vn);
+                    if (B.per[c]) {
+                        if (r < 0.0) r += L;
+                        else if (r >= L) r -= L;
+                    }
+                    rf = (float)r;
+                    if (!(fabs(r) < 1e6)) bad = 1;
+                } else {
+                    const long long L = (long long)Li << 40;
+                    r = cur[3 * b + c] + float_to_ll((float)(dt * Vn) * (float)PHI_SCALE);
+                    if (B.per[c]) {
+                        if (r < 0) r += L;
+                        else if (r >= L) r -= L;
+                    }
+                    rf = ll_to_float(r) * (float)PHI_INV;
+                    if (!(r < (1ll << 60) && r > -(1ll << 60))) bad = 1;
                 }
-                Rs[t] = r;
-                Rf[t] = (float)r;
-                scan_bounds(r, rcw, worg[t], wlo[t], wn[t], Rloc[t], bad);
-            } else {
-                const long long L = (long long)Li << 40;
-                long long r = Rq[t] + float_to_ll((float)(dt * sV[t]) * (float)PHI_SCALE);
-                if (B.per[c]) {
-                    if (r < 0) r += L;
-                    else if (r >= L) r -= L;
-                }
-                Rq[t] = r;
-                Rf[t] = ll_to_float(r) * (float)PHI_INV;
-                scan_bounds_q(r, rcq, worg[t], wlo[t], wn[t], Rloc[t], bad);
             }
-            if (bad) sBad = 1;
+            // lane c + 3 k hands component c to block k
+            const int c = lane % 3, k = lane / 3;
+            r = __shfl_sync(0xffffffffu, r, c);
+            rf = __shfl_sync(0xffffffffu, rf, c);
+            if (k < MD_BLOCKS) {
+                cluster_st(cluster_map(nxt + 3 * b + c, k), r);
+                cluster_st(cluster_map(nxtf + 3 * b + c, k), rf);
+            }
+            __syncwarp();
         }
-        __syncthreads();
+        // new positions visible to every block, old ones no longer read
+        cluster_barrier();
     }
+    if (bad) sBad = 1;
+    __syncthreads();
     if (threadIdx.x == 0 && sBad) atomicOr(a.status, ST_BEAD);
-    for (int t = threadIdx.x; t < 3 * nb; t += blockDim.x) {
-        if constexpr (SERIAL) B.Rb[t] = Rs[t];
-        else B.Rb[t] = __ll2double_rn(Rq[t]) * PHI_INV;
-        B.Vb[t] = sV[t];
+    const P *end = pos + (nsub & 1) * 3 * nb;
+    for (int t = threadIdx.x; t < 3 * own; t += blockDim.x) {
+        if constexpr (F64) B.Rb[3 * b0 + t] = end[3 * b0 + t];
+        else B.Rb[3 * b0 + t] = __ll2double_rn(end[3 * b0 + t]) * PHI_INV;
+        B.Vb[3 * b0 + t] = sV[t];
     }
     // spread: per slot, entries in bead order (ascending b), then per particle
-    for (int k = threadIdx.x; k < pc; k += blockDim.x) {
+    for (int k = rank * blockDim.x + threadIdx.x; k < pc; k += MD_BLOCKS * blockDim.x) {
         R acc[9];
         for (int t = 0; t < 9; t++) acc[t] = R(0);
         const int t0 = B.slot_first[k], t1 = B.slot_first[k + 1];
@@ -1755,31 +1844,36 @@ __device__ void bead_md_body(const MdArgs<S, R, PhiT, DEV> &A)
 #pragma unroll
             for (int j = 0; j < 8; j++) {
                 if (w[j] == R(0)) continue;
-                const int bb = e[j] >> 3;
-                for (int u = 0; u < 9; u++) acc[u] += sAcc[bb * 9 + u] * w[j];
+                const int bb = e[j] >> 3, blk = bb / per;
+                const unsigned at = cluster_map(sAcc + (bb - blk * per) * 9, blk);
+                for (int u = 0; u < 9; u++) acc[u] += cluster_ld(at + u * (unsigned)sizeof(R), R(0)) * w[j];
             }
         }
         const R *mo = B.patch_mom + (long long)k * 15;
-        for (int s = 0; s < NS; s++)
+        for (int s = 0; s < NS; s++) {
+            const R n = __ldcg(mo + s);
             for (int c = 0; c < 3; c++) {
                 R v = acc[3 * s + c];
-                B.patch_f[(long long)k * 9 + 3 * s + c] = v != R(0) ? v / mo[s] : R(0);
+                B.patch_f[(long long)k * 9 + 3 * s + c] = v != R(0) ? v / n : R(0);
             }
+        }
     }
+    cluster_barrier();  // a block's drag is read by the others until here
 }
 
 template <typename S, typename R, typename PhiT, bool DEV>
-__global__ void __launch_bounds__(MdThreads<R>::value) bead_md_kernel(MdArgs<S, R, PhiT, DEV> A)
+__global__ void __cluster_dims__(MD_BLOCKS, 1, 1) __launch_bounds__(MD_THREADS) bead_md_kernel(MdArgs<S, R, PhiT, DEV> A)
 {
     bead_md_body<S, R, PhiT, DEV>(A);
 }
 
+// every replica of a batch: one cluster per blockIdx.y
 template <typename S, typename R, typename PhiT, bool DEV>
-__global__ void __launch_bounds__(MdThreads<R>::value)
+__global__ void __cluster_dims__(MD_BLOCKS, 1, 1) __launch_bounds__(MD_THREADS)
     bead_md_batch_kernel(const MdArgs<S, R, PhiT, DEV> *reps, long long step)
 {
     MdArgs<S, R, PhiT, DEV> A = reps[blockIdx.y];
-    if (A.b.nb == 0) return;
+    if (A.b.nb == 0) return;  // the whole cluster
     A.step = step;
     bead_md_body<S, R, PhiT, DEV>(A);
 }
@@ -1841,15 +1935,15 @@ __device__ __forceinline__ void lb_body(const StepArgs<S, R, PhiT> &a, long long
                 h[s] = R(0.5) * a.wd[s];
                 ih[s] = R(1) / (R(1) + h[s]);
                 // reduced-precision paths multiply by reciprocals; the FP64
-                // path divides exactly as the oracle does
-                const R in_ = DEV ? R(1) / n[s] : R(0);
+                // path rounds its quotients as the oracle does
+                const R in_ = R(1) / n[s];
                 R j[3] = {jx, jy, jz};
                 for (int c = 0; c < 3; c++) {
                     R zk = a.zv[s] * Consts<R>::KT;
                     R Gc = a.body[s][c] - zk * gphi[c] + zk * a.E[c];
                     if (slot >= 0) Gc = Gc + a.patch_f[(long long)slot * 9 + 3 * s + c];
                     G[s][c] = Gc;
-                    av[s][c] = (DEV ? j[c] * in_ : j[c] / n[s]) + R(0.5) * Gc;
+                    av[s][c] = (DEV ? j[c] * in_ : quot(j[c], n[s], in_)) + R(0.5) * Gc;
                 }
             }
             R num[3] = {R(0), R(0), R(0)}, den = R(0), us[3];
@@ -1859,21 +1953,17 @@ __device__ __forceinline__ void lb_body(const StepArgs<S, R, PhiT> &a, long long
                     den += n[s] * ih[s];
                     for (int c = 0; c < 3; c++) num[c] += n[s] * av[s][c] * ih[s];
                 } else {
-                    den += n[s] / (R(1) + h[s]);
-                    for (int c = 0; c < 3; c++) num[c] += n[s] * av[s][c] / (R(1) + h[s]);
+                    den += quot(n[s], R(1) + h[s], ih[s]);
+                    for (int c = 0; c < 3; c++) num[c] += quot(n[s] * av[s][c], R(1) + h[s], ih[s]);
                 }
             }
-            if constexpr (DEV) {
-                const R iden = R(1) / den;
-                for (int c = 0; c < 3; c++) us[c] = num[c] * iden;
-            } else {
-                for (int c = 0; c < 3; c++) us[c] = num[c] / den;
-            }
+            const R iden = R(1) / den;
+            for (int c = 0; c < 3; c++) us[c] = DEV ? num[c] * iden : quot(num[c], den, iden);
 #pragma unroll
             for (int s = 0; s < NS; s++) {
                 R ue[3], Ph[3];
                 for (int c = 0; c < 3; c++) {
-                    R ua = DEV ? (av[s][c] + h[s] * us[c]) * ih[s] : (av[s][c] + h[s] * us[c]) / (R(1) + h[s]);
+                    R ua = DEV ? (av[s][c] + h[s] * us[c]) * ih[s] : quot(av[s][c] + h[s] * us[c], R(1) + h[s], ih[s]);
                     Ph[c] = G[s][c] - a.wd[s] * (ua - us[c]);
                     ue[c] = (a.flags & EKL_EQ_BARYCENTRIC) ? us[c] : ua;
                 }
@@ -1911,16 +2001,40 @@ __device__ __forceinline__ void lb_body(const StepArgs<S, R, PhiT> &a, long long
                     }
                 };
                 if constexpr (!DEV) {
+                    // FP64: f - om (f - f_eq) + cS S, rounded operation by
+                    // operation as the oracle evaluates Eqs. 10, 12 and 13.
+                    // Bound by the FP64 rate, so a velocity and its opposite
+                    // share what is odd or even in c, products with the
+                    // components 0 and +-1 of c are left out, and quotients
+                    // take three operations (quot), with the same results
+                    // (64x64x128: 3.21 -> 1.46 ms).
+                    const R VT2 = Consts<R>::VT2;
+                    const R b1 = VT2, b2 = R(2) * VT2 * VT2, b3 = VT2 * VT2;
+                    const R r1 = R(1) / b1, r2 = R(1) / b2, r3 = R(1) / b3;
+                    const R vu2 = VT2 * u2, vFu = VT2 * Fu;
 #pragma unroll
-                    for (int p = 0; p < Q; p++) {
-                        const R cu = (R)cx_(p) * ue[0] + (R)cy_(p) * ue[1] + (R)cz_(p) * ue[2];
-                        const R cF = (R)cx_(p) * Ph[0] + (R)cy_(p) * Ph[1] + (R)cz_(p) * Ph[2];
-                        const R w = (R)w_(p);
-                        const R VT2 = Consts<R>::VT2;
-                        R feq = w * n[s] * (R(1) + cu / VT2 + (cu * cu - VT2 * u2) / (R(2) * VT2 * VT2));
-                        R Sp = w * n[s] * (cF / VT2 + (cu * cF - VT2 * Fu) / (VT2 * VT2));
-                        R fs = f[s][p] - om * (f[s][p] - feq) + cS * Sp;
-                        Store<S>::st(out + (long long)p * g.N, noisy(fs, p));
+                    for (int p = 0; p < Q; p += (p == 0 ? 1 : 2)) {
+                        R cu = R(0), cF = R(0);
+                        bool first = true;
+#pragma unroll
+                        for (int c = 0; c < 3; c++) {
+                            const int e = c == 0 ? cx_(p) : c == 1 ? cy_(p) : cz_(p);
+                            if (e == 0) continue;
+                            cu = first ? (e > 0 ? ue[c] : -ue[c]) : (e > 0 ? cu + ue[c] : cu - ue[c]);
+                            cF = first ? (e > 0 ? Ph[c] : -Ph[c]) : (e > 0 ? cF + Ph[c] : cF - Ph[c]);
+                            first = false;
+                        }
+                        const R wn = (R)w_(p) * n[s];
+                        const R a1 = quot(cu, b1, r1), a2 = quot(cu * cu - vu2, b2, r2);
+                        const R s1 = quot(cF, b1, r1), s2 = quot(cu * cF - vFu, b3, r3);
+#pragma unroll
+                        for (int o = 0; o < (p == 0 ? 1 : 2); o++) {
+                            const int q = p + o;  // p, then its opposite
+                            const R feq = wn * (R(1) + (o ? -a1 : a1) + a2);
+                            const R Sp = wn * ((o ? -s1 : s1) + s2);
+                            const R fs = f[s][q] - om * (f[s][q] - feq) + cS * Sp;
+                            Store<S>::st(out + (long long)q * g.N, noisy(fs, q));
+                        }
                     }
                 } else {
                     // deviation form, s_eq = f_eq - w n_ref:

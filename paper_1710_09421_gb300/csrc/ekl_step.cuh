@@ -429,7 +429,7 @@ template <typename S, typename R, typename PhiT, bool DEV> int steps_impl(Ctx &c
                                      (int)md_smem_bytes<R>(MAX_BEADS));
                 attr_set = true;
             }
-            bead_md_kernel<S, R, PhiT, DEV><<<1, MdThreads<R>::value, md_smem_bytes<R>(c.nb), c.stream>>>(md);
+            bead_md_kernel<S, R, PhiT, DEV><<<MD_BLOCKS, MD_THREADS, md_smem_bytes<R>(c.nb), c.stream>>>(md);
             c.launches++;
         }
         phase_end(c, PH_MD);
@@ -836,7 +836,7 @@ template <typename S, typename R, typename PhiT, bool DEV> int batch_impl(Batch 
                                      (int)md_smem_bytes<R>(MAX_BEADS));
                 attr = md_smem_bytes<R>(MAX_BEADS);
             }
-            bead_md_batch_kernel<S, R, PhiT, DEV><<<dim3(1, n), MdThreads<R>::value, smem, B.stream>>>(
+            bead_md_batch_kernel<S, R, PhiT, DEV><<<dim3(MD_BLOCKS, n), MD_THREADS, smem, B.stream>>>(
                 (const MdArgs<S, R, PhiT, DEV> *)B.d_mdargs[q], step);
             B.launches++;
         }
