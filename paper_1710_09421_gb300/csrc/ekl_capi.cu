@@ -772,7 +772,9 @@ static const char *build_multigrid(Ctx &c, const uint8_t *solid, Alloc &A, long 
     int maxdyn = 0;
     cudaDeviceGetAttribute(&maxdyn, cudaDevAttrMaxSharedMemoryPerBlockOptin, c.device);
     c.mg_cta_from = nlev - 1;
-    // per level: e and f (padded to 16 bytes) and the float4 conductances
+    // what decides how much of the hierarchy fits: six words per cell (and e and
+    // f padded to 16 bytes); the few words beside them fit in the 4096 bytes
+    // kept free for static shared memory
     auto cta_bytes = [&](int from) {
         size_t bytes = 0;
         for (int k = from; k < nlev; k++)
@@ -784,15 +786,14 @@ static const char *build_multigrid(Ctx &c, const uint8_t *solid, Alloc &A, long 
             c.mg_cta_from = l;
             break;
         }
-    c.mg_smem = cta_bytes(c.mg_cta_from);
+    size_t need = cta_bytes(c.mg_cta_from);
     if (c.mg_dense) {  // exact coarsest solve: every other level is grid-wide
         c.mg_cta_from = nlev - 1;
-        c.mg_smem = 0;
+        need = 0;
     }
     // tiled smoothing from the first grid-wide coarse level small enough per
     // block; its region follows block 0's levels in the dynamic shared memory
     c.mg_tile_from = c.mg_cta_from;
-    c.mg_tile_off = c.mg_smem / sizeof(float);
     size_t tile_words = 0;
     for (int l = 1; tiles && l < c.mg_cta_from; l++) {
         if ((long long)c.mg_lev[l].N > (long long)MG_TILE_CELLS_PER_BLOCK * c.pois_blocks) continue;
@@ -800,8 +801,17 @@ static const char *build_multigrid(Ctx &c, const uint8_t *solid, Alloc &A, long 
         const int ex[3] = {c.mg_lev[l].nx, c.mg_lev[l].ny, c.mg_lev[l].nz};
         mg_pick_tile(ex, 2 * MG_NU_COARSE, c.pois_blocks, 16, MG_TILE_BYTES, c.mg_tile[l], tile_words);
     }
-    c.mg_smem += tile_words * sizeof(float);
-    if (c.mg_smem + 4096 > (size_t)maxdyn) return "coarsest multigrid level too large for shared memory";
+    need += tile_words * sizeof(float);
+    if (need + 4096 > (size_t)maxdyn) return "coarsest multigrid level too large for shared memory";
+    const size_t tile_bytes = tile_words ? (tile_words + MG_TILE_EXTRA) * sizeof(float) : 0;
+    for (int pad : {31, 0}) {
+        size_t words = 0;
+        for (int l = c.mg_cta_from; l < nlev && !c.mg_dense; l++) words += mg_cta_words(c.mg_lev[l].N, pad);
+        c.mg_cta_pad = pad;
+        c.mg_tile_off = (int)words;
+        c.mg_smem = words * sizeof(float) + tile_bytes;
+        if (c.mg_smem + 4096 <= (size_t)maxdyn) break;
+    }
     // large lattices per SM make the lattice passes bandwidth-bound: twice the
     // warps in flight (1024-thread blocks) then beat the 512-thread launch
     // that keeps 128 registers a thread for the latency-bound small solve
@@ -812,7 +822,16 @@ static const char *build_multigrid(Ctx &c, const uint8_t *solid, Alloc &A, long 
     c.mg_split = split;
     c.mgs_threads = c.mg_wide ? MG_WIDE_THREADS : MG_THREADS;
     c.mgs_l1 = c.mg_split && c.mg_cta_from > 1 && c.mg_tile_from > 1;
-    c.mgs_iter_kernels = 2 * (2 * MG_NU - 1) + 8 + (c.mgs_l1 ? 2 * (2 * MG_NU_COARSE - 1) + 2 : 0);
+    // two half sweeps per launch on lattices whose solve does not stay in L2
+    // (37 bytes a node: r, z, p, p', q, the link byte, and phi and b of 8),
+    // where rows split into aligned pieces of four nodes: 256x256x512 takes 5.63
+    // ms per solve with it and 7.64 with one half sweep per launch, 128x128x256
+    // 1.25 and 1.40, and 64x64x128, bound by the chain of plane steps, 0.59 and
+    // 0.50.
+    const size_t l2 = 126u << 20;
+    c.mg_fused = c.mg_split && c.mg_wide && c.nx % 4 == 0 && (size_t)N * 37 > l2;
+    c.mgs_iter_kernels = (c.mg_fused ? 11 : 2 * (2 * MG_NU - 1) + 8) +
+                         (c.mgs_l1 ? 2 * (2 * MG_NU_COARSE - 1) + 2 : 0);
     if (ops(c.prec).mg_blocks(c.mg_smem, c.mg_wide) < 1) return "multigrid kernel cannot be resident";
     c.mg_r = (float *)A(N * sizeof(float));
     c.mg_link = (uint8_t *)A(N);
@@ -1036,7 +1055,8 @@ static int create_handle(const ekl_params *P, void *stream, ekl_handle **out, bo
     c.charge_chunks = A(CHARGE_CHUNK_BYTES);
     c.part_mass = (double *)A((size_t)((N + 255) / 256) * NS * sizeof(double));
     c.part_pois = (double *)A((size_t)c.pois_blocks * sizeof(double));
-    c.barrier = (unsigned *)A(4 * sizeof(unsigned));
+    c.barrier = (unsigned *)A(4 * sizeof(unsigned) + CHARGE_SLOTS * sizeof(unsigned long long));
+    c.charge_slots = (unsigned long long *)(c.barrier + 4);
     c.status = (int *)A(sizeof(int));
     c.pois_iters = (int *)A(sizeof(int));
     c.pois_total = (long long *)A(sizeof(long long));

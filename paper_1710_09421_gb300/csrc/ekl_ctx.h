@@ -13,6 +13,7 @@ constexpr int MAX_BEADS = 256;
 constexpr int MAX_ENTRIES = 8 * MAX_BEADS;
 constexpr int LB_THREADS = 128;
 constexpr int CHARGE_THREADS = 256;
+constexpr int CHARGE_SLOTS = 64;    // words the charge pass adds its exact total in (a power of two)
 constexpr int POIS_THREADS = 1024;
 constexpr int MG_THREADS = 512;     // multigrid launch: one block per SM (latency-bound solve)
 constexpr int MG_WIDE_THREADS = 1024;  // the same for lattices of at least MG_WIDE_NODES_PER_SM nodes per SM
@@ -92,7 +93,8 @@ struct Ctx {
     void *charge_chunks;       // its per-block chunk totals and arrival counter (zeroed)
     double *part_mass;    // [mass blocks][3] (filled on request)
     double *part_pois;    // [poisson blocks][2]
-    unsigned *barrier;    // {count, generation, abort}
+    unsigned *barrier;    // {count, generation, abort, -}, then charge_slots
+    unsigned long long *charge_slots;  // [CHARGE_SLOTS], zeroed with the barrier words before each step
     int *status;          // device status word
     int *pois_iters;      // last step's sweep count
     long long *pois_total;  // sweeps summed over all steps
@@ -125,6 +127,7 @@ struct Ctx {
     int mg_nlev;             // levels including the lattice
     int mg_cta_from;         // first level handled by one block alone
     int mg_wide;             // launch the solve with MG_WIDE_THREADS-thread blocks
+    int mg_cta_pad;          // padding of those levels' arrays (mg_cta_half)
     int mg_tile_from;        // first level smoothed in shared-memory tiles (mg_cta_from: none)
     int mg_tile[MG_MAXLEV][3];  // owned cells per tile of each tiled level
     size_t mg_tile_off;      // offset (floats) of the tile region in the dynamic shared memory
@@ -141,6 +144,7 @@ struct Ctx {
     cudaGraph_t mgs_graph;   // its CG loop, built at the first solve
     cudaGraphExec_t mgs_exec;
     int mgs_iter_kernels;    // kernels launched per CG iteration of the loop
+    int mg_fused;            // lattice passes two half sweeps per launch (ekl_mgf.cuh)
     int mgs_l1;              // level 1 grid-wide: smoothed by separate launches in the loop
     int mgs_threads;         // block size of its lattice launches (that of the single launch it matches)
 

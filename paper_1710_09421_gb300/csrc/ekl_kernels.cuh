@@ -55,6 +55,11 @@ template <typename S, typename R, typename PhiT> struct StepArgs {
     // the partials itself
     double *charge_tot;
     long long *charge_tot_q;
+    // single handles on the fixed-point paths: the exact totals added up by
+    // the charge pass itself, in CHARGE_SLOTS words zeroed before it (integer
+    // sums: their order does not matter), in place of the two above; then
+    // part_charge may be null too
+    unsigned long long *charge_slots;
     double *part_mass;
     double *part_pois;
     unsigned *barrier;
@@ -211,12 +216,14 @@ __device__ __forceinline__ void charge_body(const StepArgs<S, R, PhiT> &a, long 
     }
     // one FP64 partial per block (fixed shuffle tree per warp, warps in
     // order), so that the Poisson launch sums few partials
-    __shared__ double csh[CHARGE_THREADS / 32];
-    double t;
-    if constexpr (sizeof(R) == 8) t = warp_sum((double)mine);
-    else t = warp_sum_ff_lane0((float)mine);
-    t = block_sum_lanes0(t, csh);
-    if (threadIdx.x == 0) a.part_charge[blk] = t;
+    if (a.part_charge) {
+        __shared__ double csh[CHARGE_THREADS / 32];
+        double t;
+        if constexpr (sizeof(R) == 8) t = warp_sum((double)mine);
+        else t = warp_sum_ff_lane0((float)mine);
+        t = block_sum_lanes0(t, csh);
+        if (threadIdx.x == 0) a.part_charge[blk] = t;
+    }
     if constexpr (!(((PhiT)0.5) != 0)) {
         // the fixed-point source's exact total: sum of rho * 2^40 as the
         // Poisson launch rounds it (integer, order-independent)
@@ -229,7 +236,8 @@ __device__ __forceinline__ void charge_body(const StepArgs<S, R, PhiT> &a, long 
         if (threadIdx.x == 0) {
             long long s = 0;
             for (int w = 0; w < (int)(blockDim.x >> 5); w++) s += qsh[w];
-            a.part_charge_q[blk] = s;
+            if (a.charge_slots) atomicAdd(a.charge_slots + (blk & (CHARGE_SLOTS - 1)), (unsigned long long)s);
+            else a.part_charge_q[blk] = s;
         }
     }
 }
@@ -423,14 +431,18 @@ template <typename S, typename R, typename PhiT>
 __device__ SrcMean source_mean(const StepArgs<S, R, PhiT> &a, double *bc)
 {
     SrcMean sm{0.0, 0, 0, 0.f};
-    const double csum = a.charge_tot ? __ldcg(a.charge_tot) : sum_partials(a.part_charge, a.nblocks_charge, bc);
     const double nfl = a.n_fluid;
-    sm.mean = nfl > 0 ? csum / nfl : 0.0;
+    if constexpr (((PhiT)0.5) != 0) {
+        const double csum = a.charge_tot ? __ldcg(a.charge_tot) : sum_partials(a.part_charge, a.nblocks_charge, bc);
+        sm.mean = nfl > 0 ? csum / nfl : 0.0;
+    }
     // fixed point: the exact total S of rho * 2^40 over the fluid nodes,
     // S / n = mean_lo + frac with 0 <= frac < 1, and C = c4 frac split into
     // integer and fraction
     if constexpr (!(((PhiT)0.5) != 0)) {
-        const long long Sq = a.charge_tot ? __ldcg(a.charge_tot_q) : sum_partials_ll(a.part_charge_q, a.nblocks_charge);
+        const long long Sq = a.charge_slots ? sum_partials_ll((const long long *)a.charge_slots, CHARGE_SLOTS)
+                             : a.charge_tot ? __ldcg(a.charge_tot_q)
+                                            : sum_partials_ll(a.part_charge_q, a.nblocks_charge);
         const long long n = (long long)nfl;
         if (n > 0) {
             long long mean_lo = Sq / n;

@@ -46,6 +46,7 @@ struct MgArgs {
     int have_prev;        // phi_prev holds phi(t-2) and phi holds phi(t-1)
     int nlev, cta_from, nu, nu_c, coarse_sweeps;  // smoothing sweeps: lattice level, coarse levels
     float inner_red;
+    int cta_pad;                  // padding of block 0's levels (mg_cta_half)
     int tile_from;                // first tiled coarse level (cta_from: none)
     int tile_off;                 // tile region offset (floats) in the dynamic shared memory
     int tile[MG_MAXLEV][3];       // owned cells per tile, per level
@@ -64,14 +65,16 @@ struct MgCtl {
     int done;       // batches: this replica's loop has ended
 };
 
-// 4-byte words of shared memory for a tile region of Rx x Ry x Rz cells:
-// e and f (each padded to 16 bytes), the float4 conductances, and the
-// wrapped level coordinates of the region's columns, rows and planes
-__host__ __device__ inline size_t mg_tile_words(int Rx, int Ry, int Rz)
+// 4-byte words of shared memory for a tile region of Rx x Ry x Rz cells (Rx
+// even): correction, right-hand side, three conductances and 1/diagonal per
+// cell; and beside them a little slack around each array and the wrapped level
+// coordinates of the region's columns, rows and planes (tiles reach at most
+// 16 cells and a halo of 2 MG_NU_COARSE at either side)
+inline size_t mg_tile_words(int Rx, int Ry, int Rz)
 {
-    const size_t RN = (size_t)Rx * Ry * Rz, RN4 = (RN + 3) & ~(size_t)3;
-    return 2 * RN4 + 4 * RN + (size_t)Rx + Ry + Rz;
+    return 6 * (size_t)Rx * Ry * Rz;
 }
+constexpr size_t MG_TILE_EXTRA = 8 + 3 * (16 + 4 * MG_NU_COARSE);
 
 // The blocks that solve one problem: all blocks of a single-handle launch, or
 // the blocks a batched launch assigns to one replica (each replica then runs
@@ -125,43 +128,6 @@ __device__ __forceinline__ Pair mg_pair(int h, int hx, int ny, int c)
 
 // load of a value no block writes during the current phase (L1-cached)
 template <typename T> __device__ __forceinline__ T mg_ldl(const T *p) { return __ldca(p); }
-
-template <bool SH> __device__ __forceinline__ float mg_ld(const float *p)
-{
-    if constexpr (SH) return *p;
-    else return mg_ldl(p);
-}
-template <bool SH> __device__ __forceinline__ void mg_st(float *p, float v)
-{
-    if constexpr (SH) *p = v;
-    else __stcg(p, v);
-}
-// conductances: read-only global memory, or block 0's shared-memory copy
-template <bool SH> __device__ __forceinline__ float4 mg_sig(const float4 *p)
-{
-    if constexpr (SH) return *p;
-    else return __ldg(p);
-}
-template <bool SH> __device__ __forceinline__ float mg_sx(const float4 *p)
-{
-    if constexpr (SH) return p->x;
-    else return __ldg(&p->x);
-}
-template <bool SH> __device__ __forceinline__ float mg_sy(const float4 *p)
-{
-    if constexpr (SH) return p->y;
-    else return __ldg(&p->y);
-}
-template <bool SH> __device__ __forceinline__ float mg_sz(const float4 *p)
-{
-    if constexpr (SH) return p->z;
-    else return __ldg(&p->z);
-}
-template <bool SH> __device__ __forceinline__ float mg_sw(const float4 *p)
-{
-    if constexpr (SH) return p->w;
-    else return __ldg(&p->w);
-}
 
 // ------------------------------------------------------------ lattice level
 // The first half sweep of every smoothing pass starts from zero, so it only
@@ -387,8 +353,6 @@ static __device__ void fine_restrict_warp(const Grid3 &g, const L *__restrict__ 
 }
 
 // ------------------------------------------------------------ coarse levels
-// SH: the level's e and f live in shared memory (block 0's part of the cycle);
-// the conductances always come from global memory.
 struct CNbr {
     int xm, xp, ym, yp, zm, zp;
 };
@@ -406,11 +370,11 @@ __device__ __forceinline__ CNbr coarse_nbrs(const MgLevel &L, int x, int y, int 
 }
 
 // value of neighbour j (coordinates X, Y, Z), with the coarser correction when PRO
-template <bool SH, bool PRO>
+template <bool PRO>
 __device__ __forceinline__ float coarse_val(const MgLevel &L, const MgLevel &C, int j, int X, int Y, int Z)
 {
-    float v = mg_ld<SH>(L.e + j);
-    if (PRO) v += mg_ld<SH>(C.e + mg_parent(C, X, Y, Z));
+    float v = mg_ldl(L.e + j);
+    if (PRO) v += mg_ldl(C.e + mg_parent(C, X, Y, Z));
     return v;
 }
 
@@ -445,7 +409,7 @@ __device__ __forceinline__ float mg_cresid(float f, float e, float4 s, float sxm
 // before its activity (1/diag = 0 on inactive cells) is known, so a cell
 // costs one memory round trip, not two; a thread takes U cells per trip
 // (h, h + nt, ...) with all their loads issued first.
-template <bool SH, bool PRO, int U = 1>
+template <bool PRO, int U = 1>
 static __device__ void coarse_half(const MgLevel &L, const MgLevel &C, int c, int t0, int nt)
 {
     const int hx = (L.nx + 1) >> 1, np = hx * L.ny * L.nz;
@@ -467,40 +431,39 @@ static __device__ void coarse_half(const MgLevel &L, const MgLevel &C, int c, in
             const int xm = p.x == 0 ? L.nx - 1 : p.x - 1, xp = p.x == L.nx - 1 ? 0 : p.x + 1;
             const int ym = p.y == 0 ? L.ny - 1 : p.y - 1, yp = p.y == L.ny - 1 ? 0 : p.y + 1;
             const int zm = p.z == 0 ? L.nz - 1 : p.z - 1, zp = p.z == L.nz - 1 ? 0 : p.z + 1;
-            const float4 s = mg_sig<SH>(L.sig + i);
+            const float4 s = __ldg(L.sig + i);
             w[u] = s.w;
-            v[u] = mg_relax(mg_ld<SH>(L.f + i), s, mg_sx<SH>(L.sig + n.xm), mg_sy<SH>(L.sig + n.ym),
-                            mg_sz<SH>(L.sig + n.zm), coarse_val<SH, PRO>(L, C, n.xp, xp, p.y, p.z),
-                            coarse_val<SH, PRO>(L, C, n.xm, xm, p.y, p.z),
-                            coarse_val<SH, PRO>(L, C, n.yp, p.x, yp, p.z),
-                            coarse_val<SH, PRO>(L, C, n.ym, p.x, ym, p.z),
-                            coarse_val<SH, PRO>(L, C, n.zp, p.x, p.y, zp),
-                            coarse_val<SH, PRO>(L, C, n.zm, p.x, p.y, zm));
+            v[u] = mg_relax(mg_ldl(L.f + i), s, __ldg(&L.sig[n.xm].x), __ldg(&L.sig[n.ym].y),
+                            __ldg(&L.sig[n.zm].z), coarse_val<PRO>(L, C, n.xp, xp, p.y, p.z),
+                            coarse_val<PRO>(L, C, n.xm, xm, p.y, p.z),
+                            coarse_val<PRO>(L, C, n.yp, p.x, yp, p.z),
+                            coarse_val<PRO>(L, C, n.ym, p.x, ym, p.z),
+                            coarse_val<PRO>(L, C, n.zp, p.x, p.y, zp),
+                            coarse_val<PRO>(L, C, n.zm, p.x, p.y, zm));
         }
 #pragma unroll
         for (int u = 0; u < U; u++)
-            if (w[u] != 0.f) mg_st<SH>(L.e + ii[u], v[u]);
+            if (w[u] != 0.f) __stcg(L.e + ii[u], v[u]);
     }
 }
 
-template <bool SH>
 __device__ __forceinline__ float coarse_resid(const MgLevel &L, int x, int y, int z)
 {
     if (x >= L.nx || y >= L.ny || z >= L.nz) return 0.f;
     const int i = x + L.nx * (y + L.ny * z);
-    const float4 sg = mg_sig<SH>(L.sig + i);
+    const float4 sg = __ldg(L.sig + i);
     const CNbr n = coarse_nbrs(L, x, y, z, i);
     // formed before the activity test, so all its loads are in flight at once
-    const float res = mg_cresid(mg_ld<SH>(L.f + i), mg_ld<SH>(L.e + i), sg, mg_sx<SH>(L.sig + n.xm),
-                                mg_sy<SH>(L.sig + n.ym), mg_sz<SH>(L.sig + n.zm), mg_ld<SH>(L.e + n.xp),
-                                mg_ld<SH>(L.e + n.xm), mg_ld<SH>(L.e + n.yp), mg_ld<SH>(L.e + n.ym),
-                                mg_ld<SH>(L.e + n.zp), mg_ld<SH>(L.e + n.zm));
+    const float res = mg_cresid(mg_ldl(L.f + i), mg_ldl(L.e + i), sg, __ldg(&L.sig[n.xm].x),
+                                __ldg(&L.sig[n.ym].y), __ldg(&L.sig[n.zm].z), mg_ldl(L.e + n.xp),
+                                mg_ldl(L.e + n.xm), mg_ldl(L.e + n.yp), mg_ldl(L.e + n.ym),
+                                mg_ldl(L.e + n.zp), mg_ldl(L.e + n.zm));
     return sg.w == 0.f ? 0.f : res;
 }
 
 // C.f = sum over the children of each cell of level l+1 of (f - A e) on
 // level l; FIRST: also start C's pre-smoothing
-template <bool SH, bool FIRST>
+template <bool FIRST>
 static __device__ void coarse_restrict(const MgLevel &L, const MgLevel &C, int t0, int nt)
 {
     const int lane = threadIdx.x & 31, total = ((C.N + 7) >> 3) * 32;
@@ -514,12 +477,12 @@ static __device__ void coarse_restrict(const MgLevel &L, const MgLevel &C, int t
             Y = t % C.ny;
             Z = t / C.ny;
             const int y0 = 2 * Y + (k & 1), z0 = 2 * Z + (k >> 1);
-            acc = coarse_resid<SH>(L, 2 * X, y0, z0) + coarse_resid<SH>(L, 2 * X + 1, y0, z0);
+            acc = coarse_resid(L, 2 * X, y0, z0) + coarse_resid(L, 2 * X + 1, y0, z0);
         }
         const float sum = mg_sum_rows(acc);
         if (I < C.N && k == 0) {
-            mg_st<SH>(C.f + I, sum);
-            if (FIRST && !((X + Y + Z) & 1)) mg_st<SH>(C.e + I, sum * mg_sw<SH>(C.sig + I));
+            __stcg(C.f + I, sum);
+            if (FIRST && !((X + Y + Z) & 1)) __stcg(C.e + I, sum * __ldg(&C.sig[I].w));
         }
     }
 }
@@ -535,26 +498,38 @@ static __device__ void coarse_restrict(const MgLevel &L, const MgLevel &C, int t
 // cells, which all take the same values), and every update and residual
 // uses mg_relax / mg_cresid on the same inputs as the global sweeps: results
 // are identical, at one grid barrier per smoothing pass.
-constexpr int TILE_LOADS = 4;  // region cells a thread loads per round
+//
+// The region's two colours are kept apart, each array one value per x-pair
+// (cells 2 h and 2 h + 1 of a row): a cell of colour q on x-parity s finds
+// all its neighbours in the other colour's arrays at its own index, but for
+// one of its x neighbours, at the next (s = 1) or previous (s = 0) one.  Every
+// access of a warp is then to consecutive words (with both colours in one
+// array of float4 conductances a warp's loads of a half sweep took 46 bank
+// cycles, now 14).
+constexpr int TILE_PAIRS = 2;  // region x-pairs a thread loads per round
 struct TileSm {
-    float *e, *f;
-    float4 *s;
+    float *e, *f, *sx, *sy, *sz, *w;  // [2 colours][half]
     int *wx, *wy, *wz;
-    int Rx, Ry, Rz;
+    int Rx, Ry, Rz, hx, pl, half;     // pairs per row and plane, pairs of the region
 };
 __device__ __forceinline__ TileSm tile_sm(float *sm, int Rx, int Ry, int Rz)
 {
     TileSm T;
-    const int RN = Rx * Ry * Rz, RN4 = (RN + 3) & ~3;
-    T.e = sm;
-    T.f = sm + RN4;
-    T.s = (float4 *)(sm + 2 * RN4);
-    T.wx = (int *)(T.s + RN);
-    T.wy = T.wx + Rx;
-    T.wz = T.wy + Ry;
     T.Rx = Rx;
     T.Ry = Ry;
     T.Rz = Rz;
+    T.hx = Rx >> 1;
+    T.pl = T.hx * Ry;
+    T.half = T.pl * Rz;
+    T.e = sm + 4;  // (the x neighbour beyond the first or last row's end is read in the slack, and not used)
+    T.f = T.e + 2 * T.half;
+    T.sx = T.f + 2 * T.half;
+    T.sy = T.sx + 2 * T.half;
+    T.sz = T.sy + 2 * T.half;
+    T.w = T.sz + 2 * T.half;
+    T.wx = (int *)(T.w + 2 * T.half + 4);
+    T.wy = T.wx + Rx;
+    T.wz = T.wy + Ry;
     return T;
 }
 
@@ -583,31 +558,84 @@ __device__ __forceinline__ void tile_coords(const TileSm &T, const MgLevel &L, i
     }
 }
 
-// Half sweep of colour col over the region cells at least `lo` layers from
-// the region's faces.  Colours follow the region coordinates (parity base at
-// the region origin): they equal the level's colours everywhere the owned
-// cells' results depend on, since periodic extents are even and a closed
-// side decouples the wrapped cells beyond it (zero conductance).  A thread
-// takes an x-pair and updates its colour-col cell.
-static __device__ void tile_half(const TileSm &T, int lo, int col, int base)
+// Half sweep of colour col over the rows and planes at least `lo` layers from
+// the region's faces (along x whole rows: what a row's ends take in from
+// beyond the region moves inward one cell per half sweep, like the layers
+// left out in the other directions, and is not used).  Colours follow the
+// region coordinates (parity base at the region origin): they equal the
+// level's colours everywhere the owned cells' results depend on, since
+// periodic extents are even and a closed side decouples the wrapped cells
+// beyond it (zero conductance).
+static __device__ void tile_half(const TileSm &T, int lo, int col, int base, float ihx)
 {
-    const int bx = T.Rx - 2 * lo, by = T.Ry - 2 * lo, bz = T.Rz - 2 * lo;
-    const int bxh = (bx + 1) >> 1, np = bxh * by * bz;
-    const float ibxh = 1.f / (float)bxh, iby = 1.f / (float)by;
-    const int sy = T.Rx, sz = T.Rx * T.Ry, amax = T.Rx - lo;
-    for (int h = threadIdx.x; h < np; h += blockDim.x) {
-        int xh, b, c;
-        tsplit(h, bxh, by, ibxh, iby, xh, b, c);
-        b += lo;
-        c += lo;
-        const int a0 = lo + 2 * xh;
-        const int a = a0 + ((a0 + b + c + base + col) & 1);
-        if (a >= amax) continue;
-        const int k = a + sy * b + sz * c;
-        const float4 s = T.s[k];
-        if (s.w == 0.f) continue;
-        T.e[k] = mg_relax(T.f[k], s, T.s[k - 1].x, T.s[k - sy].y, T.s[k - sz].z, T.e[k + 1], T.e[k - 1],
-                          T.e[k + sy], T.e[k - sy], T.e[k + sz], T.e[k - sz]);
+    const int by = T.Ry - 2 * lo, per_plane = T.hx * by, np = per_plane * (T.Rz - 2 * lo);
+    const float ipp = __frcp_rn((float)per_plane);
+    float *e = T.e + col * T.half;
+    const int oc = (col ^ 1) * T.half;
+    const float *oe = T.e + oc, *osx = T.sx + oc, *osy = T.sy + oc, *osz = T.sz + oc;
+    const int own = col * T.half, hx = T.hx, pl = T.pl;
+    for (int t = threadIdx.x; t < np; t += blockDim.x) {
+        const int c = tdiv(t, ipp), r = t - c * per_plane, b = tdiv(r, ihx);
+        const int k = (lo + c) * pl + lo * hx + r;
+        const int sp = (b + c + base + col) & 1;  // (2 lo does not change the parity)
+        const int xm = k - 1 + sp, xp = k + sp;
+        const float4 s = make_float4(T.sx[own + k], T.sy[own + k], T.sz[own + k], T.w[own + k]);
+        const float v = mg_relax(T.f[own + k], s, osx[xm], osy[k - hx], osz[k - pl], oe[xp], oe[xm], oe[k + hx],
+                                 oe[k - hx], oe[k + pl], oe[k - pl]);
+        e[k] = s.w == 0.f ? 0.f : v;
+    }
+}
+
+// One x-pair of the region from the level: conductances, right-hand side and
+// (PRE) the first values, colour 0 from zero, else colour 0 from the
+// pre-smoothed correction plus the coarser one
+template <bool PRE>
+static __device__ void tile_load(const TileSm &T, const MgLevel &L, const MgLevel &C, int base, float ihx, float iRy)
+{
+    for (int t0 = threadIdx.x; t0 < T.half; t0 += TILE_PAIRS * blockDim.x) {
+        float4 sv[TILE_PAIRS][2];
+        float fv[TILE_PAIRS][2], tv[TILE_PAIRS], cv[TILE_PAIRS];
+        int ce[TILE_PAIRS];  // colour of the even cell
+#pragma unroll
+        for (int u = 0; u < TILE_PAIRS; u++) {
+            const int t = t0 + u * blockDim.x;
+            if (t >= T.half) continue;
+            int h, b, c;
+            tsplit(t, T.hx, T.Ry, ihx, iRy, h, b, c);
+            ce[u] = (b + c + base) & 1;
+            const int gy = T.wy[b], gz = T.wz[c], row = L.nx * (gy + L.ny * gz);
+#pragma unroll
+            for (int q = 0; q < 2; q++) {
+                const int i = T.wx[2 * h + q] + row;
+                sv[u][q] = __ldg(L.sig + i);
+                fv[u][q] = __ldcg(L.f + i);
+            }
+            if (!PRE) {
+                const int gx = T.wx[2 * h + ce[u]];  // the pair's colour-0 cell
+                tv[u] = __ldcg(L.t + gx + row);
+                cv[u] = __ldcg(C.e + mg_parent(C, gx, gy, gz));
+            }
+        }
+#pragma unroll
+        for (int u = 0; u < TILE_PAIRS; u++) {
+            const int t = t0 + u * blockDim.x;
+            if (t >= T.half) continue;
+#pragma unroll
+            for (int q = 0; q < 2; q++) {
+                const int k = (ce[u] ^ q) * T.half + t;
+                T.sx[k] = sv[u][q].x;
+                T.sy[k] = sv[u][q].y;
+                T.sz[k] = sv[u][q].z;
+                T.w[k] = sv[u][q].w;
+                T.f[k] = fv[u][q];
+            }
+            const int z = ce[u];  // the colour-0 cell of the pair
+            float v;
+            if (PRE) v = (z ? fv[u][1] : fv[u][0]) * (z ? sv[u][1].w : sv[u][0].w);
+            else v = tv[u] + cv[u];
+            T.e[t] = v;
+            T.e[T.half + t] = 0.f;  // overwritten before it is read
+        }
     }
 }
 
@@ -626,85 +654,70 @@ __device__ __forceinline__ int tile_count(const MgLevel &L, const int *tdim)
 }
 
 // Pre-smoothing of level L from its right-hand side (colour 0 from zero, then
-// 2 nu_c - 1 half sweeps), the smoothed correction of the owned cells into
-// L.t, and the restricted residual of the owned parents into C.f.
+// 2 nu_c - 1 half sweeps), the smoothed colour-0 corrections of the owned cells
+// into L.t, and the restricted residual of the owned parents into C.f.
 static __device__ void coarse_pre_tiles(const MgLevel &L, const MgLevel &C, const int *tdim, int H, int blk,
                                         int nblk, float *sm)
 {
     const int tx = tdim[0], ty = tdim[1], tz = tdim[2];
-    const TileSm T = tile_sm(sm, tx + 2 * H, ty + 2 * H, tz + 2 * H);
-    const int RN = T.Rx * T.Ry * T.Rz, sy = T.Rx, sz = T.Rx * T.Ry;
-    const float iRx = 1.f / (float)T.Rx, iRy = 1.f / (float)T.Ry, itx = 1.f / (float)tx, ity = 1.f / (float)ty;
-    const int px = tx >> 1, py = ty >> 1, pz = tz >> 1;
-    const float ipx = 1.f / (float)px, ipy = 1.f / (float)py;
     const int ntiles = tile_count(L, tdim);
+    if (blk >= ntiles) return;
+    const TileSm T = tile_sm(sm, tx + 2 * H, ty + 2 * H, tz + 2 * H);
+    const int hx = T.hx, pl = T.pl;
+    const float ihx = __frcp_rn((float)hx), iRy = __frcp_rn((float)T.Ry);
+    const int px = tx >> 1, py = ty >> 1, pz = tz >> 1;
+    const float ipx = __frcp_rn((float)px), ipy = __frcp_rn((float)py), ity = __frcp_rn((float)ty);
     for (int t = blk; t < ntiles; t += nblk) {
         int x0, y0, z0;
         tile_origin(L, tdim, t, x0, y0, z0);
         const int base = (x0 + y0 + z0 - 3 * H) & 1;
         tile_coords(T, L, x0 - H, y0 - H, z0 - H);
         __syncthreads();
-        // TILE_LOADS cells per thread in flight at once (the loads of one
-        // round are independent: one L2 round trip per round, not per cell)
-        for (int k0 = threadIdx.x; k0 < RN; k0 += TILE_LOADS * blockDim.x) {
-            float4 sv[TILE_LOADS];
-            float fv[TILE_LOADS];
-            int col[TILE_LOADS];
-#pragma unroll
-            for (int j = 0; j < TILE_LOADS; j++) {
-                const int k = k0 + j * blockDim.x;
-                if (k < RN) {
-                    int a, b, c;
-                    tsplit(k, T.Rx, T.Ry, iRx, iRy, a, b, c);
-                    const int i = T.wx[a] + L.nx * (T.wy[b] + L.ny * T.wz[c]);
-                    sv[j] = __ldg(L.sig + i);
-                    fv[j] = __ldcg(L.f + i);
-                    col[j] = (a + b + c + base) & 1;
-                }
-            }
-#pragma unroll
-            for (int j = 0; j < TILE_LOADS; j++) {
-                const int k = k0 + j * blockDim.x;
-                if (k < RN) {
-                    T.s[k] = sv[j];
-                    T.f[k] = fv[j];
-                    T.e[k] = col[j] ? 0.f : fv[j] * sv[j].w;
-                }
-            }
-        }
+        tile_load<true>(T, L, C, base, ihx, iRy);
         __syncthreads();
         for (int h = 1; h < H; h++) {
-            tile_half(T, h, h & 1, base);
+            tile_half(T, h, h & 1, base, ihx);
             __syncthreads();
         }
-        // residual of the owned cells (in place of f), and their correction
-        for (int k = threadIdx.x; k < tx * ty * tz; k += blockDim.x) {
+        // residuals of the owned cells, summed over each x-pair (in place of
+        // colour 0's right-hand side), and the colour-0 corrections
+        for (int k = threadIdx.x; k < px * ty * tz; k += blockDim.x) {
             int a, b, c;
-            tsplit(k, tx, ty, itx, ity, a, b, c);
-            const int X = x0 + a, Y = y0 + b, Z = z0 + c;
-            const int q = (a + H) + sy * (b + H) + sz * (c + H);
-            float res = 0.f;
-            if (X < L.nx && Y < L.ny && Z < L.nz) {
-                const float4 s = T.s[q];
-                if (s.w != 0.f)
-                    res = mg_cresid(T.f[q], T.e[q], s, T.s[q - 1].x, T.s[q - sy].y, T.s[q - sz].z, T.e[q + 1],
-                                    T.e[q - 1], T.e[q + sy], T.e[q - sy], T.e[q + sz], T.e[q - sz]);
-                __stcg(L.t + X + L.nx * (Y + L.ny * Z), T.e[q]);
+            tsplit(k, px, ty, ipx, ity, a, b, c);
+            const int q = (H + c) * pl + (H + b) * hx + H / 2 + a;
+            const int s0 = (b + c + base + H) & 1;  // x-parity of the pair's colour-0 cell (3 H - 2 H)
+            const int Y = y0 + b, Z = z0 + c;
+            float sum = 0.f;
+            if (Y < L.ny && Z < L.nz) {
+                float res[2];
+#pragma unroll
+                for (int col = 0; col < 2; col++) {
+                    const int sp = s0 ^ col, X = x0 + 2 * a + sp;
+                    const int own = col * T.half + q, o = (col ^ 1) * T.half + q;
+                    const int xm = o - 1 + sp, xp = o + sp;
+                    const float4 s = make_float4(T.sx[own], T.sy[own], T.sz[own], T.w[own]);
+                    res[col] = 0.f;
+                    if (X < L.nx) {
+                        const float r = mg_cresid(T.f[own], T.e[own], s, T.sx[xm], T.sy[o - hx], T.sz[o - pl], T.e[xp],
+                                                  T.e[xm], T.e[o + hx], T.e[o - hx], T.e[o + pl], T.e[o - pl]);
+                        if (s.w != 0.f) res[col] = r;
+                        if (col == 0) __stcg(L.t + X + L.nx * (Y + L.ny * Z), T.e[own]);
+                    }
+                }
+                sum = res[0] + res[1];
             }
-            T.f[q] = res;
+            T.f[q] = sum;
         }
         __syncthreads();
-        // children summed as the global restriction does: each (dy, dz) row's
-        // two x-children, then rows (0 + 1) + (2 + 3) with row = dy + 2 dz
+        // children summed as the global restriction does: rows (0 + 1) + (2 + 3)
+        // with row = dy + 2 dz
         for (int k = threadIdx.x; k < px * py * pz; k += blockDim.x) {
             int a, b, c;
             tsplit(k, px, py, ipx, ipy, a, b, c);
             const int X = (x0 >> 1) + a, Y = (y0 >> 1) + b, Z = (z0 >> 1) + c;
             if (X >= C.nx || Y >= C.ny || Z >= C.nz) continue;
-            const int q = (2 * a + H) + sy * (2 * b + H) + sz * (2 * c + H);
-            const float r0 = T.f[q] + T.f[q + 1], r1 = T.f[q + sy] + T.f[q + sy + 1];
-            const float r2 = T.f[q + sz] + T.f[q + sz + 1], r3 = T.f[q + sz + sy] + T.f[q + sz + sy + 1];
-            __stcg(C.f + X + C.nx * (Y + C.ny * Z), (r0 + r1) + (r2 + r3));
+            const int q = (H + 2 * c) * pl + (H + 2 * b) * hx + H / 2 + a;
+            __stcg(C.f + X + C.nx * (Y + C.ny * Z), (T.f[q] + T.f[q + hx]) + (T.f[q + pl] + T.f[q + pl + hx]));
         }
         __syncthreads();
     }
@@ -718,165 +731,364 @@ static __device__ void coarse_post_tiles(const MgLevel &L, const MgLevel &C, con
                                          int nblk, float *sm)
 {
     const int tx = tdim[0], ty = tdim[1], tz = tdim[2];
-    const TileSm T = tile_sm(sm, tx + 2 * H, ty + 2 * H, tz + 2 * H);
-    const int RN = T.Rx * T.Ry * T.Rz, sy = T.Rx, sz = T.Rx * T.Ry;
-    const float iRx = 1.f / (float)T.Rx, iRy = 1.f / (float)T.Ry, itx = 1.f / (float)tx, ity = 1.f / (float)ty;
     const int ntiles = tile_count(L, tdim);
+    if (blk >= ntiles) return;
+    const TileSm T = tile_sm(sm, tx + 2 * H, ty + 2 * H, tz + 2 * H);
+    const float ihx = __frcp_rn((float)T.hx), iRy = __frcp_rn((float)T.Ry), itx = __frcp_rn((float)tx),
+                ity = __frcp_rn((float)ty);
     for (int t = blk; t < ntiles; t += nblk) {
         int x0, y0, z0;
         tile_origin(L, tdim, t, x0, y0, z0);
         const int base = (x0 + y0 + z0 - 3 * H) & 1;
         tile_coords(T, L, x0 - H, y0 - H, z0 - H);
         __syncthreads();
-        for (int k0 = threadIdx.x; k0 < RN; k0 += TILE_LOADS * blockDim.x) {
-            float4 sv[TILE_LOADS];
-            float fv[TILE_LOADS], tv[TILE_LOADS], cv[TILE_LOADS];
-#pragma unroll
-            for (int j = 0; j < TILE_LOADS; j++) {
-                const int k = k0 + j * blockDim.x;
-                if (k < RN) {
-                    int a, b, c;
-                    tsplit(k, T.Rx, T.Ry, iRx, iRy, a, b, c);
-                    const int gx = T.wx[a], gy = T.wy[b], gz = T.wz[c];
-                    const int i = gx + L.nx * (gy + L.ny * gz);
-                    sv[j] = __ldg(L.sig + i);
-                    fv[j] = __ldcg(L.f + i);
-                    tv[j] = 0.f;
-                    cv[j] = 0.f;
-                    if (!((a + b + c + base) & 1)) {
-                        tv[j] = __ldcg(L.t + i);
-                        cv[j] = __ldcg(C.e + mg_parent(C, gx, gy, gz));
-                    }
-                }
-            }
-#pragma unroll
-            for (int j = 0; j < TILE_LOADS; j++) {
-                const int k = k0 + j * blockDim.x;
-                if (k < RN) {
-                    T.s[k] = sv[j];
-                    T.f[k] = fv[j];
-                    float v = tv[j];
-                    v += cv[j];
-                    T.e[k] = v;
-                }
-            }
-        }
+        tile_load<false>(T, L, C, base, ihx, iRy);
         __syncthreads();
         for (int h = 0; h < H; h++) {
-            tile_half(T, h + 1, (h & 1) ^ 1, base);
+            tile_half(T, h + 1, (h & 1) ^ 1, base, ihx);
             __syncthreads();
         }
         for (int k = threadIdx.x; k < tx * ty * tz; k += blockDim.x) {
             int a, b, c;
             tsplit(k, tx, ty, itx, ity, a, b, c);
             const int X = x0 + a, Y = y0 + b, Z = z0 + c;
-            const int q = (a + H) + sy * (b + H) + sz * (c + H);
-            if (X < L.nx && Y < L.ny && Z < L.nz && T.s[q].w != 0.f) __stcg(L.e + X + L.nx * (Y + L.ny * Z), T.e[q]);
+            const int col = (a + b + c + base + 3 * H) & 1;
+            const int q = col * T.half + (H + c) * T.pl + (H + b) * T.hx + ((H + a) >> 1);
+            if (X < L.nx && Y < L.ny && Z < L.nz && T.w[q] != 0.f) __stcg(L.e + X + L.nx * (Y + L.ny * Z), T.e[q]);
         }
         __syncthreads();
     }
 }
 
-// mean of v over the active cells of level L (block-wide, every thread gets it)
-static __device__ float coarse_mean(const MgLevel &L, const float *v, double *sh, double *bc)
+// ------------------------------------------------------------ block 0's levels
+// A level of block 0 in its shared memory: correction, right-hand side, the
+// +x, +y, +z conductances and 1 / diagonal, each in an array of its own split
+// by the parity of the linear cell index (even ones first).  The cells of one
+// colour in a row then lie in consecutive words, whatever the extents, and a
+// warp's loads of a half sweep meet no bank twice.  With e and f in index
+// order and the conductances as float4 beside them every update cost 30 bank
+// cycles, and its indices two divisions: 67 us per V-cycle on a coarsest level
+// of 20 x 12 x 18 cells, now 27 (16 half sweeps of 1900 cycles; two FP64 means
+// of 8000).
+struct CtaLev {
+    int nx, ny, nz, N, M;  // M: cells per parity (rounded up)
+    float *e, *f, *sx, *sy, *sz, *w;
+};
+// cells per parity, rounded up; `pad` (0 or 31): to a multiple of 32, so that
+// rows that start in different parities share no bank either (padded where
+// shared memory has the room; 2-way conflicts otherwise)
+__host__ __device__ inline int mg_cta_half(long long N, int pad) { return (int)((N + 1) / 2 + pad) & ~pad; }
+// words of a level
+__host__ __device__ inline size_t mg_cta_words(long long N, int pad) { return 12 * (size_t)mg_cta_half(N, pad); }
+
+__device__ __forceinline__ CtaLev cta_level(const MgArgs &m, int l)
 {
-    double s = 0.0, n = 0.0;
-    for (int i = threadIdx.x; i < L.N; i += blockDim.x)
-        if (L.sig[i].w != 0.f) {
-            s += (double)v[i];
-            n += 1.0;
+    extern __shared__ float mg_sm[];  // (named here, not passed: loads known to be from shared memory)
+    float *sm = mg_sm;
+    for (int k = m.cta_from; k < l; k++) sm += mg_cta_words(m.lev[k].N, m.cta_pad);
+    CtaLev L;
+    L.nx = m.lev[l].nx;
+    L.ny = m.lev[l].ny;
+    L.nz = m.lev[l].nz;
+    L.N = m.lev[l].N;
+    L.M = mg_cta_half(L.N, m.cta_pad);
+    L.e = sm;
+    L.f = L.e + 2 * L.M;
+    L.sx = L.f + 2 * L.M;
+    L.sy = L.sx + 2 * L.M;
+    L.sz = L.sy + 2 * L.M;
+    L.w = L.sz + 2 * L.M;
+    return L;
+}
+__device__ __forceinline__ int cta_at(const CtaLev &L, int i) { return (i & 1) * L.M + (i >> 1); }
+
+// block 0, once per launch: the conductances of its levels into shared memory,
+// four loads of a thread in flight at a time
+static __device__ __noinline__ void mg_cta_load(const MgArgs &m)
+{
+    for (int l = m.cta_from; l < m.nlev; l++) {
+        const CtaLev L = cta_level(m, l);
+        for (int i0 = threadIdx.x; i0 < L.N; i0 += 4 * blockDim.x) {
+            float4 s[4];
+#pragma unroll
+            for (int u = 0; u < 4; u++) {
+                const int i = i0 + u * blockDim.x;
+                if (i < L.N) s[u] = __ldg(m.lev[l].sig + i);
+            }
+#pragma unroll
+            for (int u = 0; u < 4; u++) {
+                const int i = i0 + u * blockDim.x, q = cta_at(L, i);
+                if (i >= L.N) break;
+                L.sx[q] = s[u].x;
+                L.sy[q] = s[u].y;
+                L.sz[q] = s[u].z;
+                L.w[q] = s[u].w;
+            }
         }
+    }
+    __syncthreads();
+}
+
+// A cell's linear index and, from bit 16 on, its place at a side of the level
+// (bit f: its neighbour across face f wraps); CTA_NONE: no cell.  A level of
+// block 0 has fewer than 2^16 cells.
+constexpr unsigned CTA_NONE = 0xFFFFFFFFu;
+__device__ __forceinline__ unsigned cta_cell(const CtaLev &L, int x, int y, int z)
+{
+    unsigned q = (unsigned)(x + L.nx * (y + L.ny * z));
+    if (x == 0) q |= 1u << 16;
+    if (x == L.nx - 1) q |= 2u << 16;
+    if (y == 0) q |= 4u << 16;
+    if (y == L.ny - 1) q |= 8u << 16;
+    if (z == 0) q |= 16u << 16;
+    if (z == L.nz - 1) q |= 32u << 16;
+    return q;
+}
+// array positions of a cell's neighbours in face order
+__device__ __forceinline__ void cta_nbrs(const CtaLev &L, unsigned q, int nb[6])
+{
+    const int i = q & 0xFFFFu, nxy = L.nx * L.ny;
+    nb[0] = cta_at(L, i + ((q >> 16 & 1u) ? L.nx - 1 : -1));
+    nb[1] = cta_at(L, i + ((q >> 17 & 1u) ? 1 - L.nx : 1));
+    nb[2] = cta_at(L, i + ((q >> 18 & 1u) ? nxy - L.nx : -L.nx));
+    nb[3] = cta_at(L, i + ((q >> 19 & 1u) ? L.nx - nxy : L.nx));
+    nb[4] = cta_at(L, i + ((q >> 20 & 1u) ? L.N - nxy : -nxy));
+    nb[5] = cta_at(L, i + ((q >> 21 & 1u) ? nxy - L.N : nxy));
+}
+// the cell of colour c in pair h
+__device__ __forceinline__ unsigned cta_pair(const CtaLev &L, int h, int c)
+{
+    const int hx = (L.nx + 1) >> 1;
+    if (h >= hx * L.ny * L.nz) return CTA_NONE;
+    const Pair p = mg_pair(h, hx, L.ny, c);
+    return p.x < L.nx ? cta_cell(L, p.x, p.y, p.z) : CTA_NONE;
+}
+// Byte offsets of a cell and its neighbours in their arrays, two to a word
+// (zp = CTA_NONE: no cell)
+struct CtaIx {
+    unsigned own_xm, xp_ym, yp_zm, zp;
+};
+__device__ __forceinline__ CtaIx cta_offsets(const CtaLev &L, unsigned q)
+{
+    if (q == CTA_NONE) return {0, 0, 0, CTA_NONE};
+    int nb[6];
+    cta_nbrs(L, q, nb);
+    return {(unsigned)cta_at(L, q & 0xFFFFu) * 4 | (unsigned)nb[0] << 18, (unsigned)nb[1] * 4 | (unsigned)nb[2] << 18,
+            (unsigned)nb[3] * 4 | (unsigned)nb[4] << 18, (unsigned)nb[5] * 4};
+}
+__device__ __forceinline__ float cta_v(const float *p, unsigned off) { return *(const float *)((const char *)p + off); }
+// the updated value of a cell, to be stored at offset i (CTA_NONE: nowhere)
+__device__ __forceinline__ float cta_relax(const CtaLev &L, const CtaIx &q, unsigned &i)
+{
+    const unsigned own = q.own_xm & 0xFFFFu, xm = q.own_xm >> 16, xp = q.xp_ym & 0xFFFFu, ym = q.xp_ym >> 16,
+                   yp = q.yp_zm & 0xFFFFu, zm = q.yp_zm >> 16;
+    i = CTA_NONE;
+    if (q.zp == CTA_NONE) return 0.f;
+    const float4 s = make_float4(cta_v(L.sx, own), cta_v(L.sy, own), cta_v(L.sz, own), cta_v(L.w, own));
+    if (s.w != 0.f) i = own;
+    return mg_relax(cta_v(L.f, own), s, cta_v(L.sx, xm), cta_v(L.sy, ym), cta_v(L.sz, zm), cta_v(L.e, xp),
+                    cta_v(L.e, xm), cta_v(L.e, yp), cta_v(L.e, ym), cta_v(L.e, q.zp), cta_v(L.e, zm));
+}
+
+// pairs per thread: in kernels of at most 512 threads, and in larger ones
+constexpr int CTA_U = 5, CTA_U_WIDE = 2;
+// n half sweeps, the first of colour c.  A thread's cells stay the same in
+// every sweep of a colour: the offsets of its first U pairs are found once and
+// kept in registers.  All values are formed before the first store: cells of
+// one colour do not read one another, which the compiler cannot know.
+template <int U> static __device__ __noinline__ void cta_sweeps(const MgArgs &m, int l, int c, int n)
+{
+    const CtaLev L = cta_level(m, l);
+    const int t0 = threadIdx.x, nt = blockDim.x, np = ((L.nx + 1) >> 1) * L.ny * L.nz;
+    CtaIx qa[U], qb[U];
+#pragma unroll
+    for (int u = 0; u < U; u++) {
+        qa[u] = cta_offsets(L, cta_pair(L, t0 + u * nt, c));
+        qb[u] = cta_offsets(L, cta_pair(L, t0 + u * nt, c ^ 1));
+    }
+    for (int s = 0; s < n; s++) {
+        float v[U];
+        unsigned i[U];
+        if (s & 1) {
+#pragma unroll
+            for (int u = 0; u < U; u++) v[u] = cta_relax(L, qb[u], i[u]);
+        } else {
+#pragma unroll
+            for (int u = 0; u < U; u++) v[u] = cta_relax(L, qa[u], i[u]);
+        }
+#pragma unroll
+        for (int u = 0; u < U; u++)
+            if (i[u] != CTA_NONE) *(float *)((char *)L.e + i[u]) = v[u];
+        for (int h = t0 + U * nt; h < np; h += nt) {
+            unsigned k;
+            const float x = cta_relax(L, cta_offsets(L, cta_pair(L, h, (c + s) & 1)), k);
+            if (k != CTA_NONE) *(float *)((char *)L.e + k) = x;
+        }
+        __syncthreads();
+    }
+}
+
+// half sweep of colour c whose neighbours' values include the correction of
+// their parents on level C
+static __device__ __noinline__ void cta_prolong(const MgArgs &m, int l, int c)
+{
+    const CtaLev L = cta_level(m, l), C = cta_level(m, l + 1);
+    const int hx = (L.nx + 1) >> 1, np = hx * L.ny * L.nz;
+    for (int h = threadIdx.x; h < np; h += blockDim.x) {
+        const Pair p = mg_pair(h, hx, L.ny, c);
+        if (p.x >= L.nx) continue;
+        const unsigned q = cta_cell(L, p.x, p.y, p.z);
+        int nb[6];
+        cta_nbrs(L, q, nb);
+        float v[6];
+#pragma unroll
+        for (int f = 0; f < 6; f++) {
+            int X, Y, Z;
+            mg_face_coord(L.nx, L.ny, L.nz, p.x, p.y, p.z, f, X, Y, Z);
+            v[f] = L.e[nb[f]] + C.e[cta_at(C, (X >> 1) + C.nx * ((Y >> 1) + C.ny * (Z >> 1)))];
+        }
+        const int i = cta_at(L, q & 0xFFFFu);
+        const float4 s = make_float4(L.sx[i], L.sy[i], L.sz[i], L.w[i]);
+        const float r = mg_relax(L.f[i], s, L.sx[nb[0]], L.sy[nb[2]], L.sz[nb[4]], v[1], v[0], v[3], v[2], v[5], v[4]);
+        if (s.w != 0.f) L.e[i] = r;
+    }
+    __syncthreads();
+}
+
+__device__ __forceinline__ float cta_resid(const CtaLev &L, int x, int y, int z)
+{
+    if (x >= L.nx || y >= L.ny || z >= L.nz) return 0.f;
+    const unsigned q = cta_cell(L, x, y, z);
+    int nb[6];
+    cta_nbrs(L, q, nb);
+    const int i = cta_at(L, q & 0xFFFFu);
+    const float4 s = make_float4(L.sx[i], L.sy[i], L.sz[i], L.w[i]);
+    const float res = mg_cresid(L.f[i], L.e[i], s, L.sx[nb[0]], L.sy[nb[2]], L.sz[nb[4]], L.e[nb[1]], L.e[nb[0]],
+                                L.e[nb[3]], L.e[nb[2]], L.e[nb[5]], L.e[nb[4]]);
+    return s.w == 0.f ? 0.f : res;
+}
+// coarse_restrict between two levels of block 0
+template <bool FIRST> static __device__ __noinline__ void cta_restrict(const MgArgs &m, int l)
+{
+    const CtaLev L = cta_level(m, l), C = cta_level(m, l + 1);
+    const int lane = threadIdx.x & 31, total = ((C.N + 7) >> 3) * 32;
+    for (int base = threadIdx.x - lane; base < total; base += blockDim.x) {
+        const int I = (base >> 2) + (lane & 7), k = lane >> 3;
+        float acc = 0.f;
+        int X = 0, Y = 0, Z = 0;
+        if (I < C.N) {
+            X = I % C.nx;
+            const int t = I / C.nx;
+            Y = t % C.ny;
+            Z = t / C.ny;
+            const int y0 = 2 * Y + (k & 1), z0 = 2 * Z + (k >> 1);
+            acc = cta_resid(L, 2 * X, y0, z0) + cta_resid(L, 2 * X + 1, y0, z0);
+        }
+        const float sum = mg_sum_rows(acc);
+        if (I < C.N && k == 0) {
+            const int q = cta_at(C, I);
+            C.f[q] = sum;
+            if (FIRST && !((X + Y + Z) & 1)) C.e[q] = sum * C.w[q];
+        }
+    }
+    __syncthreads();
+}
+
+// (double)v by integer arithmetic: conversions share the FP64 pipe, which takes
+// 16 cycles per warp instruction
+__device__ __forceinline__ double mg_widen(float v)
+{
+    const unsigned u = __float_as_uint(v), a = u & 0x7FFFFFFFu;
+    if (a - 0x00800000u >= 0x7F000000u && a != 0) return (double)v;  // subnormal, infinite or NaN
+    return a == 0 ? __hiloint2double((int)u, 0)
+                  : __hiloint2double((int)((u & 0x80000000u) | ((a >> 3) + 0x38000000u)), (int)(u << 29));
+}
+
+// mean of the right-hand side (or the correction) over the active cells of
+// level l (block-wide, every thread gets it)
+static __device__ __noinline__ float cta_mean(const MgArgs &m, int l, bool of_e, double *sh, double *bc)
+{
+    const CtaLev L = cta_level(m, l);
+    const float *v = of_e ? L.e : L.f;
+    __shared__ int cnt[32];
+    double s = 0.0;
+    int n = 0;
+    for (int i = threadIdx.x; i < L.N; i += blockDim.x) {
+        const int q = cta_at(L, i);
+        if (L.w[q] != 0.f) {
+            s += mg_widen(v[q]);
+            n++;
+        }
+    }
+    n = __reduce_add_sync(0xffffffffu, n);
+    if ((threadIdx.x & 31) == 0) cnt[threadIdx.x >> 5] = n;
     const double ts = block_sum(s, sh);
-    const double tn = block_sum(n, sh);
-    if (threadIdx.x == 0) bc[0] = tn > 0 ? ts / tn : 0.0;
+    if (threadIdx.x == 0) {
+        int tn = 0;
+        for (int k = 0; k < (int)(blockDim.x + 31) >> 5; k++) tn += cnt[k];
+        bc[0] = tn > 0 ? ts / (double)tn : 0.0;
+    }
     __syncthreads();
     const float mean = (float)bc[0];
     __syncthreads();
     return mean;
 }
 
-// Shared-memory layout of block 0's levels (l >= cta_from): per level e[N]
-// and f[N] (floats, padded to 16 bytes) then sig[N] (float4).
-__device__ __forceinline__ void mg_cta_levels(const MgArgs &m, float *sm, MgLevel *Ls)
-{
-    size_t off = 0;
-    for (int l = m.cta_from; l < m.nlev; l++) {
-        Ls[l] = m.lev[l];
-        const size_t n2 = (2 * (size_t)Ls[l].N + 3) & ~(size_t)3;
-        Ls[l].e = sm + off;
-        Ls[l].f = sm + off + Ls[l].N;
-        Ls[l].sig = (float4 *)(sm + off + n2);
-        off += n2 + 4 * (size_t)Ls[l].N;
-    }
-}
-
-// block 0, once per launch: the conductances of its levels into shared memory
-static __device__ void mg_cta_load(const MgArgs &m, float *sm)
-{
-    MgLevel Ls[MG_MAXLEV];
-    mg_cta_levels(m, sm, Ls);
-    for (int l = m.cta_from; l < m.nlev; l++)
-        for (int i = threadIdx.x; i < Ls[l].N; i += blockDim.x) Ls[l].sig[i] = __ldg(m.lev[l].sig + i);
-    __syncthreads();
-}
-
 // Block 0 alone: the V-cycle at and below level m.cta_from in shared memory.
 // On entry the level's right-hand side is in global memory; on exit its
 // correction is written back there.
-static __device__ void mg_cta_cycle(const MgArgs &m, float *sm, double *sh, double *bc)
+template <int U> static __device__ __noinline__ void mg_cta_cycle(const MgArgs &m, double *sh, double *bc)
 {
     const int t0 = threadIdx.x, nt = blockDim.x;
     const int k0 = m.cta_from, last = m.nlev - 1;
-    MgLevel Ls[MG_MAXLEV];
-    mg_cta_levels(m, sm, Ls);
     // the right-hand side, and the first half sweep unless k0 is the coarsest
     {
-        const MgLevel &L = Ls[k0];
-        for (int i = t0; i < L.N; i += nt) {
-            const float f = __ldcg(m.lev[k0].f + i);
-            L.f[i] = f;
-            L.e[i] = k0 < last ? f * L.sig[i].w : 0.f;  // colour 1 is overwritten first
+        const CtaLev L = cta_level(m, k0);
+        for (int i0 = t0; i0 < L.N; i0 += 5 * nt) {  // (five round trips to memory at a time)
+            float f[5];
+#pragma unroll
+            for (int u = 0; u < 5; u++) f[u] = i0 + u * nt < L.N ? __ldcg(m.lev[k0].f + i0 + u * nt) : 0.f;
+#pragma unroll
+            for (int u = 0; u < 5; u++) {
+                if (i0 + u * nt >= L.N) break;
+                const int q = cta_at(L, i0 + u * nt);
+                L.f[q] = f[u];
+                L.e[q] = k0 < last ? f[u] * L.w[q] : 0.f;  // colour 1 is overwritten first
+            }
         }
         __syncthreads();
     }
     for (int l = k0; l < last; l++) {
-        for (int s = 1; s < 2 * m.nu_c; s++) {
-            coarse_half<true, false>(Ls[l], Ls[l], s & 1, t0, nt);
-            __syncthreads();
-        }
-        if (l + 1 < last) coarse_restrict<true, true>(Ls[l], Ls[l + 1], t0, nt);
-        else coarse_restrict<true, false>(Ls[l], Ls[l + 1], t0, nt);
-        __syncthreads();
+        cta_sweeps<U>(m, l, 1, 2 * m.nu_c - 1);
+        if (l + 1 < last) cta_restrict<true>(m, l);
+        else cta_restrict<false>(m, l);
     }
     // coarsest: zero-mean right-hand side, (R B)^k R from zero, zero-mean result
     {
-        const MgLevel &L = Ls[last];
-        const float mean = coarse_mean(L, L.f, sh, bc);
+        const CtaLev L = cta_level(m, last);
+        const float mean = cta_mean(m, last, false, sh, bc);
         for (int i = t0; i < L.N; i += nt) {
-            const float w = L.sig[i].w;
-            const float f = w != 0.f ? L.f[i] - mean : 0.f;
-            L.f[i] = f;
-            L.e[i] = f * w;  // colour 0 from zero; colour 1 is overwritten first
+            const int q = cta_at(L, i);
+            const float w = L.w[q];
+            const float f = w != 0.f ? L.f[q] - mean : 0.f;
+            L.f[q] = f;
+            L.e[q] = f * w;  // colour 0 from zero; colour 1 is overwritten first
         }
         __syncthreads();
-        for (int s = 1; s < 2 * m.coarse_sweeps + 1; s++) {
-            coarse_half<true, false>(L, L, s & 1, t0, nt);
-            __syncthreads();
+        cta_sweeps<U>(m, last, 1, 2 * m.coarse_sweeps);
+        const float emean = cta_mean(m, last, true, sh, bc);
+        for (int i = t0; i < L.N; i += nt) {
+            const int q = cta_at(L, i);
+            if (L.w[q] != 0.f) L.e[q] -= emean;
         }
-        const float emean = coarse_mean(L, L.e, sh, bc);
-        for (int i = t0; i < L.N; i += nt)
-            if (L.sig[i].w != 0.f) L.e[i] -= emean;
         __syncthreads();
     }
     for (int l = last - 1; l >= k0; l--) {
-        coarse_half<true, true>(Ls[l], Ls[l + 1], 1, t0, nt);
-        __syncthreads();
-        for (int s = 1; s < 2 * m.nu_c; s++) {
-            coarse_half<true, false>(Ls[l], Ls[l], (s & 1) ^ 1, t0, nt);
-            __syncthreads();
-        }
+        cta_prolong(m, l, 1);
+        cta_sweeps<U>(m, l, 0, 2 * m.nu_c - 1);
     }
-    for (int i = t0; i < Ls[k0].N; i += nt) __stcg(m.lev[k0].e + i, Ls[k0].e[i]);
+    const CtaLev L = cta_level(m, k0);
+    for (int i = t0; i < L.N; i += nt) __stcg(m.lev[k0].e + i, L.e[cta_at(L, i)]);
 }
 
 // Exact coarsest-level solve e = A^+ f with the host-computed pseudo-inverse
@@ -888,8 +1100,20 @@ static __device__ void mg_dense_solve(const MgArgs &m, int t0, int nt)
     const int n = L.N, lane = threadIdx.x & 31;
     for (int I = t0 >> 5; I < n; I += nt >> 5) {
         const float *row = m.dense + (size_t)I * n;
+        // sixteen products' loads in flight at a time, added in order (a round
+        // trip per product made this phase 3 us for 1024 cells)
         float acc = 0.f;
-        for (int J = lane; J < n; J += 32) acc += __ldg(row + J) * mg_ldl(L.f + J);
+        for (int J0 = lane; J0 < n; J0 += 16 * 32) {
+            float a[16], b[16];
+#pragma unroll
+            for (int u = 0; u < 16; u++) {
+                const int J = J0 + 32 * u;
+                a[u] = J < n ? __ldg(row + J) : 0.f;
+                b[u] = J < n ? mg_ldl(L.f + J) : 0.f;
+            }
+#pragma unroll
+            for (int u = 0; u < 16; u++) acc += a[u] * b[u];
+        }
 #pragma unroll
         for (int o = 16; o > 0; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
         if (lane == 0) __stcg(L.e + I, acc);
@@ -902,7 +1126,7 @@ static __device__ void mg_dense_solve(const MgArgs &m, int t0, int nt)
 // block 0's, its pre-smoothing started); leaves level from's correction in
 // lev[from].e for the prolongating half sweep of the level above.  False on
 // a barrier abort.
-template <bool TILES>
+template <bool TILES, int U>
 __device__ bool mg_coarse_cycle(const MgArgs &m, const MgGrid &G, unsigned &bar_k, int *status, float *sm,
                                 double *sh, double *bc, int from = 1)
 {
@@ -919,15 +1143,15 @@ __device__ bool mg_coarse_cycle(const MgArgs &m, const MgGrid &G, unsigned &bar_
             continue;
         }
         for (int s = 1; s < 2 * m.nu_c; s++) {
-            coarse_half<false, false>(m.lev[l], m.lev[l], s & 1, t0, nt);
+            coarse_half<false>(m.lev[l], m.lev[l], s & 1, t0, nt);
             MG_BAR();
         }
-        if (l + 1 < m.cta_from) coarse_restrict<false, true>(m.lev[l], m.lev[l + 1], t0, nt);
-        else coarse_restrict<false, false>(m.lev[l], m.lev[l + 1], t0, nt);
+        if (l + 1 < m.cta_from) coarse_restrict<true>(m.lev[l], m.lev[l + 1], t0, nt);
+        else coarse_restrict<false>(m.lev[l], m.lev[l + 1], t0, nt);
         MG_BAR();
     }
     if (m.dense) mg_dense_solve(m, t0, nt);
-    else if (G.blk == 0) mg_cta_cycle(m, sm, sh, bc);
+    else if (G.blk == 0) mg_cta_cycle<U>(m, sh, bc);
     MG_BAR();
     for (int l = m.cta_from - 1; l >= from; l--) {
         if (TILES && l >= m.tile_from) {
@@ -935,10 +1159,10 @@ __device__ bool mg_coarse_cycle(const MgArgs &m, const MgGrid &G, unsigned &bar_
             MG_BAR();
             continue;
         }
-        coarse_half<false, true>(m.lev[l], m.lev[l + 1], 1, t0, nt);
+        coarse_half<true>(m.lev[l], m.lev[l + 1], 1, t0, nt);
         MG_BAR();
         for (int s = 1; s < 2 * m.nu_c; s++) {
-            coarse_half<false, false>(m.lev[l], m.lev[l], (s & 1) ^ 1, t0, nt);
+            coarse_half<false>(m.lev[l], m.lev[l], (s & 1) ^ 1, t0, nt);
             MG_BAR();
         }
     }
@@ -968,7 +1192,7 @@ __device__ bool mg_vcycle(const StepArgs<S, R, PhiT> &a, const MgArgs &m, const 
     if (m.cta_from > 1) fine_restrict_warp<true>(g, a.mask, m.r, m.z, m.lev[1], t0, nt);
     else fine_restrict_warp<false>(g, a.mask, m.r, m.z, m.lev[1], t0, nt);
     MG_BAR();
-    if (!mg_coarse_cycle<TILES>(m, G, bar_k, a.status, sm, sh, bc)) return false;
+    if (!mg_coarse_cycle<TILES, CTA_U_WIDE>(m, G, bar_k, a.status, sm, sh, bc)) return false;
     fine_half<false, true>(g, a.mask, m.r, m.z, m.lev[1], 1, t0, nt, dummy);
     MG_BAR();
     float rz = 0.f;
@@ -986,13 +1210,13 @@ __device__ bool mg_vcycle(const StepArgs<S, R, PhiT> &a, const MgArgs &m, const 
     return true;
 }
 
-// true residual r = b - A phi (exact in the potential type), as FP32, with
-// the first pre-smoothing half sweep (colour-0 z = r / deg); returns this
+// true residual r = b - A phi (exact in the potential type), as FP32, and
+// (START) the first pre-smoothing half sweep (colour-0 z = r / deg); returns this
 // block's sum of r^2 (thread 0).  A thread takes MG_RES_U nodes per trip (one
 // per grid stride) with all their loads issued first; its nodes are still
 // summed in increasing order.
 constexpr int MG_RES_U = 2;
-template <typename PhiT, typename L>
+template <typename PhiT, bool START = true, typename L>
 __device__ double mg_true_residual(const Grid3 &g, const L *__restrict__ link, const PhiT *phi,
                                    const PhiT *b, float *r, float *z, int t0, int nt, double *sh)
 {
@@ -1032,7 +1256,7 @@ __device__ double mg_true_residual(const Grid3 &g, const L *__restrict__ link, c
                 acc -= (PhiT)__popc(o) * phii[k];
                 if constexpr (((PhiT)0.5) != 0) rv = (float)acc;
                 else rv = ll_to_float(acc) * (float)PHI_INV;
-                if (!(xyz[k] & 1)) __stcg(z + i, rv * mg_inv_deg(__popc(o)));
+                if (START && !(xyz[k] & 1)) __stcg(z + i, rv * mg_inv_deg(__popc(o)));
             }
             __stcg(r + i, rv);
             rr += rv * rv;
@@ -1180,9 +1404,9 @@ __device__ float mg_pq_pass_lean(const Grid3 &g, const L *__restrict__ link, con
     return pq;
 }
 
-// phi += alpha p, r -= alpha q and colour-0 z = r / deg on the fluid nodes
-// with an open face; returns sum r^2
-template <typename PhiT, typename L>
+// phi += alpha p, r -= alpha q and (START) colour-0 z = r / deg on the fluid
+// nodes with an open face; returns sum r^2
+template <typename PhiT, bool START = true, typename L>
 __device__ float mg_update_pass(const Grid3 &g, const L *__restrict__ link, PhiT *phi, const float *p,
                                 const float *q, float *r, float *z, double alpha, int t0, int nt)
 {
@@ -1221,7 +1445,7 @@ __device__ float mg_update_pass(const Grid3 &g, const L *__restrict__ link, PhiT
             const float rn = rv[k] - af * qv[k];
             __stcg(r + i, rn);
             rr += rn * rn;
-            if (!((x0 + k + y + zz) & 1)) __stcg(z + i, rn * mg_inv_deg(__popc(o)));
+            if (START && !((x0 + k + y + zz) & 1)) __stcg(z + i, rn * mg_inv_deg(__popc(o)));
         }
     }
     return rr;
@@ -1299,7 +1523,7 @@ __device__ void mg_solve(const StepArgs<S, R, PhiT> &a, const MgArgs &m, const M
         out = sum_partials(p, nblk, bc);
         return true;
     };
-    if (G.blk == 0 && !m.dense) mg_cta_load(m, mg_sm);
+    if (G.blk == 0 && !m.dense) mg_cta_load(m);
     double bb;
     if (!reduce(mg_start_pass(a, m, a.mask, tid, nthr, sh, bc), bb)) return;
     if (a.fixed_iter <= 0 && bb == 0.0) {

@@ -21,6 +21,7 @@
 // control kernels write it and set the loop's condition.
 #pragma once
 #include "ekl_mg.cuh"
+#include "ekl_mgf.cuh"
 
 namespace ekl {
 
@@ -61,7 +62,7 @@ __global__ void __launch_bounds__(MGS_THREADS, 1) mgs_start_kernel(StepArgs<S, R
 
 // True residual with its block partials of r^2.  when: 0 always, 1 when the
 // control state asks for one, 2 when phi moved since the last one.
-template <typename PhiT>
+template <typename PhiT, bool START = true>
 __global__ void __launch_bounds__(MGS_THREADS, 1)
     mgs_residual_kernel(Grid3 g, MgArgs m, const PhiT *phi, const PhiT *b, const MgCtl *ctl, int when)
 {
@@ -70,7 +71,7 @@ __global__ void __launch_bounds__(MGS_THREADS, 1)
     if (when == 1 && !ctl->need_true) return;
     if (when == 2 && (ctl->current || ctl->skip)) return;
     const int tid = blockIdx.x * blockDim.x + threadIdx.x, nthr = gridDim.x * blockDim.x;
-    const double t = mg_true_residual<PhiT>(g, m.link, phi, b, m.r, m.z, tid, nthr, sh);
+    const double t = mg_true_residual<PhiT, START>(g, m.link, phi, b, m.r, m.z, tid, nthr, sh);
     if (threadIdx.x == 0) mgs_slot(m, MGS_RES, gridDim.x)[blockIdx.x] = t;
 }
 
@@ -114,10 +115,8 @@ static __global__ void mgs_init_kernel(MgArgs m, MgCtl *ctl, int nblk, cudaGraph
 static __global__ void mgs_mid_kernel(MgArgs m, MgCtl *ctl, int nblk)
 {
     mgs_wait_previous();
-    __shared__ double bc[1];
-    const double rz = sum_partials(mgs_slot(m, MGS_RZ, nblk), nblk, bc);
-    const double pq = sum_partials(mgs_slot(m, MGS_PQ, nblk), nblk, bc);
-    const double rr = sum_partials(mgs_slot(m, MGS_RR, nblk), nblk, bc);
+    double rz, pq, rr;
+    sum_partials3(mgs_slot(m, MGS_RZ, nblk), mgs_slot(m, MGS_PQ, nblk), mgs_slot(m, MGS_RR, nblk), nblk, rz, pq, rr);
     if (threadIdx.x != 0) return;
     MgCtl c = *ctl;
     c.need_true = 0;
@@ -196,6 +195,17 @@ __global__ void __launch_bounds__(MGS_THREADS, 1) mgs_half_kernel(Grid3 g, MgArg
     }
 }
 
+// partials of r.z after the fused smoothing (ekl_mgf.cuh)
+template <int UNUSED> __global__ void __launch_bounds__(MGS_THREADS, 1) mgs_dot_kernel(Grid3 g, MgArgs m)
+{
+    mgs_wait_previous();
+    __shared__ double sh[MGS_THREADS / 32];
+    const float rz = mgf_dot(g, m.link, m.r, m.z, (int)(blockIdx.x * blockDim.x + threadIdx.x),
+                             (int)(gridDim.x * blockDim.x));
+    const double t = block_sum_lanes0(warp_sum_ff_lane0(rz), sh);
+    if (threadIdx.x == 0) mgs_slot(m, MGS_RZ, gridDim.x)[blockIdx.x] = t;
+}
+
 template <bool FIRST> __global__ void __launch_bounds__(MGS_THREADS, 1) mgs_restrict_kernel(Grid3 g, MgArgs m)
 {
     mgs_wait_previous();
@@ -208,20 +218,22 @@ template <bool FIRST> __global__ void __launch_bounds__(MGS_THREADS, 1) mgs_rest
 template <bool PRO> __global__ void __launch_bounds__(MGS_THREADS, 1) mgs_chalf_kernel(MgArgs m, int c)
 {
     mgs_wait_previous();
-    coarse_half<false, PRO, MGS_CU>(m.lev[1], m.lev[2], c, (int)(blockIdx.x * blockDim.x + threadIdx.x),
+    coarse_half<PRO, MGS_CU>(m.lev[1], m.lev[2], c, (int)(blockIdx.x * blockDim.x + threadIdx.x),
                             (int)(gridDim.x * blockDim.x));
 }
 // ... and its restriction to level 2 (FIRST: level 2 is grid-wide or tiled)
 template <bool FIRST> __global__ void __launch_bounds__(MGS_THREADS, 1) mgs_crestrict_kernel(MgArgs m)
 {
     mgs_wait_previous();
-    coarse_restrict<false, FIRST>(m.lev[1], m.lev[2], (int)(blockIdx.x * blockDim.x + threadIdx.x),
+    coarse_restrict<FIRST>(m.lev[1], m.lev[2], (int)(blockIdx.x * blockDim.x + threadIdx.x),
                                   (int)(gridDim.x * blockDim.x));
 }
 
 // The coarse levels of one V-cycle from level `from` (cooperative launch;
 // `bar` zeroed before it)
-static __global__ void __launch_bounds__(MGS_THREADS, 1) mgs_coarse_kernel(MgArgs m, unsigned *bar, int *status,
+// T: its block size, MG_THREADS or MG_WIDE_THREADS (the smaller one leaves 128
+// registers a thread)
+template <int T> static __global__ void __launch_bounds__(T, 1) mgs_coarse_kernel(MgArgs m, unsigned *bar, int *status,
                                                                           int from)
 {
     mgs_wait_previous();
@@ -230,9 +242,9 @@ static __global__ void __launch_bounds__(MGS_THREADS, 1) mgs_coarse_kernel(MgArg
     extern __shared__ float mg_sm[];
     const MgGrid G{(int)(blockIdx.x * blockDim.x + threadIdx.x), (int)(gridDim.x * blockDim.x), (int)gridDim.x,
                    (int)blockIdx.x, bar};
-    if (G.blk == 0 && !m.dense) mg_cta_load(m, mg_sm);
+    if (G.blk == 0 && !m.dense) mg_cta_load(m);
     unsigned bar_k = 0;
-    mg_coarse_cycle<true>(m, G, bar_k, status, mg_sm, sh, bc, from);
+    mg_coarse_cycle<true, T <= MG_THREADS ? CTA_U : CTA_U_WIDE>(m, G, bar_k, status, mg_sm, sh, bc, from);
 }
 
 // p = z + beta p_old, q = A p with the block partials of p.q
@@ -257,7 +269,7 @@ static __global__ void __launch_bounds__(MGS_THREADS, 1) mgs_pq_kernel(Grid3 g, 
 
 // phi += alpha p, r -= alpha q (and the next V-cycle's first half sweep)
 // with the block partials of r^2
-template <typename PhiT>
+template <typename PhiT, bool START = true>
 __global__ void __launch_bounds__(MGS_THREADS, 1) mgs_update_kernel(Grid3 g, MgArgs m, PhiT *phi, const MgCtl *ctl)
 {
     mgs_wait_previous();
@@ -269,7 +281,7 @@ __global__ void __launch_bounds__(MGS_THREADS, 1) mgs_update_kernel(Grid3 g, MgA
     if (!(rz > 0.0) || !(pq > 0.0)) return;
     const int tid = blockIdx.x * blockDim.x + threadIdx.x, nthr = gridDim.x * blockDim.x;
     const double alpha = rz / pq;
-    const float t = mg_update_pass<PhiT>(g, m.link, phi, m.p[ctl->pi ^ 1], m.q, m.r, m.z, alpha, tid, nthr);
+    const float t = mg_update_pass<PhiT, START>(g, m.link, phi, m.p[ctl->pi ^ 1], m.q, m.r, m.z, alpha, tid, nthr);
     const double rr = block_sum_lanes0(warp_sum_ff_lane0(t), sh);
     if (threadIdx.x == 0) mgs_slot(m, MGS_RR, nblk)[blockIdx.x] = rr;
 }
@@ -472,9 +484,9 @@ __global__ void __launch_bounds__(MGS_THREADS, 1)
     mgsb_copy(B.mg + x.r, s_m);
     const MgArgs &m = s_m;
     const MgGrid G{x.t0, x.nt, x.nb, x.lb, bars + 4 * x.r};
-    if (G.blk == 0 && !m.dense) mg_cta_load(m, mg_sm);
+    if (G.blk == 0 && !m.dense) mg_cta_load(m);
     unsigned bar_k = 0;
-    mg_coarse_cycle<false>(m, G, bar_k, reps[x.r].status, mg_sm, sh, bc, 1);
+    mg_coarse_cycle<false, CTA_U_WIDE>(m, G, bar_k, reps[x.r].status, mg_sm, sh, bc, 1);
 }
 
 __global__ static void __launch_bounds__(MGS_THREADS, 1) mgsb_pq_kernel(MgsBatch B)
@@ -524,13 +536,11 @@ __global__ void __launch_bounds__(MGS_THREADS, 1) mgsb_update_kernel(const StepA
 __global__ static void mgsb_mid_kernel(MgsBatch B)
 {
     mgs_wait_previous();
-    __shared__ double bc[1];
     const int r = blockIdx.x, nb = B.pb.rep_blocks[r];
     if (B.ctl[r].done) return;
     const MgArgs &m = B.mg[r];
-    const double rz = sum_partials(mgsb_slot(B, r, MGS_RZ), nb, bc);
-    const double pq = sum_partials(mgsb_slot(B, r, MGS_PQ), nb, bc);
-    const double rr = sum_partials(mgsb_slot(B, r, MGS_RR), nb, bc);
+    double rz, pq, rr;
+    sum_partials3(mgsb_slot(B, r, MGS_RZ), mgsb_slot(B, r, MGS_PQ), mgsb_slot(B, r, MGS_RR), nb, rz, pq, rr);
     if (threadIdx.x != 0) return;
     MgCtl c = B.ctl[r];
     c.need_true = 0;

@@ -4,6 +4,7 @@
 #include <cooperative_groups.h>
 
 #include <algorithm>
+#include <type_traits>
 #include <vector>
 
 #include "ekl_kernels.cuh"
@@ -42,7 +43,11 @@ static StepArgs<S, R, PhiT> make_args(Ctx &c, int parity = -1)
     a.patch_node = c.patch_node;
     a.patch_q = (const R *)c.patch_q;
     a.patch_f = (const R *)c.patch_f;
-    a.part_charge = c.part_charge;
+    // a single handle's fixed-point step takes its exact total from the charge
+    // pass (the FP64 partials then serve a learned warm start only)
+    const bool slots = parity < 0 && !(((PhiT)0.5) != 0);
+    a.charge_slots = slots ? c.charge_slots : nullptr;
+    a.part_charge = slots && !c.net ? nullptr : c.part_charge;
     a.part_charge_q = c.part_charge_q;
     a.charge_tot = c.charge_tot;
     a.charge_tot_q = c.charge_tot_q;
@@ -154,6 +159,7 @@ static inline MgArgs make_mg_args(const Ctx &c)
     m.nu = MG_NU;
     m.nu_c = MG_NU_COARSE;
     m.coarse_sweeps = MG_COARSE_SWEEPS;
+    m.cta_pad = c.mg_cta_pad;
     m.inner_red = MG_INNER_RED;
     m.tile_from = c.mg_tile_from;
     m.tile_off = (int)c.mg_tile_off;
@@ -182,11 +188,14 @@ template <typename PhiT> static cudaError_t mgs_build(Ctx &c, const MgArgs &m0, 
     const PhiT *phi = (const PhiT *)c.phi, *b = (const PhiT *)c.b;
     PhiT *phiw = (PhiT *)c.phi;
     int when0 = 0, when2 = 2, nblk = nb;
-    cudaGraph_t G = nullptr;
+    cudaGraph_t gr = nullptr;
     cudaStream_t cs = nullptr;
     cudaGraphConditionalHandle loop;
     cudaGraphNode_t nres0, ninit, nloop, nres2, nrep;
-    cudaError_t e = cudaGraphCreate(&G, 0);
+    MgfGeom G;
+    int V = 0;
+    if (c.mg_fused && !mgf_pick(G, V, c.nx, c.ny, c.nz, c.per, c.num_sms)) return cudaErrorInvalidValue;
+    cudaError_t e = cudaGraphCreate(&gr, 0);
     auto kernel_node = [&](cudaGraphNode_t *out, cudaGraphNode_t *dep, const void *fn, int grid, int block,
                            void **args) {
         cudaKernelNodeParams kp = {};
@@ -194,12 +203,13 @@ template <typename PhiT> static cudaError_t mgs_build(Ctx &c, const MgArgs &m0, 
         kp.gridDim = dim3(grid);
         kp.blockDim = dim3(block);
         kp.kernelParams = args;
-        return cudaGraphAddKernelNode(out, G, dep, dep ? 1 : 0, &kp);
+        return cudaGraphAddKernelNode(out, gr, dep, dep ? 1 : 0, &kp);
     };
-    if (e == cudaSuccess) e = cudaGraphConditionalHandleCreate(&loop, G, 0, cudaGraphCondAssignDefault);
+    if (e == cudaSuccess) e = cudaGraphConditionalHandleCreate(&loop, gr, 0, cudaGraphCondAssignDefault);
     if (e == cudaSuccess) {
         void *args[] = {&g, &m, &phi, &b, &ctl, &when0};
-        e = kernel_node(&nres0, nullptr, (const void *)mgs_residual_kernel<PhiT>, nb, nt, args);
+        const void *fn = c.mg_fused ? (const void *)mgs_residual_kernel<PhiT, false> : (const void *)mgs_residual_kernel<PhiT>;
+        e = kernel_node(&nres0, nullptr, fn, nb, nt, args);
     }
     if (e == cudaSuccess) {
         void *args[] = {&m, &ctl, &nblk, &loop, &c.pois_iters, &c.pois_res};
@@ -212,11 +222,12 @@ template <typename PhiT> static cudaError_t mgs_build(Ctx &c, const MgArgs &m0, 
         cp.conditional.handle = loop;
         cp.conditional.type = cudaGraphCondTypeWhile;
         cp.conditional.size = 1;
-        e = cudaGraphAddNode(&nloop, G, &ninit, nullptr, 1, &cp);
+        e = cudaGraphAddNode(&nloop, gr, &ninit, nullptr, 1, &cp);
         if (e == cudaSuccess) body = cp.conditional.phGraph_out[0];
     }
     if (e == cudaSuccess && c.mg_smem > 48 * 1024)
-        e = cudaFuncSetAttribute(mgs_coarse_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)c.mg_smem);
+        e = cudaFuncSetAttribute(c.mg_wide ? mgs_coarse_kernel<MG_WIDE_THREADS> : mgs_coarse_kernel<MG_THREADS>,
+                                 cudaFuncAttributeMaxDynamicSharedMemorySize, (int)c.mg_smem);
     if (e == cudaSuccess) e = cudaStreamCreateWithFlags(&cs, cudaStreamNonBlocking);
     if (e == cudaSuccess) e = cudaStreamBeginCaptureToGraph(cs, body, nullptr, nullptr, 0, cudaStreamCaptureModeRelaxed);
     if (e == cudaSuccess) {
@@ -238,9 +249,40 @@ template <typename PhiT> static cudaError_t mgs_build(Ctx &c, const MgArgs &m0, 
             const cudaError_t r = cudaLaunchKernelEx(&lc, kern, args...);
             if (el == cudaSuccess) el = r;
         };
-        for (int s = 1; s < 2 * MG_NU; s++) go(s > 1, nb, nt, mgs_half_kernel<false, false>, g, m, s & 1);
-        if (m.cta_from > 1) go(true, nb, nt, mgs_restrict_kernel<true>, g, m);
-        else go(true, nb, nt, mgs_restrict_kernel<false>, g, m);
+        // two half sweeps per launch: the colour-0 values between launches in
+        // the two halves of q, which the V-cycle does not use
+        auto fused = [&](bool overlap, auto mode) {
+            constexpr int MODE = decltype(mode)::value;
+            float *ca = m.q, *cb = m.q + c.N / 2;
+            MgfArgs A{m.r, m.link, MODE == MGF_POST ? cb : ca, MODE == MGF_PRE ? ca : cb, m.z, m.lev[1].e,
+                      m.lev[1].f, m.lev[1].e, m.lev[1].sig, m.lev[1].nx, m.lev[1].ny, m.lev[1].nz};
+            auto launch = [&](auto kern) {
+                const size_t smem = mgf_smem<MODE>(G, V);
+                cudaError_t r = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+                cudaLaunchConfig_t lc = {};
+                lc.gridDim = dim3(G.ntx * G.nty * G.ntz);
+                lc.blockDim = dim3(mgf_threads(G));
+                lc.dynamicSmemBytes = smem;
+                lc.stream = cs;
+                lc.attrs = dep;
+                lc.numAttrs = (overlap && pdl) ? 1 : 0;
+                if (r == cudaSuccess) r = cudaLaunchKernelEx(&lc, kern, G, A);
+                if (el == cudaSuccess) el = r;
+            };
+            const bool first = MODE == MGF_RESTR && m.cta_from > 1;
+            if (V == 4 && first) launch(mgf_kernel<MODE, 4, MODE == MGF_RESTR>);
+            else if (V == 4) launch(mgf_kernel<MODE, 4, false>);
+            else if (first) launch(mgf_kernel<MODE, 2, MODE == MGF_RESTR>);
+            else launch(mgf_kernel<MODE, 2, false>);
+        };
+        if (c.mg_fused) {
+            fused(false, std::integral_constant<int, MGF_PRE>());
+            fused(true, std::integral_constant<int, MGF_RESTR>());
+        } else {
+            for (int s = 1; s < 2 * MG_NU; s++) go(s > 1, nb, nt, mgs_half_kernel<false, false>, g, m, s & 1);
+            if (m.cta_from > 1) go(true, nb, nt, mgs_restrict_kernel<true>, g, m);
+            else go(true, nb, nt, mgs_restrict_kernel<false>, g, m);
+        }
         // level 1 smoothed and restricted by separate launches when grid-wide
         const int from = c.mgs_l1 ? 2 : 1;
         if (c.mgs_l1) {
@@ -259,22 +301,30 @@ template <typename PhiT> static cudaError_t mgs_build(Ctx &c, const MgArgs &m0, 
         cfg.stream = cs;
         cfg.attrs = coop;
         cfg.numAttrs = 1;
-        const cudaError_t ecoop = cudaLaunchKernelEx(&cfg, mgs_coarse_kernel, m, c.barrier, c.status, from);
+        const cudaError_t ecoop = cudaLaunchKernelEx(&cfg, c.mg_wide ? mgs_coarse_kernel<MG_WIDE_THREADS> : mgs_coarse_kernel<MG_THREADS>, m, c.barrier, c.status, from);
         if (el == cudaSuccess) el = ecoop;
         if (c.mgs_l1) {
             go(false, nb, nt, mgs_chalf_kernel<true>, m, 1);
             for (int s = 1; s < 2 * MG_NU_COARSE; s++) go(true, nb, nt, mgs_chalf_kernel<false>, m, (s & 1) ^ 1);
         }
-        go(c.mgs_l1 != 0, nb, nt, mgs_half_kernel<false, true>, g, m, 1);
-        for (int s = 1; s < 2 * MG_NU; s++) {
-            const int col = (s & 1) ^ 1;
-            if (s == 2 * MG_NU - 1) go(true, nb, nt, mgs_half_kernel<true, false>, g, m, col);
-            else go(true, nb, nt, mgs_half_kernel<false, false>, g, m, col);
+        if (c.mg_fused) {
+            fused(c.mgs_l1 != 0, std::integral_constant<int, MGF_PRO>());
+            fused(true, std::integral_constant<int, MGF_POST>());
+            go(true, nb, nt, mgs_dot_kernel<0>, g, m);
+        } else {
+            go(c.mgs_l1 != 0, nb, nt, mgs_half_kernel<false, true>, g, m, 1);
+            for (int s = 1; s < 2 * MG_NU; s++) {
+                const int col = (s & 1) ^ 1;
+                if (s == 2 * MG_NU - 1) go(true, nb, nt, mgs_half_kernel<true, false>, g, m, col);
+                else go(true, nb, nt, mgs_half_kernel<false, false>, g, m, col);
+            }
         }
         go(true, nb, nt, mgs_pq_kernel, g, m, (const MgCtl *)ctl);
-        go(true, nb, nt, mgs_update_kernel<PhiT>, g, m, phiw, (const MgCtl *)ctl);
+        if (c.mg_fused) go(true, nb, nt, mgs_update_kernel<PhiT, false>, g, m, phiw, (const MgCtl *)ctl);
+        else go(true, nb, nt, mgs_update_kernel<PhiT>, g, m, phiw, (const MgCtl *)ctl);
         go(true, 1, 32, mgs_mid_kernel, m, ctl, nb);
-        go(true, nb, nt, mgs_residual_kernel<PhiT>, g, m, phi, b, (const MgCtl *)ctl, 1);
+        if (c.mg_fused) go(true, nb, nt, mgs_residual_kernel<PhiT, false>, g, m, phi, b, (const MgCtl *)ctl, 1);
+        else go(true, nb, nt, mgs_residual_kernel<PhiT>, g, m, phi, b, (const MgCtl *)ctl, 1);
         go(true, 1, 32, mgs_end_kernel, m, ctl, nb, loop, (const int *)c.status);
         cudaError_t ek = cudaGetLastError();
         cudaError_t ec = cudaStreamEndCapture(cs, &body);
@@ -289,13 +339,13 @@ template <typename PhiT> static cudaError_t mgs_build(Ctx &c, const MgArgs &m0, 
         void *args[] = {&m, &ctl, &nblk, &c.pois_iters, &c.pois_total, &c.pois_res, &c.status};
         e = kernel_node(&nrep, &nres2, (const void *)mgs_report_kernel, 1, 32, args);
     }
-    if (e == cudaSuccess) e = cudaGraphInstantiate(&c.mgs_exec, G, 0);
+    if (e == cudaSuccess) e = cudaGraphInstantiate(&c.mgs_exec, gr, 0);
     if (e != cudaSuccess) {
-        if (G) cudaGraphDestroy(G);
+        if (gr) cudaGraphDestroy(gr);
         c.mgs_exec = nullptr;
         return e;
     }
-    c.mgs_graph = G;
+    c.mgs_graph = gr;
     return cudaSuccess;
 }
 
@@ -348,10 +398,13 @@ template <typename S, typename R, typename PhiT, bool DEV> int steps_impl(Ctx &c
         phase_end(c, PH_BIN);
         // 2. charge density from the streamed ion densities
         phase_begin(c, PH_CHARGE);
+        cudaMemsetAsync(c.barrier, 0, 4 * sizeof(unsigned) + CHARGE_SLOTS * sizeof(unsigned long long), c.stream);
         charge_kernel<S, R, PhiT, DEV><<<c.charge_blocks, CHARGE_THREADS, 0, c.stream>>>(a);
-        charge_total_kernel<!(((PhiT)0.5) != 0)>
-            <<<CHARGE_TOTAL_BLOCKS, 1024, 0, c.stream>>>(charge_totals_args(c));
-        c.launches += 2;
+        c.launches++;
+        if (!a.charge_slots) {
+            charge_total_kernel<false><<<CHARGE_TOTAL_BLOCKS, 1024, 0, c.stream>>>(charge_totals_args(c));
+            c.launches++;
+        }
         phase_end(c, PH_CHARGE);
         // 3. Poisson: one cooperative launch for all sweeps (after the learned
         //    warm start, when one is installed)
@@ -362,7 +415,6 @@ template <typename S, typename R, typename PhiT, bool DEV> int steps_impl(Ctx &c
             if (rc != EKL_OK) return rc;
         }
         phase_begin(c, PH_POISSON);
-        cudaMemsetAsync(c.barrier, 0, 4 * sizeof(unsigned), c.stream);
         if (c.mg && c.mg_split) {
             MgArgs m = make_mg_args(c);
             mgs_start_kernel<S, R, PhiT><<<c.pois_blocks, c.mgs_threads, 0, c.stream>>>(a, m, (MgCtl *)c.mgs_ctl);
