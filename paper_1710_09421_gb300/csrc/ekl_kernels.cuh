@@ -356,10 +356,18 @@ template <typename PhiT> struct PoisUpd;
 template <> struct PoisUpd<double> {
     typedef double acc_t;
     typedef double om_t;
-    __device__ static double resid(double acc, int deg, double pi) { return acc - deg * pi; }
+    // degrees as FP64 literals: a conversion, like a division's ten
+    // operations, goes through the FP64 pipe (16 cycles per warp instruction)
+    __device__ static double d(int deg)
+    {
+        return deg == 6 ? 6.0 : deg == 5 ? 5.0 : deg == 4 ? 4.0 : deg == 3 ? 3.0 : deg == 2 ? 2.0 : 1.0;
+    }
+    __device__ static double resid(double acc, int deg, double pi) { return acc - d(deg) * pi; }
     __device__ static double apply(double pi, double omega, double r, int deg)
     {
-        return pi + omega * r / deg;
+        const double inv = deg == 6 ? 1.0 / 6.0 : deg == 5 ? 1.0 / 5.0 : deg == 4 ? 0.25
+                         : deg == 3 ? 1.0 / 3.0 : deg == 2 ? 0.5 : 1.0;
+        return pi + quot(omega * r, d(deg), inv);
     }
     __device__ static double r2(double r) { return r * r; }
 };
@@ -657,35 +665,85 @@ __global__ void __launch_bounds__(POIS_THREADS, 1) poisson_kernel(StepArgs<S, R,
 // shared memory for the whole solve.  A sweep updates the red nodes of T and
 // of the first halo layer (the halo red values are recomputed from the same
 // inputs as their owner's, so they are bitwise the owner's), then the black
-// nodes of T, writes T to global memory and passes one grid barrier; the
-// next sweep reloads only the halo.  Results are bitwise those of the
-// global-memory kernel (same node updates, same schedule).
+// nodes of T, writes the rows that other tiles read to global memory and passes
+// one grid barrier; the next sweep reloads only the halo.  Results are bitwise
+// those of the global-memory kernel (same node updates, same schedule).
 struct TileGeom {
     int ty, tz, nty, ntz;  // tile extents and tile counts along y and z
 };
 
-template <typename PhiT>
-__device__ __forceinline__ void tile_update(PhiT *ps, const PhiT *bs, const uint32_t *ms, int nx, int ey,
-                                            int e, int x, uint32_t m, typename PoisUpd<PhiT>::om_t omega,
-                                            typename PoisUpd<PhiT>::acc_t &r2, bool count)
+// The extended tile's potential and source, split by the parity of the linear
+// index e = x + nx (ly + ey lz): nodes of one colour in a row lie in
+// consecutive words.
+struct TileFrame {
+    int nx, ey, ex, M;  // row length, rows per plane, nodes per plane, nodes per parity
+};
+__device__ __forceinline__ int tile_at(const TileFrame &t, int e) { return (e & 1) * t.M + (e >> 1); }
+// position of the node d further, relative to that of node e
+__device__ __forceinline__ int tile_step(const TileFrame &t, int d, bool odd)
 {
-    const int ex = nx * ey;  // stride of lz
-    // face neighbours in the extended frame (x wraps inside the row)
-    const int nb[6] = {x == 0 ? e + nx - 1 : e - 1, x == nx - 1 ? e - nx + 1 : e + 1, e - nx, e + nx,
-                       e - ex, e + ex};
-    PhiT acc = bs[e];
-    int deg = 0;
+    if ((d & 1) == 0) return d / 2;
+    return odd ? (d + 1) / 2 - t.M : (d - 1) / 2 + t.M;
+}
+// One update: the node's index e, its open faces (bits 16-21), whether its -x
+// or +x neighbour wraps (22, 23) and whether the tile owns it (24)
+constexpr unsigned TILE_NONE = ~0u, TILE_XLO = 1u << 22, TILE_XHI = 1u << 23, TILE_OWN = 1u << 24;
+__device__ __forceinline__ unsigned tile_item(const TileFrame &t, const uint32_t *ms, int ly, int lz, int x, bool own)
+{
+    if (x >= t.nx) return TILE_NONE;
+    const int e = x + t.nx * ly + t.ex * lz;
+    const uint32_t m = ms[e];
+    const unsigned open = ~(m >> 1) & 63u;
+    if ((m & SOLID_BIT) || open == 0) return TILE_NONE;
+    return (unsigned)e | open << 16 | (x == 0 ? TILE_XLO : 0u) | (x == t.nx - 1 ? TILE_XHI : 0u) | (own ? TILE_OWN : 0u);
+}
+// the updated value of an item, to be stored at position p (-1: nowhere)
+template <typename PhiT>
+__device__ __forceinline__ PhiT tile_relax(const TileFrame &t, const PhiT *ps, const PhiT *bs, unsigned q,
+                                           typename PoisUpd<PhiT>::om_t omega, bool need,
+                                           typename PoisUpd<PhiT>::acc_t &r2, int &p)
+{
+    p = -1;
+    if (q == TILE_NONE) return (PhiT)0;
+    const int e = q & 0xFFFFu;
+    const bool odd = e & 1;
+    p = tile_at(t, e);
+    const PhiT v[6] = {ps[p + ((q & TILE_XLO) ? tile_step(t, t.nx - 1, odd) : tile_step(t, -1, odd))],
+                       ps[p + ((q & TILE_XHI) ? tile_step(t, 1 - t.nx, odd) : tile_step(t, 1, odd))],
+                       ps[p + tile_step(t, -t.nx, odd)],
+                       ps[p + tile_step(t, t.nx, odd)],
+                       ps[p + tile_step(t, -t.ex, odd)],
+                       ps[p + tile_step(t, t.ex, odd)]};
+    PhiT acc = bs[p];
+    const PhiT pi = ps[p];
 #pragma unroll
     for (int f = 0; f < 6; f++)
-        if (!((m >> (f + 1)) & 1u)) {
-            acc += ps[nb[f]];
-            deg++;
-        }
-    if (deg == 0) return;
-    const PhiT pi = ps[e];
+        if ((q >> (16 + f)) & 1u) acc += v[f];
+    const int deg = __popc(q & (63u << 16));
     const PhiT r = PoisUpd<PhiT>::resid(acc, deg, pi);
-    ps[e] = PoisUpd<PhiT>::apply(pi, omega, r, deg);
-    if (count) r2 += PoisUpd<PhiT>::r2(r);
+    if (need && (q & TILE_OWN)) r2 += PoisUpd<PhiT>::r2(r);
+    return PoisUpd<PhiT>::apply(pi, omega, r, deg);
+}
+// one colour's half sweep: the items q of this thread, then those of index
+// U * blockDim.x + threadIdx.x on, formed by item(k) (all values before the first
+// store: nodes of one colour do not read one another)
+template <int U, typename PhiT, typename F>
+__device__ __forceinline__ void tile_sweep(const TileFrame &t, PhiT *ps, const PhiT *bs, const unsigned (&q)[U], int n,
+                                           F item, typename PoisUpd<PhiT>::om_t omega, bool need,
+                                           typename PoisUpd<PhiT>::acc_t &r2)
+{
+    PhiT v[U];
+    int p[U];
+#pragma unroll
+    for (int u = 0; u < U; u++) v[u] = tile_relax<PhiT>(t, ps, bs, q[u], omega, need, r2, p[u]);
+#pragma unroll
+    for (int u = 0; u < U; u++)
+        if (p[u] >= 0) ps[p[u]] = v[u];
+    for (int k = threadIdx.x + U * blockDim.x; k < n; k += blockDim.x) {
+        int i;
+        const PhiT x = tile_relax<PhiT>(t, ps, bs, item(k), omega, need, r2, i);
+        if (i >= 0) ps[i] = x;
+    }
 }
 
 template <typename S, typename R, typename PhiT>
@@ -701,9 +759,10 @@ __global__ void __launch_bounds__(POIS_THREADS, 1) poisson_tiled_kernel(StepArgs
     const int nthr = nblk * blockDim.x;
     unsigned bar_k = 0;
     const int nx = g.nx, ey = tg.ty + 4, ez = tg.tz + 4, E = nx * ey * ez;
+    const TileFrame T{nx, ey, nx * ey, (E + 1) >> 1};
     PhiT *ps = (PhiT *)tsm;
-    PhiT *bs = ps + E;
-    uint32_t *ms = (uint32_t *)(bs + E);
+    PhiT *bs = ps + 2 * T.M;
+    uint32_t *ms = (uint32_t *)(bs + 2 * T.M);
     const int by = blockIdx.x % tg.nty, bz = blockIdx.x / tg.nty;
     const int y0 = by * tg.ty - 2, z0 = bz * tg.tz - 2;  // global coordinates of the extended origin
     // --- source (grid-wide, as in the global kernel)
@@ -744,9 +803,10 @@ __global__ void __launch_bounds__(POIS_THREADS, 1) poisson_tiled_kernel(StepArgs
         const bool in = gidx(ly, lz, gi);
         const int e0 = nx * row;
         for (int x = lane; x < nx; x += 32) {
+            const int p = tile_at(T, e0 + x);
             ms[e0 + x] = in ? a.mask[gi + x] : SOLID_BIT;
-            bs[e0 + x] = in ? __ldcg(a.b + gi + x) : (PhiT)0;
-            ps[e0 + x] = in ? __ldcg(a.phi + gi + x) : (PhiT)0;
+            bs[p] = in ? __ldcg(a.b + gi + x) : (PhiT)0;
+            ps[p] = in ? __ldcg(a.phi + gi + x) : (PhiT)0;
         }
     }
     __syncthreads();
@@ -756,64 +816,153 @@ __global__ void __launch_bounds__(POIS_THREADS, 1) poisson_tiled_kernel(StepArgs
     const typename PoisUpd<PhiT>::om_t *oms = (const typename PoisUpd<PhiT>::om_t *)a.omegas;
     const int ty = tg.ty, tz = tg.tz;
     const int hx = (nx + 1) >> 1;
+    // red nodes of T and of the first halo layer (its corner rows are nobody's
+    // neighbours), black nodes of T: pair k of x-neighbours
+    const int nred = hx * (ty * tz + 2 * (ty + tz)), nblack = hx * ty * tz;
+    auto red = [&](int k) -> unsigned {
+        if (k >= nred) return TILE_NONE;
+        int row = k / hx, ly, lz;
+        const int xh = k - row * hx;
+        if (row < ty) {
+            lz = 1;
+            ly = 2 + row;
+        } else if (row < ty + tz * (ty + 2)) {
+            row -= ty;
+            lz = 2 + row / (ty + 2);
+            ly = 1 + row % (ty + 2);
+        } else {
+            lz = tz + 2;
+            ly = 2 + row - ty - tz * (ty + 2);
+        }
+        const bool own = ly >= 2 && ly < ty + 2 && lz >= 2 && lz < tz + 2;
+        return tile_item(T, ms, ly, lz, 2 * xh + ((y0 + ly + z0 + lz) & 1), own);  // red: (x + y + z) even
+    };
+    auto black = [&](int k) -> unsigned {
+        if (k >= nblack) return TILE_NONE;
+        const int row = k / hx, xh = k - row * hx, ly = 2 + row % ty, lz = 2 + row / ty;
+        return tile_item(T, ms, ly, lz, 2 * xh + ((y0 + ly + z0 + lz + 1) & 1), true);
+    };
+    // the halo rows a sweep reads: two layers at each side of T, and the
+    // corner rows of the first
+    const int nhalo = hx * 4 * (ty + tz + 1);
+    auto halo = [&](int k, int &e, int &gi) -> bool {
+        if (k >= nhalo) return false;
+        int row = k / hx, ly, lz;
+        const int xh = k - row * hx;
+        if (row < 4 * ty) {
+            const int s = row / ty;
+            lz = s < 2 ? s : tz + s;
+            ly = 2 + row - s * ty;
+        } else if (row < 4 * (ty + tz)) {
+            row -= 4 * ty;
+            const int s = row / tz;
+            ly = s < 2 ? s : ty + s;
+            lz = 2 + row - s * tz;
+        } else {
+            row -= 4 * (ty + tz);
+            ly = (row & 1) ? ty + 2 : 1;
+            lz = (row & 2) ? tz + 2 : 1;
+        }
+        if (!gidx(ly, lz, gi)) return false;
+        gi += 2 * xh;
+        e = nx * ly + T.ex * lz + 2 * xh;
+        return true;
+    };
+    // the rows of T that are some block's halo: two at each side
+    const bool thin = ty <= 4 || tz <= 4;
+    const int nrim = hx * (thin ? ty * tz : 4 * (ty + tz) - 16);
+    auto rim = [&](int k, int &e, int &gi) -> bool {
+        if (k >= nrim) return false;
+        int row = k / hx, ly, lz;
+        const int xh = k - row * hx;
+        if (thin) {
+            lz = 2 + row / ty;
+            ly = 2 + row % ty;
+        } else if (row < 4 * ty) {
+            const int s = row / ty;
+            lz = s < 2 ? 2 + s : tz - 2 + s;
+            ly = 2 + row - s * ty;
+        } else {
+            row -= 4 * ty;
+            const int s = row / (tz - 4);
+            ly = s < 2 ? 2 + s : ty - 2 + s;
+            lz = 4 + row - s * (tz - 4);
+        }
+        gi = nx * ((y0 + ly) + g.ny * (z0 + lz)) + 2 * xh;
+        e = nx * ly + T.ex * lz + 2 * xh;
+        return true;
+    };
+    const bool even = (nx & 1) == 0;  // rows split into aligned 16-byte pairs
+    auto pair_last = [&](int e) { return !even && (e + 1) % nx == 0; };  // the pair's second node is none
+    auto publish = [&](int e, int gi) {
+        const PhiT v0 = ps[tile_at(T, e)];
+        if (even) {
+            const longlong2 w = {__builtin_bit_cast(long long, v0),
+                                 __builtin_bit_cast(long long, ps[tile_at(T, e + 1)])};
+            __stcg((longlong2 *)(a.phi + gi), w);
+        } else {
+            __stcg(a.phi + gi, v0);
+            if (!pair_last(e)) __stcg(a.phi + gi + 1, ps[tile_at(T, e + 1)]);
+        }
+    };
+    // what a thread does in every sweep, found once: positions of its first
+    // items (the remaining ones, of large tiles, are formed in every sweep)
+    constexpr int UR = 4, UB = 3, UH = 3, UP = 2;
+    unsigned qr[UR], qb[UB];
+    int he[UH], hg[UH], pe[UP], pg[UP];
+#pragma unroll
+    for (int u = 0; u < UR; u++) qr[u] = red(threadIdx.x + u * blockDim.x);
+#pragma unroll
+    for (int u = 0; u < UB; u++) qb[u] = black(threadIdx.x + u * blockDim.x);
+#pragma unroll
+    for (int u = 0; u < UH; u++)
+        if (!halo(threadIdx.x + u * blockDim.x, he[u], hg[u])) he[u] = -1;
+#pragma unroll
+    for (int u = 0; u < UP; u++)
+        if (!rim(threadIdx.x + u * blockDim.x, pe[u], pg[u])) pe[u] = -1;
     for (it = 0; it < limit; it++) {
         typename PoisUpd<PhiT>::acc_t r2 = 0;
+        // the residual norm is only needed on the sweeps that test it
+        const bool need = (a.fixed_iter <= 0 && ((it + 1) % a.check_every) == 0) || it + 1 == limit;
         if (it > 0) {
-            // reload the halo rows (rows outside the owned tile)
-            for (int row = warp; row < rows; row += nwarps) {
-                const int ly = row % ey, lz = row / ey;
-                if (ly >= 2 && ly < ty + 2 && lz >= 2 && lz < tz + 2) continue;
-                int gi;
-                if (!gidx(ly, lz, gi)) continue;
-                const int e0 = nx * row;
-                for (int x = lane; x < nx; x += 32) ps[e0 + x] = __ldcg(a.phi + gi + x);
+            // reload the halo: every load of a thread is issued before the
+            // first is used
+            longlong2 w[UH];
+#pragma unroll
+            for (int u = 0; u < UH; u++) {
+                if (he[u] < 0) continue;
+                const long long *src = (const long long *)a.phi + hg[u];
+                if (even) w[u] = __ldcg((const longlong2 *)src);
+                else w[u] = {__ldcg(src), pair_last(he[u]) ? 0ll : __ldcg(src + 1)};
+            }
+#pragma unroll
+            for (int u = 0; u < UH; u++) {
+                if (he[u] < 0) continue;
+                ps[tile_at(T, he[u])] = __builtin_bit_cast(PhiT, w[u].x);
+                if (!pair_last(he[u])) ps[tile_at(T, he[u] + 1)] = __builtin_bit_cast(PhiT, w[u].y);
+            }
+            for (int k = threadIdx.x + UH * blockDim.x; k < nhalo; k += blockDim.x) {
+                int e, gi;
+                if (!halo(k, e, gi)) continue;
+                const PhiT v0 = __ldcg(a.phi + gi);
+                if (!pair_last(e)) ps[tile_at(T, e + 1)] = __ldcg(a.phi + gi + 1);
+                ps[tile_at(T, e)] = v0;
             }
             __syncthreads();
         }
         const typename PoisUpd<PhiT>::om_t om_r = __ldg(oms + 2 * it), om_b = __ldg(oms + 2 * it + 1);
-        // red nodes of T and of the first halo layer
-        {
-            const int ny1 = ty + 2, nrow = ny1 * (tz + 2);
-            for (int rr = warp; rr < nrow; rr += nwarps) {
-                const int ly = 1 + rr % ny1, lz = 1 + rr / ny1;
-                const int par = (y0 + ly + z0 + lz) & 1;   // red: (x + y + z) even
-                const bool own = ly >= 2 && ly < ty + 2 && lz >= 2 && lz < tz + 2;
-                const int e0 = nx * (ly + ey * lz);
-                for (int xh = lane; xh < hx; xh += 32) {
-                    const int x = 2 * xh + par;
-                    if (x >= nx) continue;
-                    const uint32_t m = ms[e0 + x];
-                    if (m & SOLID_BIT) continue;
-                    tile_update<PhiT>(ps, bs, ms, nx, ey, e0 + x, x, m, om_r, r2, own);
-                }
-            }
-        }
+        tile_sweep<UR, PhiT>(T, ps, bs, qr, nred, red, om_r, need, r2);
         __syncthreads();
-        // black nodes of T
-        {
-            const int nrow = ty * tz;
-            for (int rr = warp; rr < nrow; rr += nwarps) {
-                const int ly = 2 + rr % ty, lz = 2 + rr / ty;
-                const int par = (y0 + ly + z0 + lz + 1) & 1;  // black: (x + y + z) odd
-                const int e0 = nx * (ly + ey * lz);
-                for (int xh = lane; xh < hx; xh += 32) {
-                    const int x = 2 * xh + par;
-                    if (x >= nx) continue;
-                    const uint32_t m = ms[e0 + x];
-                    if (m & SOLID_BIT) continue;
-                    tile_update<PhiT>(ps, bs, ms, nx, ey, e0 + x, x, m, om_b, r2, true);
-                }
-            }
-        }
+        tile_sweep<UB, PhiT>(T, ps, bs, qb, nblack, black, om_b, need, r2);
         __syncthreads();
-        // owned rows back to global memory
-        for (int rr = warp; rr < ty * tz; rr += nwarps) {
-            const int ly = 2 + rr % ty, lz = 2 + rr / ty;
-            const int gi = nx * ((y0 + ly) + g.ny * (z0 + lz));
-            const int e0 = nx * (ly + ey * lz);
-            for (int x = lane; x < nx; x += 32) __stcg(a.phi + gi + x, ps[e0 + x]);
+#pragma unroll
+        for (int u = 0; u < UP; u++)
+            if (pe[u] >= 0) publish(pe[u], pg[u]);
+        for (int k = threadIdx.x + UP * blockDim.x; k < nrim; k += blockDim.x) {
+            int e, gi;
+            rim(k, e, gi);
+            publish(e, gi);
         }
-        const bool need = (a.fixed_iter <= 0 && ((it + 1) % a.check_every) == 0) || it + 1 == limit;
         if (need) {
             double wsum;
             if constexpr (((PhiT)0.5) != 0) wsum = warp_sum((double)r2);
@@ -830,6 +979,11 @@ __global__ void __launch_bounds__(POIS_THREADS, 1) poisson_tiled_kernel(StepArgs
                 break;
             }
         }
+    }
+    // the whole tile to global memory (the sweeps wrote its rim)
+    for (int k = threadIdx.x; k < nblack; k += blockDim.x) {
+        const int row = k / hx, ly = 2 + row % ty, lz = 2 + row / ty, x = 2 * (k - row * hx);
+        publish(nx * ly + T.ex * lz + x, nx * ((y0 + ly) + g.ny * (z0 + lz)) + x);
     }
     if (tid == 0) {
         *a.pois_iters = it;
@@ -972,7 +1126,8 @@ __global__ void __launch_bounds__(POIS_THREADS, 1) poisson_batch_kernel(const St
 
 template <typename PhiT> inline size_t tile_smem_bytes(int nx, const TileGeom &tg)
 {
-    return (size_t)nx * (tg.ty + 4) * (tg.tz + 4) * (2 * sizeof(PhiT) + sizeof(uint32_t));
+    const size_t E = (size_t)nx * (tg.ty + 4) * (tg.tz + 4);
+    return ((E + 1) & ~(size_t)1) * 2 * sizeof(PhiT) + E * sizeof(uint32_t);
 }
 
 // ============================================================== beads
