@@ -1054,7 +1054,7 @@ static int create_handle(const ekl_params *P, void *stream, ekl_handle **out, bo
     c.charge_tot_q = (long long *)A(sizeof(long long));
     c.charge_chunks = A(CHARGE_CHUNK_BYTES);
     c.part_mass = (double *)A((size_t)((N + 255) / 256) * NS * sizeof(double));
-    c.part_pois = (double *)A((size_t)c.pois_blocks * sizeof(double));
+    c.part_pois = (double *)A(2 * (size_t)c.pois_blocks * sizeof(double));
     c.barrier = (unsigned *)A(4 * sizeof(unsigned) + CHARGE_SLOTS * sizeof(unsigned long long));
     c.charge_slots = (unsigned long long *)(c.barrier + 4);
     c.status = (int *)A(sizeof(int));

@@ -356,29 +356,41 @@ template <typename PhiT> struct PoisUpd;
 template <> struct PoisUpd<double> {
     typedef double acc_t;
     typedef double om_t;
-    // degrees as FP64 literals: a conversion, like a division's ten
-    // operations, goes through the FP64 pipe (16 cycles per warp instruction)
-    __device__ static double d(int deg)
+    // a degree and its inverse, as literals or from a table: a conversion,
+    // like a division's ten operations, goes through the FP64 pipe (16 cycles
+    // per warp instruction)
+    typedef double deg_t;
+    typedef double inv_t;
+    __device__ static deg_t d(int deg)
     {
         return deg == 6 ? 6.0 : deg == 5 ? 5.0 : deg == 4 ? 4.0 : deg == 3 ? 3.0 : deg == 2 ? 2.0 : 1.0;
     }
-    __device__ static double resid(double acc, int deg, double pi) { return acc - d(deg) * pi; }
-    __device__ static double apply(double pi, double omega, double r, int deg)
+    __device__ static inv_t inv(int deg)
     {
-        const double inv = deg == 6 ? 1.0 / 6.0 : deg == 5 ? 1.0 / 5.0 : deg == 4 ? 0.25
-                         : deg == 3 ? 1.0 / 3.0 : deg == 2 ? 0.5 : 1.0;
-        return pi + quot(omega * r, d(deg), inv);
+        return deg == 6 ? 1.0 / 6.0 : deg == 5 ? 1.0 / 5.0 : deg == 4 ? 0.25
+             : deg == 3 ? 1.0 / 3.0 : deg == 2 ? 0.5 : 1.0;
+    }
+    __device__ static double resid(double acc, deg_t deg, double pi) { return acc - deg * pi; }
+    __device__ static double apply(double pi, double omega, double r, deg_t deg, inv_t inv)
+    {
+        return pi + quot(omega * r, deg, inv);
     }
     __device__ static double r2(double r) { return r * r; }
 };
 template <> struct PoisUpd<long long> {
     typedef float acc_t;
     typedef float om_t;
-    __device__ static long long resid(long long acc, int deg, long long pi) { return acc - deg * pi; }
-    __device__ static long long apply(long long pi, float omega, long long r, int deg)
+    typedef int deg_t;
+    typedef float inv_t;
+    __device__ static deg_t d(int deg) { return deg; }
+    __device__ static inv_t inv(int deg)
     {
-        const float inv = deg == 6 ? (1.f / 6.f) : deg == 5 ? 0.2f : deg == 4 ? 0.25f
-                        : deg == 3 ? (1.f / 3.f) : deg == 2 ? 0.5f : 1.f;
+        return deg == 6 ? (1.f / 6.f) : deg == 5 ? 0.2f : deg == 4 ? 0.25f
+             : deg == 3 ? (1.f / 3.f) : deg == 2 ? 0.5f : 1.f;
+    }
+    __device__ static long long resid(long long acc, deg_t deg, long long pi) { return acc - deg * pi; }
+    __device__ static long long apply(long long pi, float omega, long long r, deg_t deg, inv_t inv)
+    {
         return pi + float_to_ll(omega * ll_to_float(r) * inv);
     }
     __device__ static float r2(long long r)
@@ -417,8 +429,9 @@ __device__ __forceinline__ void sor_apply(PhiT *phi, int i, uint32_t m, PhiT bi,
             deg++;
         }
     if (deg == 0) return;
-    PhiT r = PoisUpd<PhiT>::resid(acc, deg, pi);
-    __stcg(phi + i, PoisUpd<PhiT>::apply(pi, omega, r, deg));
+    const typename PoisUpd<PhiT>::deg_t d = PoisUpd<PhiT>::d(deg);
+    PhiT r = PoisUpd<PhiT>::resid(acc, d, pi);
+    __stcg(phi + i, PoisUpd<PhiT>::apply(pi, omega, r, d, PoisUpd<PhiT>::inv(deg)));
     r2 += PoisUpd<PhiT>::r2(r);
 }
 
@@ -677,6 +690,7 @@ struct TileGeom {
 // consecutive words.
 struct TileFrame {
     int nx, ey, ex, M;  // row length, rows per plane, nodes per plane, nodes per parity
+    bool even;          // rows of even length
 };
 __device__ __forceinline__ int tile_at(const TileFrame &t, int e) { return (e & 1) * t.M + (e >> 1); }
 // position of the node d further, relative to that of node e
@@ -697,9 +711,16 @@ __device__ __forceinline__ unsigned tile_item(const TileFrame &t, const uint32_t
     if ((m & SOLID_BIT) || open == 0) return TILE_NONE;
     return (unsigned)e | open << 16 | (x == 0 ? TILE_XLO : 0u) | (x == t.nx - 1 ? TILE_XHI : 0u) | (own ? TILE_OWN : 0u);
 }
+// degrees and their inverses by the number of open faces, in shared memory (a
+// chain of selects per update otherwise)
+template <typename PhiT> struct TileDeg {
+    typename PoisUpd<PhiT>::deg_t d[8];
+    typename PoisUpd<PhiT>::inv_t inv[8];
+};
 // the updated value of an item, to be stored at position p (-1: nowhere)
 template <typename PhiT>
-__device__ __forceinline__ PhiT tile_relax(const TileFrame &t, const PhiT *ps, const PhiT *bs, unsigned q,
+__device__ __forceinline__ PhiT tile_relax(const TileFrame &t, const TileDeg<PhiT> &dg, const PhiT *ps, const PhiT *bs,
+                                           unsigned q,
                                            typename PoisUpd<PhiT>::om_t omega, bool need,
                                            typename PoisUpd<PhiT>::acc_t &r2, int &p)
 {
@@ -708,40 +729,64 @@ __device__ __forceinline__ PhiT tile_relax(const TileFrame &t, const PhiT *ps, c
     const int e = q & 0xFFFFu;
     const bool odd = e & 1;
     p = tile_at(t, e);
-    const PhiT v[6] = {ps[p + ((q & TILE_XLO) ? tile_step(t, t.nx - 1, odd) : tile_step(t, -1, odd))],
-                       ps[p + ((q & TILE_XHI) ? tile_step(t, 1 - t.nx, odd) : tile_step(t, 1, odd))],
-                       ps[p + tile_step(t, -t.nx, odd)],
-                       ps[p + tile_step(t, t.nx, odd)],
-                       ps[p + tile_step(t, -t.ex, odd)],
-                       ps[p + tile_step(t, t.ex, odd)]};
+    int j[6];
+    if (t.even) {  // parity = colour of x: the y and z neighbours in this array, the x ones in the other
+        const int other = p + (odd ? -t.M : t.M), hx = t.nx >> 1;
+        j[0] = odd ? other : other + ((q & TILE_XLO) ? hx - 1 : -1);
+        j[1] = odd ? other + ((q & TILE_XHI) ? 1 - hx : 1) : other;
+        j[2] = p - hx;
+        j[3] = p + hx;
+        j[4] = p - (t.ex >> 1);
+        j[5] = p + (t.ex >> 1);
+    } else {
+        j[0] = p + ((q & TILE_XLO) ? tile_step(t, t.nx - 1, odd) : tile_step(t, -1, odd));
+        j[1] = p + ((q & TILE_XHI) ? tile_step(t, 1 - t.nx, odd) : tile_step(t, 1, odd));
+        j[2] = p + tile_step(t, -t.nx, odd);
+        j[3] = p + tile_step(t, t.nx, odd);
+        j[4] = p + tile_step(t, -t.ex, odd);
+        j[5] = p + tile_step(t, t.ex, odd);
+    }
+    PhiT v[6];
+#pragma unroll
+    for (int f = 0; f < 6; f++) v[f] = ps[j[f]];
     PhiT acc = bs[p];
     const PhiT pi = ps[p];
 #pragma unroll
     for (int f = 0; f < 6; f++)
         if ((q >> (16 + f)) & 1u) acc += v[f];
-    const int deg = __popc(q & (63u << 16));
-    const PhiT r = PoisUpd<PhiT>::resid(acc, deg, pi);
+    const int k = __popc(q & (63u << 16));
+    const typename PoisUpd<PhiT>::deg_t d = dg.d[k];
+    const PhiT r = PoisUpd<PhiT>::resid(acc, d, pi);
     if (need && (q & TILE_OWN)) r2 += PoisUpd<PhiT>::r2(r);
-    return PoisUpd<PhiT>::apply(pi, omega, r, deg);
+    return PoisUpd<PhiT>::apply(pi, omega, r, d, dg.inv[k]);
 }
+// warp sum of the residual squares, valid in lane 0; a warp whose nodes are
+// all walls, or that has none, adds nothing (an FP64 shuffle tree takes the
+// pipe for 80 cycles per warp)
+__device__ __forceinline__ double tile_r2(double r2)
+{
+    return __any_sync(0xffffffffu, r2 != 0.0) ? warp_sum(r2) : 0.0;
+}
+__device__ __forceinline__ double tile_r2(float r2) { return warp_sum_ff_lane0(r2); }
+
 // one colour's half sweep: the items q of this thread, then those of index
 // U * blockDim.x + threadIdx.x on, formed by item(k) (all values before the first
 // store: nodes of one colour do not read one another)
 template <int U, typename PhiT, typename F>
-__device__ __forceinline__ void tile_sweep(const TileFrame &t, PhiT *ps, const PhiT *bs, const unsigned (&q)[U], int n,
-                                           F item, typename PoisUpd<PhiT>::om_t omega, bool need,
+__device__ __forceinline__ void tile_sweep(const TileFrame &t, const TileDeg<PhiT> &dg, PhiT *ps, const PhiT *bs,
+                                           const unsigned (&q)[U], int n, F item, typename PoisUpd<PhiT>::om_t omega, bool need,
                                            typename PoisUpd<PhiT>::acc_t &r2)
 {
     PhiT v[U];
     int p[U];
 #pragma unroll
-    for (int u = 0; u < U; u++) v[u] = tile_relax<PhiT>(t, ps, bs, q[u], omega, need, r2, p[u]);
+    for (int u = 0; u < U; u++) v[u] = tile_relax<PhiT>(t, dg, ps, bs, q[u], omega, need, r2, p[u]);
 #pragma unroll
     for (int u = 0; u < U; u++)
         if (p[u] >= 0) ps[p[u]] = v[u];
     for (int k = threadIdx.x + U * blockDim.x; k < n; k += blockDim.x) {
         int i;
-        const PhiT x = tile_relax<PhiT>(t, ps, bs, item(k), omega, need, r2, i);
+        const PhiT x = tile_relax<PhiT>(t, dg, ps, bs, item(k), omega, need, r2, i);
         if (i >= 0) ps[i] = x;
     }
 }
@@ -759,7 +804,12 @@ __global__ void __launch_bounds__(POIS_THREADS, 1) poisson_tiled_kernel(StepArgs
     const int nthr = nblk * blockDim.x;
     unsigned bar_k = 0;
     const int nx = g.nx, ey = tg.ty + 4, ez = tg.tz + 4, E = nx * ey * ez;
-    const TileFrame T{nx, ey, nx * ey, (E + 1) >> 1};
+    const TileFrame T{nx, ey, nx * ey, (E + 1) >> 1, (nx & 1) == 0};
+    __shared__ TileDeg<PhiT> dg;
+    if (threadIdx.x < 8) {
+        dg.d[threadIdx.x] = PoisUpd<PhiT>::d((int)threadIdx.x);
+        dg.inv[threadIdx.x] = PoisUpd<PhiT>::inv((int)threadIdx.x);
+    }
     PhiT *ps = (PhiT *)tsm;
     PhiT *bs = ps + 2 * T.M;
     uint32_t *ms = (uint32_t *)(bs + 2 * T.M);
@@ -767,9 +817,12 @@ __global__ void __launch_bounds__(POIS_THREADS, 1) poisson_tiled_kernel(StepArgs
     const int y0 = by * tg.ty - 2, z0 = bz * tg.tz - 2;  // global coordinates of the extended origin
     // --- source (grid-wide, as in the global kernel)
     const double t = form_source(a, tid, nthr, sh, bc);
-    if (threadIdx.x == 0) a.part_pois[blockIdx.x] = t;
+    // block partials in two sets taken in turn: a block may write the next
+    // sweep's while another still reads the last one's
+    auto part = [&](int k) { return a.part_pois + (size_t)(k & 1) * nblk; };
+    if (threadIdx.x == 0) part(1)[blockIdx.x] = t;
     if (!grid_barrier(a.barrier, nblk, bar_k, a.status)) return;
-    const double bn2 = sum_partials(a.part_pois, (int)nblk, bc);
+    const double bn2 = sum_partials(part(1), (int)nblk, bc);
     const double bnorm = sqrt(bn2);
     const int limit = a.fixed_iter > 0 ? a.fixed_iter : a.max_iter;
     if (a.fixed_iter <= 0 && bnorm == 0.0) {
@@ -813,6 +866,8 @@ __global__ void __launch_bounds__(POIS_THREADS, 1) poisson_tiled_kernel(StepArgs
     int it = 0, converged = 0;
     double r2tot = 0.0;
     const double tolb = a.tol * bnorm;
+    const double tol2_lo = tolb * tolb * (1.0 - 1e-14), tol2_hi = tolb * tolb * (1.0 + 1e-14);
+    bool test = false;  // the last sweep's residual is due for a test
     const typename PoisUpd<PhiT>::om_t *oms = (const typename PoisUpd<PhiT>::om_t *)a.omegas;
     const int ty = tg.ty, tz = tg.tz;
     const int hx = (nx + 1) >> 1;
@@ -892,7 +947,7 @@ __global__ void __launch_bounds__(POIS_THREADS, 1) poisson_tiled_kernel(StepArgs
         e = nx * ly + T.ex * lz + 2 * xh;
         return true;
     };
-    const bool even = (nx & 1) == 0;  // rows split into aligned 16-byte pairs
+    const bool even = T.even;  // rows split into aligned 16-byte pairs
     auto pair_last = [&](int e) { return !even && (e + 1) % nx == 0; };  // the pair's second node is none
     auto publish = [&](int e, int gi) {
         const PhiT v0 = ps[tile_at(T, e)];
@@ -926,7 +981,8 @@ __global__ void __launch_bounds__(POIS_THREADS, 1) poisson_tiled_kernel(StepArgs
         const bool need = (a.fixed_iter <= 0 && ((it + 1) % a.check_every) == 0) || it + 1 == limit;
         if (it > 0) {
             // reload the halo: every load of a thread is issued before the
-            // first is used
+            // first is used; the first warp then tests the last sweep's
+            // residual while the loads are under way
             longlong2 w[UH];
 #pragma unroll
             for (int u = 0; u < UH; u++) {
@@ -934,6 +990,15 @@ __global__ void __launch_bounds__(POIS_THREADS, 1) poisson_tiled_kernel(StepArgs
                 const long long *src = (const long long *)a.phi + hg[u];
                 if (even) w[u] = __ldcg((const longlong2 *)src);
                 else w[u] = {__ldcg(src), pair_last(he[u]) ? 0ll : __ldcg(src + 1)};
+            }
+            if (test && threadIdx.x < 32) {
+                const double v = warp_sum(lane_partials(part(it - 1), (int)nblk));
+                if (threadIdx.x == 0) {
+                    bc[0] = v;
+                    // sqrt(v) <= tolb, with the square root taken only where
+                    // it could decide
+                    cflag = v <= tol2_hi && (v < tol2_lo || sqrt(v) <= tolb);
+                }
             }
 #pragma unroll
             for (int u = 0; u < UH; u++) {
@@ -949,11 +1014,16 @@ __global__ void __launch_bounds__(POIS_THREADS, 1) poisson_tiled_kernel(StepArgs
                 ps[tile_at(T, e)] = v0;
             }
             __syncthreads();
+            if (test && cflag) {
+                converged = 1;
+                r2tot = bc[0];
+                break;
+            }
         }
         const typename PoisUpd<PhiT>::om_t om_r = __ldg(oms + 2 * it), om_b = __ldg(oms + 2 * it + 1);
-        tile_sweep<UR, PhiT>(T, ps, bs, qr, nred, red, om_r, need, r2);
+        tile_sweep<UR, PhiT>(T, dg, ps, bs, qr, nred, red, om_r, need, r2);
         __syncthreads();
-        tile_sweep<UB, PhiT>(T, ps, bs, qb, nblack, black, om_b, need, r2);
+        tile_sweep<UB, PhiT>(T, dg, ps, bs, qb, nblack, black, om_b, need, r2);
         __syncthreads();
 #pragma unroll
         for (int u = 0; u < UP; u++)
@@ -964,22 +1034,21 @@ __global__ void __launch_bounds__(POIS_THREADS, 1) poisson_tiled_kernel(StepArgs
             publish(e, gi);
         }
         if (need) {
-            double wsum;
-            if constexpr (((PhiT)0.5) != 0) wsum = warp_sum((double)r2);
-            else wsum = warp_sum_ff_lane0((float)r2);
-            double tb = block_sum_lanes0(wsum, sh);
-            if (threadIdx.x == 0) a.part_pois[blockIdx.x] = tb;
-        }
-        if (!grid_barrier(a.barrier, nblk, bar_k, a.status)) return;
-        const bool test = a.fixed_iter <= 0 && ((it + 1) % a.check_every) == 0;
-        if (test || it + 1 == limit) {
-            if (test_partials(a.part_pois, (int)nblk, tolb, bc, &cflag, r2tot) && test) {
-                converged = 1;
-                it++;
-                break;
+            const double wsum = tile_r2(r2);
+            if (lane == 0) sh[warp] = wsum;
+            __syncthreads();
+            if (warp == 0) {
+                const double tb = warp_sum(lane < nwarps ? sh[lane] : 0.0);
+                if (lane == 0) part(it)[blockIdx.x] = tb;
             }
         }
+        if (!grid_barrier(a.barrier, nblk, bar_k, a.status)) return;
+        test = a.fixed_iter <= 0 && ((it + 1) % a.check_every) == 0;
     }
+    // every sweep taken: the last one's residual, reported and, where it is due,
+    // tested
+    if (!converged && it > 0)
+        if (test_partials(part(it - 1), (int)nblk, tolb, bc, &cflag, r2tot) && test) converged = 1;
     // the whole tile to global memory (the sweeps wrote its rim)
     for (int k = threadIdx.x; k < nblack; k += blockDim.x) {
         const int row = k / hx, ly = 2 + row % ty, lz = 2 + row / ty, x = 2 * (k - row * hx);
