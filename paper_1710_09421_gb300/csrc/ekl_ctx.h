@@ -197,6 +197,9 @@ struct Batch {
     int mgs_split;
     void *d_ctl;             // MgCtl per replica
     void *d_grids;           // Grid3 per replica
+    int mgs_fused;           // lattice passes of two half sweeps per launch (0: of one)
+    int mgf_v, mgf_grid, mgf_threads, mgf_plane;  // their vector width, blocks, threads, largest plane (floats)
+    void *d_mgf_geom, *d_mgf_blocks;  // their tiles: per replica, per block
     int *d_loops;            // loop iterations run (launch accounting)
     cudaGraph_t mgs_graph;
     cudaGraphExec_t mgs_exec;

@@ -152,19 +152,31 @@ __device__ __forceinline__ void mgf_gather(MgfVec<V> &acc, const MgfVec<V> &own,
     mgf_addv(acc, zm);
     mgf_addv(acc, zp);
 }
+// Inverse degree (0 on dead nodes) and degree of a node by its link byte, in
+// shared memory: beside walls a warp then takes one load per node, where the
+// bit counts, selects and conversions took some 20 instructions and half of
+// a step on lattices with a membrane.
+struct MgfLut {
+    float inv[256], deg[256];
+};
+__device__ __forceinline__ void mgf_lut_fill(MgfLut &t)
+{
+    for (int b = threadIdx.x; b < 256; b += blockDim.x) {
+        const int d = __popc(mg_open((unsigned)b));
+        t.inv[b] = mgf_dead((unsigned)b) ? 0.f : mg_inv_deg(d);
+        t.deg[b] = (float)d;
+    }
+    __syncthreads();
+}
 // (r + sum) / deg, zero on dead nodes
-template <int V> __device__ __forceinline__ void mgf_scale(MgfVec<V> &a, unsigned lk)
+template <int V> __device__ __forceinline__ void mgf_scale(MgfVec<V> &a, unsigned lk, const MgfLut &t)
 {
     if (lk == 0) {
 #pragma unroll
         for (int i = 0; i < V; i++) a.v[i] *= 1.f / 6.f;
     } else {
 #pragma unroll
-        for (int i = 0; i < V; i++) {
-            const unsigned b = mgf_byte(lk, i);
-            const float v = a.v[i] * mg_inv_deg(__popc(mg_open(b)));
-            a.v[i] = mgf_dead(b) ? 0.f : v;
-        }
+        for (int i = 0; i < V; i++) a.v[i] *= t.inv[mgf_byte(lk, i)];
     }
 }
 
@@ -184,6 +196,9 @@ template <int MODE, int V, bool FIRST>
 __device__ __forceinline__ void mgf_body(const MgfGeom &G, const MgfArgs &A, int tile)
 {
     extern __shared__ __align__(16) float mgf_sm[];
+    __shared__ MgfLut lut;
+    mgf_lut_fill(lut);
+    const float deg6 = lut.deg[0];  // six open faces
     const int pitch = G.lpr * V, plane = pitch * G.rows;
     constexpr int N0 = MODE == MGF_RESTR ? 3 : 2;
     float *s0 = mgf_sm, *s1 = s0 + N0 * plane, *sr = s1 + 2 * plane;
@@ -303,7 +318,7 @@ __device__ __forceinline__ void mgf_body(const MgfGeom &G, const MgfArgs &A, int
         }
         if constexpr (MODE == MGF_PRE) {
             a.c0 = a.r0;
-            mgf_scale(a.c0, a.l0);
+            mgf_scale(a.c0, a.l0, lut);
         } else if constexpr (MODE == MGF_PRO) {
             a.c0 = fc;
             mgf_addv(a.c0, fe);
@@ -320,14 +335,14 @@ __device__ __forceinline__ void mgf_body(const MgfGeom &G, const MgfArgs &A, int
         // colour 1 of plane q - 1, whose x-parity is sp there
         b.c1 = b.r1;
         mgf_gather(b.c1, b.c0, edge, sp, ym0, yp0, c.c0, a.c0);
-        mgf_scale(b.c1, b.l1);
+        mgf_scale(b.c1, b.l1, lut);
         if (thr) mgf_sts<V>(s1 + ((q - 1) & 1) * plane + o, b.c1);
         // plane q - 2: colour 0 sits on x-parity sp
         const int pz = q - 2;
         if constexpr (MODE != MGF_RESTR) {
             MgfVec<V> cn = c.r0;
             mgf_gather(cn, c.c1, edge1, sp, ym, yp, c1d, b.c1);
-            mgf_scale(cn, c.l0);
+            mgf_scale(cn, c.l0, lut);
             if (mine && pz >= za && pz < zb) {
                 if constexpr (MODE == MGF_POST) {
                     float4 *dst = (float4 *)(A.z + n0 + nxy * pz);
@@ -369,12 +384,12 @@ __device__ __forceinline__ void mgf_body(const MgfGeom &G, const MgfArgs &A, int
             const int oe0 = sp ? ol : orr;
             const float edge0 = oe0 < 0 ? 0.f : p0[oe0];
             MgfVec<V> a0, a1;
+            const bool bulk = (c.l0 | c.l1) == 0;
 #pragma unroll
             for (int t = 0; t < V; t++) {
-                // (written as in the other passes, whatever the degree, so that
-                // the compiler rounds it alike)
-                const float d0 = (float)__popc(mg_open(mgf_byte(c.l0, t))),
-                            d1 = (float)__popc(mg_open(mgf_byte(c.l1, t)));
+                // (a degree that the compiler does not know, as in the other
+                // passes, so that it rounds the product alike)
+                const float d0 = bulk ? deg6 : lut.deg[mgf_byte(c.l0, t)], d1 = bulk ? deg6 : lut.deg[mgf_byte(c.l1, t)];
                 a0.v[t] = c.r0.v[t] - d0 * c.c0.v[t];
                 a1.v[t] = c.r1.v[t] - d1 * c.c1.v[t];
             }
@@ -411,6 +426,11 @@ __global__ void __launch_bounds__(MGF_THREADS, 1) mgf_kernel(MgfGeom G, MgfArgs 
     cudaGridDependencySynchronize();
     mgf_body<MODE, V, FIRST>(G, A, blockIdx.x);
 }
+
+// one block of a launch over all replicas of a batch
+struct MgfBlock {
+    int rep, tile;
+};
 
 // Partials of r.z after the last smoothing launch, with the thread-to-node
 // map and the order of additions of the reducing half sweep it stands in for
@@ -457,10 +477,12 @@ __device__ __forceinline__ float mgf_dot(const Grid3 &g, const L *__restrict__ l
 // step costing the larger of its dependent chain (about 600 cycles) and about
 // 105 cycles per resident warp, 120 where rows do not fill whole warps (the
 // warps then hold rows of both parities).  False when the rows cannot be
-// read in aligned pieces.
-inline bool mgf_pick(MgfGeom &G, int &V, int nx, int ny, int nz, const int per[3], int num_sms, int share = 1)
+// read in aligned pieces.  share: lattices like this one in the launch; vmax 2:
+// pieces of four nodes even where eight would fit.
+inline bool mgf_pick(MgfGeom &G, int &V, int nx, int ny, int nz, const int per[3], int num_sms, int share = 1,
+                     int vmax = 4)
 {
-    V = nx % 8 == 0 ? 4 : nx % 4 == 0 ? 2 : 0;
+    V = nx % 8 == 0 && vmax == 4 ? 4 : nx % 4 == 0 ? 2 : 0;
     if (V == 0) return false;
     double best = 1e300;
     for (int tx : {nx, 32, 64, 128, 256}) {
@@ -468,7 +490,7 @@ inline bool mgf_pick(MgfGeom &G, int &V, int nx, int ny, int nz, const int per[3
         const int lpr = tx / (2 * V) + (tx < nx ? 2 : 0), ntx = (nx + tx - 1) / tx;
         for (int oy = 2; lpr * (oy + 4) <= MGF_THREADS; oy += 2) {
             const int rows = oy + 4, nty = (ny + oy - 1) / oy, thr = (lpr * rows + 31) / 32 * 32;
-            const size_t smem = 7 * (size_t)lpr * V * rows * sizeof(float) + 1024;
+            const size_t smem = 7 * (size_t)lpr * V * rows * sizeof(float) + sizeof(MgfLut) + 1024;
             int bps = (int)((227 * 1024) / smem);
             if (bps > MGF_THREADS / thr) bps = MGF_THREADS / thr;
             if (bps < 1) continue;

@@ -469,6 +469,39 @@ __global__ static void __launch_bounds__(MGS_THREADS, 1) mgsb_restrict_kernel(Mg
     else fine_restrict_cells<false>(g, m.link, m.r, m.z, l1, x.t0, x.nt);
 }
 
+// The lattice passes of every active replica, two half sweeps per launch
+// (ekl_mgf.cuh), each replica in tiles of its own.  Ten replicas of 6.5 M nodes
+// in all: the passes before and after the coarse levels take 60 and 71 us
+// against 131 and 144 us of one half sweep per launch.
+template <int MODE, int V>
+__global__ void __launch_bounds__(MGF_THREADS, 1) mgfb_kernel(MgsBatch B, const MgfGeom *geom, const MgfBlock *blocks)
+{
+    mgs_wait_previous();
+    const MgfBlock t = blocks[blockIdx.x];
+    if (B.ctl[t.rep].done) return;
+    const MgArgs &m = B.mg[t.rep];
+    const MgfGeom G = geom[t.rep];
+    float *ca = m.q, *cb = m.q + (size_t)G.nx * G.ny * G.nz / 2;
+    const MgfArgs A{m.r, m.link, MODE == MGF_POST ? cb : ca, MODE == MGF_PRE ? ca : cb, m.z, m.lev[1].e,
+                    m.lev[1].f, m.lev[1].e, m.lev[1].sig, m.lev[1].nx, m.lev[1].ny, m.lev[1].nz};
+    // (the start of level 1's smoothing is overwritten where one block takes
+    // that level whole)
+    mgf_body<MODE, V, MODE == MGF_RESTR>(G, A, t.tile);
+}
+
+__global__ static void __launch_bounds__(MGS_THREADS, 1) mgsb_dot_kernel(MgsBatch B)
+{
+    mgs_wait_previous();
+    __shared__ double sh[MGS_THREADS / 32];
+    const BRep x = mgsb_rep(B.pb);
+    if (B.ctl[x.r].done) return;
+    const MgArgs &m = B.mg[x.r];
+    const Grid3 g = B.grid[x.r];
+    const float rz = mgf_dot(g, m.link, m.r, m.z, x.t0, x.nt);
+    const double t = block_sum_lanes0(warp_sum_ff_lane0(rz), sh);
+    if (threadIdx.x == 0) mgsb_slot(B, x.r, MGS_RZ)[x.lb] = t;
+}
+
 // the coarse levels of every active replica (cooperative; `bars` zeroed)
 template <typename S, typename R, typename PhiT>
 __global__ void __launch_bounds__(MGS_THREADS, 1)
@@ -511,7 +544,7 @@ __global__ static void __launch_bounds__(MGS_THREADS, 1) mgsb_pq_kernel(MgsBatch
     if (threadIdx.x == 0) mgsb_slot(B, x.r, MGS_PQ)[x.lb] = pq;
 }
 
-template <typename S, typename R, typename PhiT>
+template <typename S, typename R, typename PhiT, bool START = true>
 __global__ void __launch_bounds__(MGS_THREADS, 1) mgsb_update_kernel(const StepArgs<S, R, PhiT> *reps, MgsBatch B)
 {
     mgs_wait_previous();
@@ -526,7 +559,7 @@ __global__ void __launch_bounds__(MGS_THREADS, 1) mgsb_update_kernel(const StepA
     if (!(rz > 0.0) || !(pq > 0.0)) return;
     const double alpha = rz / pq;
     const Grid3 g = B.grid[x.r];
-    const float t = mg_update_pass<PhiT>(g, m.link, reps[x.r].phi, m.p[c.pi ^ 1], m.q, m.r, m.z, alpha,
+    const float t = mg_update_pass<PhiT, START>(g, m.link, reps[x.r].phi, m.p[c.pi ^ 1], m.q, m.r, m.z, alpha,
                                          x.t0, x.nt);
     const double rr = block_sum_lanes0(warp_sum_ff_lane0(t), sh);
     if (threadIdx.x == 0) mgsb_slot(B, x.r, MGS_RR)[x.lb] = rr;

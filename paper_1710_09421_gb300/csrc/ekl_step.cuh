@@ -753,8 +753,33 @@ template <typename S, typename R, typename PhiT> static cudaError_t mgsb_build(B
             const cudaError_t r = cudaLaunchKernelEx(&lc, kern, args...);
             if (el == cudaSuccess) el = r;
         };
-        for (int s = 1; s < 2 * MG_NU; s++) go(s > 1, nb, nt, mgsb_half_kernel<false, false>, mb, s & 1);
-        go(true, nb, nt, mgsb_restrict_kernel, mb);
+        auto fused = [&](bool overlap, auto mode) {
+            constexpr int MODE = decltype(mode)::value;
+            const size_t smem = (MODE == MGF_RESTR ? 7 : 4) * (size_t)B.mgf_plane * sizeof(float);
+            auto launch = [&](auto kern) {
+                cudaError_t r = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+                cudaLaunchConfig_t lc = {};
+                lc.gridDim = dim3(B.mgf_grid);
+                lc.blockDim = dim3(B.mgf_threads);
+                lc.dynamicSmemBytes = smem;
+                lc.stream = cs;
+                lc.attrs = dep;
+                lc.numAttrs = (overlap && pdl) ? 1 : 0;
+                if (r == cudaSuccess)
+                    r = cudaLaunchKernelEx(&lc, kern, mb, (const MgfGeom *)B.d_mgf_geom,
+                                           (const MgfBlock *)B.d_mgf_blocks);
+                if (el == cudaSuccess) el = r;
+            };
+            if (B.mgf_v == 4) launch(mgfb_kernel<MODE, 4>);
+            else launch(mgfb_kernel<MODE, 2>);
+        };
+        if (B.mgs_fused) {
+            fused(false, std::integral_constant<int, MGF_PRE>());
+            fused(true, std::integral_constant<int, MGF_RESTR>());
+        } else {
+            for (int s = 1; s < 2 * MG_NU; s++) go(s > 1, nb, nt, mgsb_half_kernel<false, false>, mb, s & 1);
+            go(true, nb, nt, mgsb_restrict_kernel, mb);
+        }
         cudaMemsetAsync(bars, 0, 4 * sizeof(unsigned) * (size_t)n, cs);
         cudaLaunchConfig_t cfg = {};
         cudaLaunchAttribute coop[1];
@@ -768,14 +793,21 @@ template <typename S, typename R, typename PhiT> static cudaError_t mgsb_build(B
         cfg.numAttrs = 1;
         const cudaError_t ecoop = cudaLaunchKernelEx(&cfg, mgsb_coarse_kernel<S, R, PhiT>, reps, mb, bars);
         if (el == cudaSuccess) el = ecoop;
-        go(false, nb, nt, mgsb_half_kernel<false, true>, mb, 1);
-        for (int s = 1; s < 2 * MG_NU; s++) {
-            const int col = (s & 1) ^ 1;
-            if (s == 2 * MG_NU - 1) go(true, nb, nt, mgsb_half_kernel<true, false>, mb, col);
-            else go(true, nb, nt, mgsb_half_kernel<false, false>, mb, col);
+        if (B.mgs_fused) {
+            fused(false, std::integral_constant<int, MGF_PRO>());
+            fused(true, std::integral_constant<int, MGF_POST>());
+            go(true, nb, nt, mgsb_dot_kernel, mb);
+        } else {
+            go(false, nb, nt, mgsb_half_kernel<false, true>, mb, 1);
+            for (int s = 1; s < 2 * MG_NU; s++) {
+                const int col = (s & 1) ^ 1;
+                if (s == 2 * MG_NU - 1) go(true, nb, nt, mgsb_half_kernel<true, false>, mb, col);
+                else go(true, nb, nt, mgsb_half_kernel<false, false>, mb, col);
+            }
         }
         go(true, nb, nt, mgsb_pq_kernel, mb);
-        go(true, nb, nt, mgsb_update_kernel<S, R, PhiT>, reps, mb);
+        if (B.mgs_fused) go(true, nb, nt, mgsb_update_kernel<S, R, PhiT, false>, reps, mb);
+        else go(true, nb, nt, mgsb_update_kernel<S, R, PhiT>, reps, mb);
         go(true, n, 32, mgsb_mid_kernel, mb);
         go(true, nb, nt, mgsb_residual_kernel<S, R, PhiT>, reps, mb, 1);
         go(true, n, 32, mgsb_end_kernel<S, R, PhiT>, reps, mb);
@@ -802,8 +834,9 @@ template <typename S, typename R, typename PhiT> static cudaError_t mgsb_build(B
     B.mgs_graph = G;
     B.mgs_blocks = nb;
     B.mgs_cblocks = ncb;
-    // half sweeps, restriction, coarse, p/q, update, mid, residual, end, condition
-    B.mgs_iter_kernels = 2 * (2 * MG_NU - 1) + 1 + 1 + 1 + 6;
+    // half sweeps, restriction (fused: two launches before the coarse one, three
+    // after it), coarse, p/q, update, mid, residual, end, condition
+    B.mgs_iter_kernels = (B.mgs_fused ? 5 : 2 * (2 * MG_NU - 1) + 2) + 1 + 6;
     return cudaSuccess;
 }
 

@@ -52,6 +52,32 @@ def test_fused_smoothing_equals_single_launch(dims, periodic, precision):
         assert np.array_equal(fa[k], fb[k]), k
 
 
+@pytest.mark.parametrize("boxes", [
+    [(96, 96, 192), (128, 96, 128), (48, 48, 192)],   # pieces of eight nodes
+    [(100, 96, 192), (128, 96, 128), (48, 48, 192)],  # of four for all
+])
+def test_batch_fused_smoothing_equals_cooperative(boxes):
+    """The same for a batch whose replicas together exceed L2: the launches of
+    two half sweeps over all replicas and one cooperative launch (schedule 2:
+    the same blocks per replica) return the same bits."""
+    wls = [_box(*d, (0, 1, 1), "f32") for d in boxes]
+    assert sum(w.n_nodes for w in wls) * 37 > 126 << 20
+    a = E.Batch([w.replace(flags=MG) for w in wls])
+    b = E.Batch([w.replace(flags=MG | W.FLAG_POISSON_MG_SINGLE) for w in wls])
+    a.set_schedule(2)
+    b.set_schedule(2)
+    for _ in range(2):
+        assert a.step(1) >= 0 and b.step(1) >= 0
+        for r in range(len(wls)):
+            sa, sb = a.reps[r].stats(), b.reps[r].stats()
+            assert sa["poisson_iters"] == sb["poisson_iters"] > 0 and sa["poisson_res"] == sb["poisson_res"], r
+    for r in range(len(wls)):
+        fa, fb = a.reps[r].fields(("n", "phi")), b.reps[r].fields(("n", "phi"))
+        assert np.array_equal(fa["n"], fb["n"]) and np.array_equal(fa["phi"], fb["phi"]), r
+    a.close()
+    b.close()
+
+
 @pytest.mark.parametrize("dims,periodic", [
     ((40, 24, 36), (1, 1, 1)),   # 4320 cells: positions kept in registers
     ((36, 28, 60), (1, 1, 1)),   # 7560 cells: positions formed in every sweep
