@@ -824,9 +824,9 @@ static const char *build_multigrid(Ctx &c, const uint8_t *solid, Alloc &A, long 
     c.mgs_l1 = c.mg_split && c.mg_cta_from > 1 && c.mg_tile_from > 1;
     // two half sweeps per launch on lattices whose solve does not stay in L2
     // (37 bytes a node: r, z, p, p', q, the link byte, and phi and b of 8),
-    // where rows split into aligned pieces of four nodes: 256x256x512 takes 5.63
+    // where rows split into aligned pieces of four nodes: 256x256x512 takes 5.46
     // ms per solve with it and 7.64 with one half sweep per launch, 128x128x256
-    // 1.25 and 1.40, and 64x64x128, bound by the chain of plane steps, 0.59 and
+    // 1.09 and 1.40, and 64x64x128, bound by the chain of plane steps, 0.59 and
     // 0.50.
     const size_t l2 = 126u << 20;
     c.mg_fused = c.mg_split && c.mg_wide && c.nx % 4 == 0 && (size_t)N * 37 > l2;
@@ -1667,8 +1667,8 @@ int ekl_batch_create(int32_t nrep, const ekl_params *params, void *stream, ekl_b
             B.d_crb = (int *)A(4 * (size_t)nrep);
             B.d_mgs_part = (double *)A(sizeof(double) * MGS_PART_SLOTS * (size_t)nrep * B.mgs_part_stride);
             // two half sweeps per launch, as on single lattices: where the
-            // replicas together do not stay in L2 (ten of 6.5 M nodes: 3.6 ms a
-            // step without it, 2.9 with it) and all rows split into aligned pieces
+            // replicas together do not stay in L2 (ten of 6.5 M nodes: 3.65 ms a
+            // step without it, 3.22 with it) and all rows split into aligned pieces
             long long total = 0;
             int vmax = 4;
             for (int r = 0; r < nrep; r++) {
@@ -1683,6 +1683,7 @@ int ekl_batch_create(int32_t nrep, const ekl_params *params, void *stream, ekl_b
                     const Ctx &c = *B.reps[r];
                     MgfGeom &G = geom[r];
                     const int share = (int)std::max(1ll, total / c.N);
+                    // (three blocks an SM: 3.48 ms a step, with one 3.53, with six 3.73)
                     if (!mgf_pick(G, B.mgf_v, c.nx, c.ny, c.nz, c.per, 3 * sms, share, vmax)) {
                         B.mgs_fused = 0;
                         break;

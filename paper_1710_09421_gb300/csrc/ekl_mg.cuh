@@ -767,9 +767,9 @@ static __device__ void coarse_post_tiles(const MgLevel &L, const MgLevel &C, con
 // colour in a row then lie in consecutive words, whatever the extents, and a
 // warp's loads of a half sweep meet no bank twice.  With e and f in index
 // order and the conductances as float4 beside them every update cost 30 bank
-// cycles, and its indices two divisions: 67 us per V-cycle on a coarsest level
-// of 20 x 12 x 18 cells, now 27 (16 half sweeps of 1900 cycles; two FP64 means
-// of 8000).
+// cycles, and its indices two divisions: a CG iteration on 40 x 24 x 36 nodes,
+// whose coarsest level of 20 x 12 x 18 cells is smoothed here, took 103 us, now
+// 78 (of which 16 half sweeps of 1900 cycles and two FP64 means of 8000).
 struct CtaLev {
     int nx, ny, nz, N, M;  // M: cells per parity (rounded up)
     float *e, *f, *sx, *sy, *sz, *w;

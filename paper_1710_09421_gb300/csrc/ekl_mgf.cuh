@@ -27,7 +27,7 @@
 // What bounds it: the chain of a plane step (0.9 us: a plane's loads, the two
 // dependent updates and the barrier) at 15 to 16 warps an SM, so it serves
 // lattices larger than L2, where the one-half-sweep passes are bound by their
-// traffic.  256x256x512, us per launch: PRE 82, RESTR 121, PRO 87, POST 91 and
+// traffic.  256x256x512, us per launch: PRE 66, RESTR 108, PRO 79, POST 86 and
 // the r.z partials 47, in place of three half sweeps of 88, the restriction of
 // 101, and half sweeps of 127, 88, 88 and 106.  Two half sweeps per launch on
 // 64x64x128 (13 us each), a whole pass per launch in tiles with a halo of four

@@ -471,7 +471,7 @@ __global__ static void __launch_bounds__(MGS_THREADS, 1) mgsb_restrict_kernel(Mg
 
 // The lattice passes of every active replica, two half sweeps per launch
 // (ekl_mgf.cuh), each replica in tiles of its own.  Ten replicas of 6.5 M nodes
-// in all: the passes before and after the coarse levels take 60 and 71 us
+// in all: the passes before and after the coarse levels take 76 and 97 us
 // against 131 and 144 us of one half sweep per launch.
 template <int MODE, int V>
 __global__ void __launch_bounds__(MGF_THREADS, 1) mgfb_kernel(MgsBatch B, const MgfGeom *geom, const MgfBlock *blocks)
