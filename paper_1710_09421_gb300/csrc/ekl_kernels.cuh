@@ -1086,7 +1086,10 @@ __global__ void __launch_bounds__(POIS_THREADS, 1) poisson_batch_kernel(const St
 {
     __shared__ double sh[POIS_THREADS / 32];
     __shared__ double s_tolb[MAX_REPS], s_bnorm[MAX_REPS], s_res[MAX_REPS];
-    __shared__ int s_active[MAX_REPS], s_iters[MAX_REPS], s_conv[MAX_REPS], s_any;
+    __shared__ int s_active[MAX_REPS], s_iters[MAX_REPS], s_conv[MAX_REPS];
+    // each replica's sweep cap and test interval (0: fixed sweeps): read from
+    // its descriptor once (thread 0 read all of them before every sweep)
+    __shared__ int s_lim[MAX_REPS], s_chk[MAX_REPS];
     const int rep = pb.block_rep[blockIdx.x], lb = pb.block_local[blockIdx.x], kr = pb.rep_blocks[rep];
     const StepArgs<S, R, PhiT> &a = reps[rep];
     const Grid3 g = a.g;
@@ -1098,12 +1101,26 @@ __global__ void __launch_bounds__(POIS_THREADS, 1) poisson_batch_kernel(const St
     const double t = form_source(a, tid, nthr, sh, bc);
     if (threadIdx.x == 0) a.part_pois[lb] = t;
     if (!grid_barrier(pb.barrier, gridDim.x, bar_k, pb.status)) return;
+    // the sum of a replica's block partials in order, eight loads in flight
+    auto partials = [&](int r) {
+        const double *p = reps[r].part_pois;
+        const int n = pb.rep_blocks[r];
+        double v = 0.0;
+        for (int k0 = 0; k0 < n; k0 += 8) {
+            double x[8];
+#pragma unroll
+            for (int u = 0; u < 8; u++) x[u] = k0 + u < n ? __ldcg(p + k0 + u) : 0.0;
+#pragma unroll
+            for (int u = 0; u < 8; u++) v += x[u];
+        }
+        return v;
+    };
     // every replica's source norm and activity, in every block
     for (int r = threadIdx.x; r < pb.nrep; r += blockDim.x) {
         const StepArgs<S, R, PhiT> &q = reps[r];
-        double v = 0.0;
-        for (int k = 0; k < pb.rep_blocks[r]; k++) v += __ldcg(q.part_pois + k);
-        const double bn = sqrt(v);
+        const double bn = sqrt(partials(r));
+        s_lim[r] = q.fixed_iter > 0 ? q.fixed_iter : q.max_iter;
+        s_chk[r] = q.fixed_iter > 0 ? 0 : q.check_every;
         s_bnorm[r] = bn;
         s_tolb[r] = q.tol * bn;
         s_active[r] = !(q.fixed_iter <= 0 && bn == 0.0);
@@ -1117,18 +1134,12 @@ __global__ void __launch_bounds__(POIS_THREADS, 1) poisson_batch_kernel(const St
     const typename PoisUpd<PhiT>::om_t *oms = (const typename PoisUpd<PhiT>::om_t *)a.omegas;
     for (int it = 0;; it++) {
         // who is still sweeping: within its cap and not converged
-        if (threadIdx.x == 0) {
-            int any = 0;
-            for (int r = 0; r < pb.nrep; r++) {
-                const StepArgs<S, R, PhiT> &q = reps[r];
-                const int lim = q.fixed_iter > 0 ? q.fixed_iter : q.max_iter;
-                if (s_active[r] && it >= lim) s_active[r] = 0;
-                any |= s_active[r];
-            }
-            s_any = any;
+        int any = 0;
+        for (int r = threadIdx.x; r < pb.nrep; r += blockDim.x) {
+            if (s_active[r] && it >= s_lim[r]) s_active[r] = 0;
+            any |= s_active[r];
         }
-        __syncthreads();
-        if (!s_any) break;
+        if (!__syncthreads_or(any)) break;
         const bool mine = s_active[rep] != 0;
         const bool need = mine && ((a.fixed_iter <= 0 && ((it + 1) % a.check_every) == 0) ||
                                    it + 1 == (a.fixed_iter > 0 ? a.fixed_iter : a.max_iter));
@@ -1144,14 +1155,18 @@ __global__ void __launch_bounds__(POIS_THREADS, 1) poisson_batch_kernel(const St
                         const int x = 2 * xh + par;
                         if (x >= g.nx) continue;
                         const int i = x + g.nx * row;
+                        // (every load before the link word is known: one
+                        // memory round trip; neighbour indices are always
+                        // valid, and closed faces are left out later)
                         const uint32_t m = a.mask[i];
-                        if (m & SOLID_BIT) continue;
                         int nb[6];
                         face_nbrs(g, x, y, z, i, nb);
                         PhiT v[6];
 #pragma unroll
-                        for (int f = 0; f < 6; f++) v[f] = ((m >> (f + 1)) & 1u) ? (PhiT)0 : __ldcg(a.phi + nb[f]);
-                        sor_apply<PhiT>(a.phi, i, m, __ldcg(a.b + i), __ldcg(a.phi + i), v, omega, r2);
+                        for (int f = 0; f < 6; f++) v[f] = __ldcg(a.phi + nb[f]);
+                        const PhiT bi = __ldcg(a.b + i), pi = __ldcg(a.phi + i);
+                        if (m & SOLID_BIT) continue;
+                        sor_apply<PhiT>(a.phi, i, m, bi, pi, v, omega, r2);
                     }
                 }
             }
@@ -1167,12 +1182,9 @@ __global__ void __launch_bounds__(POIS_THREADS, 1) poisson_batch_kernel(const St
         // residual tests of every replica that tests at this sweep
         for (int r = threadIdx.x; r < pb.nrep; r += blockDim.x) {
             if (!s_active[r]) continue;
-            const StepArgs<S, R, PhiT> &q = reps[r];
-            const int lim = q.fixed_iter > 0 ? q.fixed_iter : q.max_iter;
-            const bool test = q.fixed_iter <= 0 && ((it + 1) % q.check_every) == 0;
-            if (!test && it + 1 != lim) continue;
-            double v = 0.0;
-            for (int k = 0; k < pb.rep_blocks[r]; k++) v += __ldcg(q.part_pois + k);
+            const bool test = s_chk[r] > 0 && ((it + 1) % s_chk[r]) == 0;
+            if (!test && it + 1 != s_lim[r]) continue;
+            const double v = partials(r);
             s_res[r] = v;
             s_iters[r] = it + 1;
             if (test && sqrt(v) <= s_tolb[r]) {
