@@ -132,6 +132,7 @@ void release(Ctx &c)
     dev_free(c, c.rho, 0);
     dev_free(c, c.b, 0);
     dev_free(c, c.phi, 0);
+    dev_free(c, c.phi_rim, 0);
     dev_free(c, c.part_charge, 0);
     dev_free(c, c.part_charge_q, 0);
     dev_free(c, c.charge_tot, 0);
@@ -1048,6 +1049,7 @@ static int create_handle(const ekl_params *P, void *stream, ekl_handle **out, bo
     c.rho = A(N * rs);
     c.b = A(N * ps);
     c.phi = A(N * ps);
+    if (c.pois_tiled && !(P->flags & EKL_POISSON_MG)) c.phi_rim = A(N * ps);
     c.part_charge = (double *)A((size_t)c.charge_blocks * (CHARGE_THREADS / 32) * sizeof(double));
     c.part_charge_q = (long long *)A((size_t)c.charge_blocks * sizeof(long long));
     c.charge_tot = (double *)A(sizeof(double));

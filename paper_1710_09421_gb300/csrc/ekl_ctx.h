@@ -86,6 +86,7 @@ struct Ctx {
     void *rho;         // Real[N]
     void *b;           // PhiT[N]
     void *phi;         // PhiT[N]
+    void *phi_rim;     // PhiT[N]: the tiled SOR's second copy of the rows its tiles exchange, or null
     double *part_charge;  // [charge blocks]
     long long *part_charge_q;  // [charge blocks] fixed-point paths: exact sum of rho * 2^40
     double *charge_tot;        // totals of the two (charge_total_kernel)

@@ -14,6 +14,7 @@
 #include <cooperative_groups.h>
 
 #include "ekl_dev.cuh"
+#include "ekl_rim.h"
 
 namespace ekl {
 
@@ -30,6 +31,7 @@ template <typename S, typename R, typename PhiT> struct StepArgs {
     const S *__restrict__ fin;  // post-collision populations of the previous step
     S *__restrict__ fout;       // post-collision populations of this step
     PhiT *phi;
+    PhiT *phi_rim;  // tiled SOR: second copy of the rows its tiles exchange
     PhiT *b;
     R *rho;
     const R *__restrict__ wall_share;  // null when no wall carries charge
@@ -678,9 +680,10 @@ __global__ void __launch_bounds__(POIS_THREADS, 1) poisson_kernel(StepArgs<S, R,
 // shared memory for the whole solve.  A sweep updates the red nodes of T and
 // of the first halo layer (the halo red values are recomputed from the same
 // inputs as their owner's, so they are bitwise the owner's), then the black
-// nodes of T, writes the rows that other tiles read to global memory and passes
-// one grid barrier; the next sweep reloads only the halo.  Results are bitwise
-// those of the global-memory kernel (same node updates, same schedule).
+// nodes of T, writes the rows that other tiles read to global memory (into two
+// copies of the potential in turn, ekl_rim.h) and passes one grid barrier; the
+// next sweep reloads only the halo.  Results are bitwise those of the
+// global-memory kernel (same node updates, same schedule).
 struct TileGeom {
     int ty, tz, nty, ntz;  // tile extents and tile counts along y and z
 };
@@ -949,15 +952,16 @@ __global__ void __launch_bounds__(POIS_THREADS, 1) poisson_tiled_kernel(StepArgs
     };
     const bool even = T.even;  // rows split into aligned 16-byte pairs
     auto pair_last = [&](int e) { return !even && (e + 1) % nx == 0; };  // the pair's second node is none
-    auto publish = [&](int e, int gi) {
+    auto copy = [&](int k) { return k ? a.phi_rim : a.phi; };
+    auto publish = [&](PhiT *phi, int e, int gi) {
         const PhiT v0 = ps[tile_at(T, e)];
         if (even) {
             const longlong2 w = {__builtin_bit_cast(long long, v0),
                                  __builtin_bit_cast(long long, ps[tile_at(T, e + 1)])};
-            __stcg((longlong2 *)(a.phi + gi), w);
+            __stcg((longlong2 *)(phi + gi), w);
         } else {
-            __stcg(a.phi + gi, v0);
-            if (!pair_last(e)) __stcg(a.phi + gi + 1, ps[tile_at(T, e + 1)]);
+            __stcg(phi + gi, v0);
+            if (!pair_last(e)) __stcg(phi + gi + 1, ps[tile_at(T, e + 1)]);
         }
     };
     // what a thread does in every sweep, found once: positions of its first
@@ -983,11 +987,12 @@ __global__ void __launch_bounds__(POIS_THREADS, 1) poisson_tiled_kernel(StepArgs
             // reload the halo: every load of a thread is issued before the
             // first is used; the first warp then tests the last sweep's
             // residual while the loads are under way
+            const PhiT *rows = copy(rim_load_copy(it));
             longlong2 w[UH];
 #pragma unroll
             for (int u = 0; u < UH; u++) {
                 if (he[u] < 0) continue;
-                const long long *src = (const long long *)a.phi + hg[u];
+                const long long *src = (const long long *)rows + hg[u];
                 if (even) w[u] = __ldcg((const longlong2 *)src);
                 else w[u] = {__ldcg(src), pair_last(he[u]) ? 0ll : __ldcg(src + 1)};
             }
@@ -1009,8 +1014,8 @@ __global__ void __launch_bounds__(POIS_THREADS, 1) poisson_tiled_kernel(StepArgs
             for (int k = threadIdx.x + UH * blockDim.x; k < nhalo; k += blockDim.x) {
                 int e, gi;
                 if (!halo(k, e, gi)) continue;
-                const PhiT v0 = __ldcg(a.phi + gi);
-                if (!pair_last(e)) ps[tile_at(T, e + 1)] = __ldcg(a.phi + gi + 1);
+                const PhiT v0 = __ldcg(rows + gi);
+                if (!pair_last(e)) ps[tile_at(T, e + 1)] = __ldcg(rows + gi + 1);
                 ps[tile_at(T, e)] = v0;
             }
             __syncthreads();
@@ -1025,13 +1030,14 @@ __global__ void __launch_bounds__(POIS_THREADS, 1) poisson_tiled_kernel(StepArgs
         __syncthreads();
         tile_sweep<UB, PhiT>(T, dg, ps, bs, qb, nblack, black, om_b, need, r2);
         __syncthreads();
+        PhiT *dst = copy(rim_store_copy(it));
 #pragma unroll
         for (int u = 0; u < UP; u++)
-            if (pe[u] >= 0) publish(pe[u], pg[u]);
+            if (pe[u] >= 0) publish(dst, pe[u], pg[u]);
         for (int k = threadIdx.x + UP * blockDim.x; k < nrim; k += blockDim.x) {
             int e, gi;
             rim(k, e, gi);
-            publish(e, gi);
+            publish(dst, e, gi);
         }
         if (need) {
             const double wsum = tile_r2(r2);
@@ -1049,10 +1055,11 @@ __global__ void __launch_bounds__(POIS_THREADS, 1) poisson_tiled_kernel(StepArgs
     // tested
     if (!converged && it > 0)
         if (test_partials(part(it - 1), (int)nblk, tolb, bc, &cflag, r2tot) && test) converged = 1;
-    // the whole tile to global memory (the sweeps wrote its rim)
+    // the whole tile to phi (a block that still loads halo rows of the last sweep
+    // from there finds the same values before and after)
     for (int k = threadIdx.x; k < nblack; k += blockDim.x) {
         const int row = k / hx, ly = 2 + row % ty, lz = 2 + row / ty, x = 2 * (k - row * hx);
-        publish(nx * ly + T.ex * lz + x, nx * ((y0 + ly) + g.ny * (z0 + lz)) + x);
+        publish(a.phi, nx * ly + T.ex * lz + x, nx * ((y0 + ly) + g.ny * (z0 + lz)) + x);
     }
     if (tid == 0) {
         *a.pois_iters = it;

@@ -24,6 +24,7 @@ static StepArgs<S, R, PhiT> make_args(Ctx &c, int parity = -1)
     a.fin = (const S *)c.f[cur];
     a.fout = (S *)c.f[1 - cur];
     a.phi = (PhiT *)c.phi;
+    a.phi_rim = (PhiT *)c.phi_rim;
     a.b = (PhiT *)c.b;
     a.rho = (R *)c.rho;
     a.wall_share = (const R *)c.wall_share;
