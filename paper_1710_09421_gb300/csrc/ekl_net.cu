@@ -958,6 +958,26 @@ void net_backward(NetWork &W, const NetInput &in, int ns, const float *d_t, cons
                                                   W.grad);
 }
 
+// Extents that the kernels' 32-bit node ids (up to 2 N, the second input
+// channel) and the splits into tiles can take: none empty, at most 2^30 nodes.
+// False with the message set otherwise.
+bool grid_ok(const int32_t dims[3])
+{
+    long long n = 1;
+    for (int a = 0; a < 3; a++) {
+        if (dims[a] < 1) {
+            set_last_error("every extent must be >= 1");
+            return false;
+        }
+        n *= dims[a];
+        if (n > (1ll << 30)) {
+            set_last_error("grid too large for 32-bit node ids");
+            return false;
+        }
+    }
+    return true;
+}
+
 NetGrid make_grid(const int32_t dims[3], const int32_t periodic[3])
 {
     NetGrid g;
@@ -1296,7 +1316,7 @@ int ekl_net_tensor_path(int32_t path)
 
 int ekl_net_eval(const int32_t dims[3], const int32_t periodic[3], const float *x, const float *w, float *y)
 {
-    if (!dims || !x || !w || !y || dims[0] < 1 || dims[1] < 1 || dims[2] < 1) return EKL_ERR_ARG;
+    if (!dims || !x || !w || !y || !grid_ok(dims)) return EKL_ERR_ARG;
     NetWork W;
     W.g = make_grid(dims, periodic);
     int rc = work_alloc(W, 1, false);
@@ -1326,7 +1346,7 @@ static long long mask_count(const uint8_t *mask, int N)
 int ekl_net_loss_grad(const int32_t dims[3], const int32_t periodic[3], const float *x, const float *target,
                       const uint8_t *mask, const float *w, double *loss, float *grad)
 {
-    if (!dims || !x || !target || !w || !grad) return EKL_ERR_ARG;
+    if (!dims || !x || !target || !w || !grad || !grid_ok(dims)) return EKL_ERR_ARG;
     NetWork W;
     W.g = make_grid(dims, periodic);
     const int N = W.g.N;
@@ -1365,11 +1385,11 @@ int ekl_net_train_grid(int32_t nsamples, const int32_t dims[3], const int32_t pe
                        const float *target, const uint8_t *mask, float *w, int32_t iters, int32_t batch, float lr,
                        uint64_t seed, float *loss_out)
 {
-    if (nsamples < 1 || !dims || !x || !target || !w || iters < 0 || batch < 1) return EKL_ERR_ARG;
+    if (nsamples < 1 || !dims || !x || !target || !w || iters < 0 || batch < 1 || !grid_ok(dims)) return EKL_ERR_ARG;
     NetWork W;
     W.g = make_grid(dims, periodic);
     const int N = W.g.N;
-    const long long fit = N > 0 ? NET_PASS_NODES / N : 1;
+    const long long fit = NET_PASS_NODES / N;
     const int group = (int)(fit < 1 ? 1 : fit < batch ? fit : batch);
     size_t off = 0;
     auto carve = [&](size_t bytes) {
