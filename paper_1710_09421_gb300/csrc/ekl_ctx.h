@@ -4,6 +4,7 @@
 #include <stdint.h>
 
 #include "../../include/ekl.h"
+#include "ekl_smem.h"
 
 namespace ekl {
 

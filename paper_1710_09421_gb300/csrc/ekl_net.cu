@@ -23,7 +23,6 @@
 #include <stdint.h>
 #include <string.h>
 
-#include <mutex>
 #include <vector>
 
 #include <new>
@@ -347,7 +346,6 @@ __device__ __forceinline__ int tile_node(const NetGrid &g, const NetTile &T, con
 // What bounds it: staging.  With a copy of the rows per offset (27 x 4 KB a
 // block, one block per SM) a 65 536-node layer took 45 us, now 11 us.
 constexpr int TC_B_BYTES = 16 * 32;             // one offset's B tile
-constexpr int TC_SMEM_MOST = 72 * 1024;          // above any tile shape's (55 KB at most)
 constexpr int TC_COLS = TL_Z * 16;              // TMEM columns (a power of two, at least 32)
 
 __device__ int tc_status;  // nonzero after a bounded wait gave up
@@ -379,6 +377,8 @@ __device__ __forceinline__ uint32_t tc_wait(uint64_t *mbar)
     return done;
 }
 
+// at most 42 560 bytes (tiles of 30 x 4 nodes): with the kernels' static shared
+// memory still within the 48 KB of any launch
 inline size_t tc_smem(const NetTile &T) { return (size_t)T.rows * 32 + K27 * TC_B_BYTES + 64; }
 
 template <bool RELU>
@@ -496,10 +496,6 @@ void conv16(const NetGrid &g, const __nv_bfloat16 *in, const __nv_bfloat16 *Wt, 
 {
     if (g_tensor_path) {
         const NetTile T = make_tile(g);
-        static std::once_flag attr;  // the largest tile of any grid
-        std::call_once(attr, [] {
-            cudaFuncSetAttribute(conv16_tc<RELU>, cudaFuncAttributeMaxDynamicSharedMemorySize, TC_SMEM_MOST);
-        });
         const int blocks = T.ntx * T.nty * T.ntz * (g.total / g.N);
         conv16_tc<RELU><<<blocks, TL_T, tc_smem(T), s>>>(g, T, in, Wt, bias, flip, out, relu_mask_src);
     } else {
@@ -839,6 +835,14 @@ struct NetWork {
 
 int cuda_err(cudaError_t e) { return e == cudaSuccess ? EKL_OK : EKL_ERR_CUDA; }
 
+// the weight-gradient kernels that need more than 48 KB, before every call that trains
+cudaError_t wgrad_opt_in()
+{
+    static_assert(wg_smem<2, 16>() <= SMEM_DEFAULT, "needs no opt-in");
+    const cudaError_t e = smem_opt_in((const void *)wgrad_k<16, 1>, wg_smem<16, 1>());
+    return e == cudaSuccess ? smem_opt_in((const void *)wgrad_k<16, 16>, wg_smem<16, 16>()) : e;
+}
+
 constexpr int LAYER_PARAMS[4] = {OW2 - OW1, OW3 - OW2, OW4 - OW3, NPARAM - OW4};
 
 // buffers for passes over `samples` samples of W.g; `extra` bytes more
@@ -919,18 +923,12 @@ void net_forward(NetWork &W, const NetInput &in, int ns, cudaStream_t s)
     conv16<true>(g, W.a1, W.W2f, W.w + OB2, 0, W.a2, nullptr, s);
     conv16<true>(g, W.a2, W.W3f, W.w + OB3, 0, W.a3, nullptr, s);
     const NetTile T = make_tile(g);
-    static std::once_flag attr;
-    std::call_once(attr, [] { cudaFuncSetAttribute(l4_fwd, cudaFuncAttributeMaxDynamicSharedMemorySize, TC_SMEM_MOST); });
     l4_fwd<<<T.ntx * T.nty * T.ntz * ns, TL_T, tc_smem(T), s>>>(g, T, W.a3, W.w, W.y);
 }
 
 template <int CI, int CO>
 void wgrad(const NetGrid &g, const NetInput &in, const __nv_bfloat16 *a, const void *dz, float *part, cudaStream_t s)
 {
-    static std::once_flag attr;
-    std::call_once(attr, [] {
-        cudaFuncSetAttribute(wgrad_k<CI, CO>, cudaFuncAttributeMaxDynamicSharedMemorySize, wg_smem<CI, CO>());
-    });
     const int blocks = (g.N + WG_NODES - 1) / WG_NODES * (g.total / g.N);
     wgrad_k<CI, CO><<<blocks, WG_T, wg_smem<CI, CO>(), s>>>(g, in, a, dz, part);
 }
@@ -1326,7 +1324,8 @@ int ekl_net_eval(const int32_t dims[3], const int32_t periodic[3], const float *
     if (e == cudaSuccess) {
         net_prepare(W, 0);
         net_forward(W, NetInput{W.x, nullptr}, 1, 0);
-        e = cudaMemcpy(y, W.y, (size_t)W.g.N * 4, cudaMemcpyDeviceToHost);
+        e = cudaGetLastError();
+        if (e == cudaSuccess) e = cudaMemcpy(y, W.y, (size_t)W.g.N * 4, cudaMemcpyDeviceToHost);
     }
     work_free(W);
     if (e == cudaSuccess) return tc_check();
@@ -1358,7 +1357,8 @@ int ekl_net_loss_grad(const int32_t dims[3], const int32_t periodic[3], const fl
     uint8_t *dm = mask ? (uint8_t *)(extra + tb) : nullptr;
     const long long cnt = mask_count(mask, N);
     const float inv_cnt = 1.f / (float)(cnt > 0 ? cnt : 1);
-    cudaError_t e = cudaMemcpy(W.x, x, 2 * (size_t)N * 4, cudaMemcpyHostToDevice);
+    cudaError_t e = wgrad_opt_in();
+    if (e == cudaSuccess) e = cudaMemcpy(W.x, x, 2 * (size_t)N * 4, cudaMemcpyHostToDevice);
     if (e == cudaSuccess) e = cudaMemcpy(W.w, w, NPARAM * 4, cudaMemcpyHostToDevice);
     if (e == cudaSuccess) e = cudaMemcpy(dt, target, (size_t)N * 4, cudaMemcpyHostToDevice);
     if (e == cudaSuccess && mask) e = cudaMemcpy(dm, mask, N, cudaMemcpyHostToDevice);
@@ -1419,7 +1419,8 @@ int ekl_net_train_grid(int32_t nsamples, const int32_t dims[3], const int32_t pe
     };
     std::vector<int> smp((size_t)iters * batch);
     for (auto &v : smp) v = (int)(next() % (uint64_t)nsamples);
-    cudaError_t e = cudaMemcpy(dx, x, (size_t)nsamples * 2 * N * 4, cudaMemcpyHostToDevice);
+    cudaError_t e = wgrad_opt_in();
+    if (e == cudaSuccess) e = cudaMemcpy(dx, x, (size_t)nsamples * 2 * N * 4, cudaMemcpyHostToDevice);
     if (e == cudaSuccess) e = cudaMemcpy(dt, target, (size_t)nsamples * N * 4, cudaMemcpyHostToDevice);
     if (e == cudaSuccess && mask) e = cudaMemcpy(dm, mask, N, cudaMemcpyHostToDevice);
     if (e == cudaSuccess) e = cudaMemcpy(W.w, w, NPARAM * 4, cudaMemcpyHostToDevice);
