@@ -1742,12 +1742,12 @@ static_assert(3 * MD_BLOCKS <= 32, "a warp hands a position to every block at on
 template <typename R> struct MdPos { typedef long long type; };
 template <> struct MdPos<double> { typedef double type; };
 
-__host__ __device__ inline int md_per_block(int nb) { return (nb + MD_BLOCKS - 1) / MD_BLOCKS; }
+__host__ __device__ constexpr int md_per_block(int nb) { return (nb + MD_BLOCKS - 1) / MD_BLOCKS; }
 
 // per bead of the chain: two copies of its position in P and in FP32, its
 // chain id, its two-step drag; per bead of the block: velocity, u^a, grad phi,
 // gamma, local position, block origin, scan box, wall flags
-template <typename R> inline size_t md_smem_bytes(int nb)
+template <typename R> constexpr size_t md_smem_bytes(int nb)
 {
     const size_t all = (size_t)nb * (6 * sizeof(double) + 6 * sizeof(float) + sizeof(int));
     const size_t own = (size_t)md_per_block(nb) * (29 * sizeof(R) + 9 * sizeof(int) + WALL_WORDS * sizeof(uint32_t));

@@ -226,9 +226,9 @@ template <typename PhiT> static cudaError_t mgs_build(Ctx &c, const MgArgs &m0, 
         e = cudaGraphAddNode(&nloop, gr, &ninit, nullptr, 1, &cp);
         if (e == cudaSuccess) body = cp.conditional.phGraph_out[0];
     }
-    if (e == cudaSuccess && c.mg_smem > 48 * 1024)
-        e = cudaFuncSetAttribute(c.mg_wide ? mgs_coarse_kernel<MG_WIDE_THREADS> : mgs_coarse_kernel<MG_THREADS>,
-                                 cudaFuncAttributeMaxDynamicSharedMemorySize, (int)c.mg_smem);
+    if (e == cudaSuccess)
+        e = smem_opt_in(c.mg_wide ? (const void *)mgs_coarse_kernel<MG_WIDE_THREADS>
+                                  : (const void *)mgs_coarse_kernel<MG_THREADS>, c.mg_smem);
     if (e == cudaSuccess) e = cudaStreamCreateWithFlags(&cs, cudaStreamNonBlocking);
     if (e == cudaSuccess) e = cudaStreamBeginCaptureToGraph(cs, body, nullptr, nullptr, 0, cudaStreamCaptureModeRelaxed);
     if (e == cudaSuccess) {
@@ -259,7 +259,7 @@ template <typename PhiT> static cudaError_t mgs_build(Ctx &c, const MgArgs &m0, 
                       m.lev[1].f, m.lev[1].e, m.lev[1].sig, m.lev[1].nx, m.lev[1].ny, m.lev[1].nz};
             auto launch = [&](auto kern) {
                 const size_t smem = mgf_smem<MODE>(G, V);
-                cudaError_t r = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+                cudaError_t r = smem_opt_in((const void *)kern, smem);
                 cudaLaunchConfig_t lc = {};
                 lc.gridDim = dim3(G.ntx * G.nty * G.ntz);
                 lc.blockDim = dim3(mgf_threads(G));
@@ -433,30 +433,23 @@ template <typename S, typename R, typename PhiT, bool DEV> int steps_impl(Ctx &c
             void *args[] = {&a, &m};
             const void *kern = c.mg_wide ? (const void *)poisson_mg_wide_kernel<S, R, PhiT>
                                          : (const void *)poisson_mg_kernel<S, R, PhiT>;
-            static size_t attr_bytes[2] = {0, 0};
-            if (c.mg_smem > attr_bytes[c.mg_wide]) {
-                cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)c.mg_smem);
-                attr_bytes[c.mg_wide] = c.mg_smem;
-            }
-            cudaError_t e = cudaLaunchCooperativeKernel(kern, dim3(c.pois_blocks),
-                                                        dim3(c.mg_wide ? MG_WIDE_THREADS : MG_THREADS), args,
-                                                        c.mg_smem, c.stream);
+            cudaError_t e = smem_opt_in(kern, c.mg_smem);
+            if (e == cudaSuccess)
+                e = cudaLaunchCooperativeKernel(kern, dim3(c.pois_blocks),
+                                                dim3(c.mg_wide ? MG_WIDE_THREADS : MG_THREADS), args, c.mg_smem,
+                                                c.stream);
             c.launches++;
             if (e != cudaSuccess) return EKL_ERR_CUDA;
             c.mg_have_prev = 1;
         } else if (c.pois_tiled) {
             TileGeom tg{c.tile_ty, c.tile_tz, c.tile_nty, c.tile_ntz};
             const size_t smem = tile_smem_bytes<PhiT>(c.nx, tg);
-            static size_t attr_bytes = 0;
-            if (smem > attr_bytes) {
-                cudaFuncSetAttribute(poisson_tiled_kernel<S, R, PhiT>,
-                                     cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-                attr_bytes = smem;
-            }
             void *args[] = {&a, &tg};
-            cudaError_t e = cudaLaunchCooperativeKernel((const void *)poisson_tiled_kernel<S, R, PhiT>,
-                                                        dim3(c.tile_nty * c.tile_ntz), dim3(POIS_THREADS),
-                                                        args, smem, c.stream);
+            const void *kern = (const void *)poisson_tiled_kernel<S, R, PhiT>;
+            cudaError_t e = smem_opt_in(kern, smem);
+            if (e == cudaSuccess)
+                e = cudaLaunchCooperativeKernel(kern, dim3(c.tile_nty * c.tile_ntz), dim3(POIS_THREADS), args, smem,
+                                                c.stream);
             c.launches++;
             if (e != cudaSuccess) return EKL_ERR_CUDA;
         } else {
@@ -476,12 +469,7 @@ template <typename S, typename R, typename PhiT, bool DEV> int steps_impl(Ctx &c
         phase_begin(c, PH_MD);
         if (c.nb > 0) {
             MdArgs<S, R, PhiT, DEV> md = make_md_args<S, R, PhiT, DEV>(c, a, ba);
-            static bool attr_set = false;
-            if (!attr_set) {
-                cudaFuncSetAttribute(bead_md_kernel<S, R, PhiT, DEV>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                     (int)md_smem_bytes<R>(MAX_BEADS));
-                attr_set = true;
-            }
+            static_assert(md_smem_bytes<R>(MAX_BEADS) <= SMEM_DEFAULT, "needs no opt-in");
             bead_md_kernel<S, R, PhiT, DEV><<<MD_BLOCKS, MD_THREADS, md_smem_bytes<R>(c.nb), c.stream>>>(md);
             c.launches++;
         }
@@ -637,10 +625,8 @@ template <typename S, typename R, typename PhiT, bool DEV> int batch_tables(Batc
         // over 512 threads; factor 1 keeps the cooperative solve's blocks and
         // results)
         int occ = 0;
-        if (B.mg_smem > 48 * 1024)
-            cudaFuncSetAttribute(mgsb_coarse_kernel<S, R, PhiT>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                 (int)B.mg_smem);
-        if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, mgsb_coarse_kernel<S, R, PhiT>, MGS_THREADS / 2,
+        if (smem_opt_in((const void *)mgsb_coarse_kernel<S, R, PhiT>, B.mg_smem) != cudaSuccess ||
+            cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, mgsb_coarse_kernel<S, R, PhiT>, MGS_THREADS / 2,
                                                           B.mg_smem) != cudaSuccess)
             occ = 0;
         cudaGetLastError();
@@ -734,9 +720,7 @@ template <typename S, typename R, typename PhiT> static cudaError_t mgsb_build(B
         e = cudaGraphAddNode(&nloop, G, &ncond, nullptr, 1, &cp);
         if (e == cudaSuccess) body = cp.conditional.phGraph_out[0];
     }
-    if (e == cudaSuccess && B.mg_smem > 48 * 1024)
-        e = cudaFuncSetAttribute(mgsb_coarse_kernel<S, R, PhiT>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                 (int)B.mg_smem);
+    if (e == cudaSuccess) e = smem_opt_in((const void *)mgsb_coarse_kernel<S, R, PhiT>, B.mg_smem);
     if (e == cudaSuccess) e = cudaStreamCreateWithFlags(&cs, cudaStreamNonBlocking);
     if (e == cudaSuccess) e = cudaStreamBeginCaptureToGraph(cs, body, nullptr, nullptr, 0, cudaStreamCaptureModeRelaxed);
     if (e == cudaSuccess) {
@@ -758,7 +742,7 @@ template <typename S, typename R, typename PhiT> static cudaError_t mgsb_build(B
             constexpr int MODE = decltype(mode)::value;
             const size_t smem = (MODE == MGF_RESTR ? 7 : 4) * (size_t)B.mgf_plane * sizeof(float);
             auto launch = [&](auto kern) {
-                cudaError_t r = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+                cudaError_t r = smem_opt_in((const void *)kern, smem);
                 cudaLaunchConfig_t lc = {};
                 lc.gridDim = dim3(B.mgf_grid);
                 lc.blockDim = dim3(B.mgf_threads);
@@ -867,12 +851,6 @@ template <typename S, typename R, typename PhiT, bool DEV> int batch_impl(Batch 
             const StepArgs<S, R, PhiT> *reps = (const StepArgs<S, R, PhiT> *)B.d_args[q];
             const MgArgs *mgs = (const MgArgs *)B.d_mgargs;
             unsigned *bars = B.mg_bars;
-            static size_t attr_bytes = 0;
-            if (B.mg_smem > attr_bytes) {
-                cudaFuncSetAttribute(poisson_mg_batch_kernel<S, R, PhiT>,
-                                     cudaFuncAttributeMaxDynamicSharedMemorySize, (int)B.mg_smem);
-                attr_bytes = B.mg_smem;
-            }
             if (B.mgs_split) {
                 static_assert(MGS_THREADS == MG_BATCH_THREADS, "split and cooperative batch solves share the grid");
                 if (B.mgs_exec && (B.mgs_blocks != B.mgs_lblocks || B.mgs_cblocks != B.mgs_cgrid)) {
@@ -891,9 +869,11 @@ template <typename S, typename R, typename PhiT, bool DEV> int batch_impl(Batch 
                 B.launches += 6;  // start, residual, init, condition, final residual, report
             } else {
                 void *args[] = {&reps, &mgs, &pb, &bars};
-                cudaError_t e = cudaLaunchCooperativeKernel((const void *)poisson_mg_batch_kernel<S, R, PhiT>,
-                                                            dim3(B.pois_blocks), dim3(MG_BATCH_THREADS), args,
-                                                            B.mg_smem, B.stream);
+                const void *kern = (const void *)poisson_mg_batch_kernel<S, R, PhiT>;
+                cudaError_t e = smem_opt_in(kern, B.mg_smem);
+                if (e == cudaSuccess)
+                    e = cudaLaunchCooperativeKernel(kern, dim3(B.pois_blocks), dim3(MG_BATCH_THREADS), args,
+                                                    B.mg_smem, B.stream);
                 B.launches++;
                 if (e != cudaSuccess) return EKL_ERR_CUDA;
             }
@@ -915,14 +895,8 @@ template <typename S, typename R, typename PhiT, bool DEV> int batch_impl(Batch 
             if (e != cudaSuccess) return EKL_ERR_CUDA;
         }
         if (B.max_nb > 0) {
-            static size_t attr = 0;
-            const size_t smem = md_smem_bytes<R>(B.max_nb);
-            if (smem > attr) {
-                cudaFuncSetAttribute(bead_md_batch_kernel<S, R, PhiT, DEV>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                     (int)md_smem_bytes<R>(MAX_BEADS));
-                attr = md_smem_bytes<R>(MAX_BEADS);
-            }
-            bead_md_batch_kernel<S, R, PhiT, DEV><<<dim3(MD_BLOCKS, n), MD_THREADS, smem, B.stream>>>(
+            bead_md_batch_kernel<S, R, PhiT, DEV>
+                <<<dim3(MD_BLOCKS, n), MD_THREADS, md_smem_bytes<R>(B.max_nb), B.stream>>>(
                 (const MdArgs<S, R, PhiT, DEV> *)B.d_mdargs[q], step);
             B.launches++;
         }
@@ -947,8 +921,7 @@ template <typename S, typename R, typename PhiT> int mg_max_blocks_per_sm(size_t
 {
     const void *kern = wide ? (const void *)poisson_mg_wide_kernel<S, R, PhiT>
                             : (const void *)poisson_mg_kernel<S, R, PhiT>;
-    if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess)
-        return 0;
+    if (smem_opt_in(kern, smem) != cudaSuccess) return 0;
     int nb = 0;
     cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, kern, wide ? MG_WIDE_THREADS : MG_THREADS, smem);
     return nb;
@@ -956,9 +929,7 @@ template <typename S, typename R, typename PhiT> int mg_max_blocks_per_sm(size_t
 
 template <typename S, typename R, typename PhiT> int mg_batch_max_blocks_per_sm(size_t smem)
 {
-    if (cudaFuncSetAttribute(poisson_mg_batch_kernel<S, R, PhiT>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                             (int)smem) != cudaSuccess)
-        return 0;
+    if (smem_opt_in((const void *)poisson_mg_batch_kernel<S, R, PhiT>, smem) != cudaSuccess) return 0;
     int nb = 0;
     cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, poisson_mg_batch_kernel<S, R, PhiT>, MG_BATCH_THREADS, smem);
     return nb;
