@@ -23,6 +23,9 @@
 #include <stdint.h>
 #include <string.h>
 
+#include <algorithm>
+#include <memory>
+#include <type_traits>
 #include <vector>
 
 #include <new>
@@ -783,12 +786,13 @@ __global__ void __launch_bounds__(WG_T) wgrad_k(NetGrid g, NetInput in, const __
 }
 
 // grad[i] (+)= sum over samples of (sum over the sample's blocks, in order, of
-// part[b][i - first parameter of its layer]), for every parameter
+// part[b][i - first parameter of its layer]), for the parameters first .. end - 1
 __global__ void __launch_bounds__(64) grad_reduce(const float *part1, const float *part2, const float *part3,
-                                                  const float *part4, int per_sample, int ns, int add, float *grad)
+                                                  const float *part4, int per_sample, int ns, int add, float *grad,
+                                                  int first, int end)
 {
-    const int i = blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= NPARAM) return;
+    const int i = first + blockIdx.x * blockDim.x + threadIdx.x;
+    if (i >= end) return;
     const float *p;
     int nw, o;
     if (i < OW2) { p = part1; nw = OW2 - OW1; o = OW1; }
@@ -829,7 +833,7 @@ struct NetWork {
     float *w = nullptr, *grad = nullptr;
     __nv_bfloat16 *W2f = nullptr, *W2b = nullptr, *W3f = nullptr, *W3b = nullptr;
     float *part[4] = {};        // weight-gradient partials per layer
-    double *lpart = nullptr, *loss = nullptr;
+    double *lpart = nullptr;
     void *arena = nullptr;
 };
 
@@ -845,58 +849,59 @@ cudaError_t wgrad_opt_in()
 
 constexpr int LAYER_PARAMS[4] = {OW2 - OW1, OW3 - OW2, OW4 - OW3, NPARAM - OW4};
 
-// buffers for passes over `samples` samples of W.g; `extra` bytes more
-// (256-byte aligned) at *extra_out
-int work_alloc(NetWork &W, int samples, bool train, size_t extra = 0, char **extra_out = nullptr)
+// What a pass needs buffers for: the in-step network and ekl_net_eval read one
+// input and give its output; training keeps the partials of all layers for one
+// reduction, or (TRAIN_TIGHT) reduces layer by layer through one buffer, so that
+// a pass over one sample needs no more than a layer's partials at a time.
+enum NetUse { NET_EVAL, NET_TRAIN, NET_TRAIN_TIGHT };
+
+// The buffers for passes over `samples` samples of W.g (and `input`: one sample's
+// input at W.x) out of `base`; returns their bytes (base null: only that).
+size_t work_layout(NetWork &W, NetUse use, int samples, bool input, char *base)
 {
     size_t off = 0;
-    auto carve = [&](size_t bytes) {
-        const size_t at = off;
+    auto carve = [&](auto *&p, size_t bytes) {
+        p = base ? (std::remove_reference_t<decltype(p)>)(base + off) : nullptr;
         off += (bytes + 255) & ~(size_t)255;
-        return at;
     };
     const size_t n = (size_t)samples * W.g.N;
-    const size_t ox = carve(2 * n * 4), o1 = carve(n * 32), o2 = carve(n * 32), o3 = carve(n * 32), oy = carve(n * 4);
-    const size_t ow = carve(NPARAM * 4), of2 = carve(27 * 512), ob2 = carve(27 * 512), of3 = carve(27 * 512),
-                 ob3 = carve(27 * 512);
-    size_t od = 0, od2 = 0, og = 0, ogr = 0, ol = 0, op[4] = {}, oloss = 0;
-    if (train) {
-        od = carve(n * 32);
-        od2 = carve(n * 32);
-        og = carve(n * 4);
-        ogr = carve(NPARAM * 4);
-        ol = carve(((n + NT - 1) / NT) * sizeof(double));
-        oloss = carve(sizeof(double));
-        const size_t nb = (size_t)samples * ((W.g.N + WG_NODES - 1) / WG_NODES);
-        for (int l = 0; l < 4; l++) op[l] = carve(nb * LAYER_PARAMS[l] * 4);
+    if (input) carve(W.x, 2 * (size_t)W.g.N * 4);
+    carve(W.a1, n * 32);
+    carve(W.a2, n * 32);
+    carve(W.a3, n * 32);
+    carve(W.y, n * 4);
+    carve(W.w, NPARAM * 4);
+    carve(W.W2f, 27 * 512);
+    carve(W.W2b, 27 * 512);
+    carve(W.W3f, 27 * 512);
+    carve(W.W3b, 27 * 512);
+    if (use == NET_EVAL) return off;
+    carve(W.dz, n * 32);
+    carve(W.dz2, n * 32);
+    carve(W.gy, n * 4);
+    carve(W.grad, NPARAM * 4);
+    carve(W.lpart, ((n + NT - 1) / NT) * sizeof(double));
+    const size_t nb = (size_t)samples * ((W.g.N + WG_NODES - 1) / WG_NODES);
+    if (use == NET_TRAIN_TIGHT) {
+        carve(W.part[0], nb * *std::max_element(LAYER_PARAMS, LAYER_PARAMS + 4) * 4);
+        for (int l = 1; l < 4; l++) W.part[l] = W.part[0];
+    } else {
+        for (int l = 0; l < 4; l++) carve(W.part[l], nb * LAYER_PARAMS[l] * 4);
     }
-    const size_t oe = carve(extra);
-    if (cudaMalloc(&W.arena, off) != cudaSuccess) {
+    return off;
+}
+
+// the same, allocated, with `extra` bytes more (256-byte aligned) at *extra_out
+int work_alloc(NetWork &W, NetUse use, int samples, bool input, size_t extra = 0, char **extra_out = nullptr)
+{
+    const size_t bytes = work_layout(W, use, samples, input, nullptr);
+    if (cudaMalloc(&W.arena, bytes + extra) != cudaSuccess) {
         cudaGetLastError();
         W.arena = nullptr;
         return EKL_ERR_ALLOC;
     }
-    char *b = (char *)W.arena;
-    W.x = (float *)(b + ox);
-    W.a1 = (__nv_bfloat16 *)(b + o1);
-    W.a2 = (__nv_bfloat16 *)(b + o2);
-    W.a3 = (__nv_bfloat16 *)(b + o3);
-    W.y = (float *)(b + oy);
-    W.w = (float *)(b + ow);
-    W.W2f = (__nv_bfloat16 *)(b + of2);
-    W.W2b = (__nv_bfloat16 *)(b + ob2);
-    W.W3f = (__nv_bfloat16 *)(b + of3);
-    W.W3b = (__nv_bfloat16 *)(b + ob3);
-    if (train) {
-        W.dz = (__nv_bfloat16 *)(b + od);
-        W.dz2 = (__nv_bfloat16 *)(b + od2);
-        W.gy = (float *)(b + og);
-        W.grad = (float *)(b + ogr);
-        W.lpart = (double *)(b + ol);
-        W.loss = (double *)(b + oloss);
-        for (int l = 0; l < 4; l++) W.part[l] = (float *)(b + op[l]);
-    }
-    if (extra_out) *extra_out = b + oe;
+    work_layout(W, use, samples, input, (char *)W.arena);
+    if (extra_out) *extra_out = (char *)W.arena + bytes;
     return EKL_OK;
 }
 
@@ -942,18 +947,26 @@ void net_backward(NetWork &W, const NetInput &in, int ns, const float *d_t, cons
     const NetGrid &g = W.g;
     const int bn = (g.total + NT - 1) / NT;
     const int per = (g.N + WG_NODES - 1) / WG_NODES;
+    const bool tight = W.part[0] == W.part[1];
+    auto reduce = [&](int first, int end) {
+        grad_reduce<<<(end - first + 63) / 64, 64, 0, s>>>(W.part[0], W.part[1], W.part[2], W.part[3], per, ns,
+                                                          add ? 1 : 0, W.grad, first, end);
+    };
     loss_grad_k<<<bn, NT, 0, s>>>(g, W.y, d_t, in.smp, d_mask, inv_cnt, W.gy, W.lpart);
     loss_sum_k<<<1, NT, 0, s>>>(W.lpart, bn, loss_scale, add ? 1 : 0, d_loss);
     wgrad<16, 1>(g, in, W.a3, W.gy, W.part[3], s);
+    if (tight) reduce(OW4, NPARAM);
     l4_bwd_data<<<bn, NT, 0, s>>>(g, W.gy, W.w, W.a3, W.dz);
     // dz holds d z3 (through relu of a3)
     wgrad<16, 16>(g, in, W.a2, W.dz, W.part[2], s);
+    if (tight) reduce(OW3, OW4);
     conv16<false>(g, W.dz, W.W3b, nullptr, 1, W.dz2, W.a2, s);
     wgrad<16, 16>(g, in, W.a1, W.dz2, W.part[1], s);
+    if (tight) reduce(OW2, OW3);
     conv16<false>(g, W.dz2, W.W2b, nullptr, 1, W.dz, W.a1, s);
     wgrad<2, 16>(g, in, nullptr, W.dz, W.part[0], s);
-    grad_reduce<<<(NPARAM + 63) / 64, 64, 0, s>>>(W.part[0], W.part[1], W.part[2], W.part[3], per, ns, add ? 1 : 0,
-                                                  W.grad);
+    if (tight) reduce(OW1, OW2);
+    else reduce(0, NPARAM);
 }
 
 // Extents that the kernels' 32-bit node ids (up to 2 N, the second input
@@ -1273,7 +1286,7 @@ static int warmstart_ensure(Ctx &c, int level = -1)
     const int32_t cdims[3] = {c.nx >> level, c.ny >> level, c.nz >> level};
     ws->W.g = make_grid(cdims, c.per);
     const int N = (int)c.N;
-    int rc = work_alloc(ws->W, 1, false);
+    int rc = work_alloc(ws->W, NET_EVAL, 1, true);
     cudaError_t e = rc == EKL_OK ? cudaSuccess : cudaErrorMemoryAllocation;
     if (e == cudaSuccess) e = cudaMalloc(&ws->bprev, (size_t)N * 4);
     if (e == cudaSuccess) e = cudaMalloc(&ws->bcur, (size_t)N * 4);
@@ -1317,7 +1330,7 @@ int ekl_net_eval(const int32_t dims[3], const int32_t periodic[3], const float *
     if (!dims || !x || !w || !y || !grid_ok(dims)) return EKL_ERR_ARG;
     NetWork W;
     W.g = make_grid(dims, periodic);
-    int rc = work_alloc(W, 1, false);
+    int rc = work_alloc(W, NET_EVAL, 1, true);
     if (rc != EKL_OK) return rc;
     cudaError_t e = cudaMemcpy(W.x, x, 2 * (size_t)W.g.N * 4, cudaMemcpyHostToDevice);
     if (e == cudaSuccess) e = cudaMemcpy(W.w, w, NPARAM * 4, cudaMemcpyHostToDevice);
@@ -1351,10 +1364,13 @@ int ekl_net_loss_grad(const int32_t dims[3], const int32_t periodic[3], const fl
     const int N = W.g.N;
     char *extra = nullptr;
     const size_t tb = ((size_t)N * 4 + 255) & ~(size_t)255;
-    int rc = work_alloc(W, 1, true, tb + (size_t)N, &extra);
+    const size_t more = tb + 256 + (mask ? (size_t)N : 0);
+    int rc = work_alloc(W, NET_TRAIN, 1, true, more, &extra);
+    if (rc != EKL_OK) rc = work_alloc(W, NET_TRAIN_TIGHT, 1, true, more, &extra);
     if (rc != EKL_OK) return rc;
     float *dt = (float *)extra;
-    uint8_t *dm = mask ? (uint8_t *)(extra + tb) : nullptr;
+    double *dloss = (double *)(extra + tb);
+    uint8_t *dm = mask ? (uint8_t *)(extra + tb + 256) : nullptr;
     const long long cnt = mask_count(mask, N);
     const float inv_cnt = 1.f / (float)(cnt > 0 ? cnt : 1);
     cudaError_t e = wgrad_opt_in();
@@ -1366,9 +1382,9 @@ int ekl_net_loss_grad(const int32_t dims[3], const int32_t periodic[3], const fl
         const NetInput in{W.x, nullptr};
         net_prepare(W, 0);
         net_forward(W, in, 1, 0);
-        net_backward(W, in, 1, dt, dm, inv_cnt, false, (double)inv_cnt, W.loss, 0);
+        net_backward(W, in, 1, dt, dm, inv_cnt, false, (double)inv_cnt, dloss, 0);
         e = cudaGetLastError();
-        if (e == cudaSuccess && loss) e = cudaMemcpy(loss, W.loss, sizeof(double), cudaMemcpyDeviceToHost);
+        if (e == cudaSuccess && loss) e = cudaMemcpy(loss, dloss, sizeof(double), cudaMemcpyDeviceToHost);
         if (e == cudaSuccess) e = cudaMemcpy(grad, W.grad, NPARAM * 4, cudaMemcpyDeviceToHost);
     }
     work_free(W);
@@ -1376,81 +1392,137 @@ int ekl_net_loss_grad(const int32_t dims[3], const int32_t periodic[3], const fl
     return cuda_err(e);
 }
 
-// Nodes of one training pass: the samples of a batch go through the network
-// together as long as their buffers stay under about 4 GB (250 bytes a
-// node), else in several passes whose gradients add up.
-static constexpr long long NET_PASS_NODES = 16ll << 20;
+// Device memory for the buffers of one training pass.  The samples of a batch go
+// through the network together as long as their buffers stay under it (168 bytes
+// a node, and 61 KB of weight-gradient partials per sample and 512 nodes of it), else
+// in several passes whose gradients add up.  Where the device has less to give,
+// passes of half as many samples are tried, and at last one sample with the
+// partials of one layer at a time.
+static constexpr uint64_t NET_PASS_BYTES = 4ull << 30;
+// sample numbers and losses that are on the device at a time
+static constexpr int NET_DRAWS = 4096, NET_LOSSES = 512;
 
-int ekl_net_train_grid(int32_t nsamples, const int32_t dims[3], const int32_t periodic[3], const float *x,
-                       const float *target, const uint8_t *mask, float *w, int32_t iters, int32_t batch, float lr,
-                       uint64_t seed, float *loss_out)
+static int train_grid(int32_t nsamples, const int32_t dims[3], const int32_t periodic[3], const float *x,
+                      const float *target, const uint8_t *mask, float *w, int32_t iters, int32_t batch, float lr,
+                      uint64_t seed, float *loss_out, uint64_t pass_bytes)
 {
     if (nsamples < 1 || !dims || !x || !target || !w || iters < 0 || batch < 1 || !grid_ok(dims)) return EKL_ERR_ARG;
     NetWork W;
     W.g = make_grid(dims, periodic);
     const int N = W.g.N;
-    const long long fit = NET_PASS_NODES / N;
-    const int group = (int)(fit < 1 ? 1 : fit < batch ? fit : batch);
-    size_t off = 0;
-    auto carve = [&](size_t bytes) {
-        const size_t at = off;
-        off += (bytes + 255) & ~(size_t)255;
-        return at;
-    };
-    const size_t ox = carve((size_t)nsamples * 2 * N * 4), ot = carve((size_t)nsamples * N * 4), o1 = carve(NPARAM * 4),
-                 o2 = carve(NPARAM * 4), om = carve((size_t)N), os = carve((size_t)iters * batch * sizeof(int)),
-                 ol = carve((size_t)iters * sizeof(double));
-    char *ex = nullptr;
-    int rc = work_alloc(W, group, true, off, &ex);
-    if (rc != EKL_OK) return rc;
-    float *dx = (float *)(ex + ox), *dt = (float *)(ex + ot), *m1 = (float *)(ex + o1), *m2 = (float *)(ex + o2);
-    uint8_t *dm = mask ? (uint8_t *)(ex + om) : nullptr;
-    int *dsmp = (int *)(ex + os);
-    double *dloss = (double *)(ex + ol);
+    const size_t one = work_layout(W, NET_TRAIN, 1, false, nullptr);
+    const size_t next = work_layout(W, NET_TRAIN, 2, false, nullptr) - one;  // bytes of one more sample
+    const uint64_t fit = std::min<uint64_t>(pass_bytes / next, (1u << 30) / (unsigned)N);
+    int group = (int)std::max<uint64_t>(1, std::min<uint64_t>(fit, (uint64_t)batch));
+    NetUse use = pass_bytes ? NET_TRAIN : NET_TRAIN_TIGHT;
+    const int64_t total = (int64_t)iters * batch;
+    float *dx, *dt, *m1, *m2;
+    uint8_t *dm = nullptr;
+    int *dsmp, draws;
+    double *dloss;
+    for (;;) {
+        draws = (int)std::max<int64_t>(group, std::min<int64_t>(total, NET_DRAWS));
+        char *base = nullptr;
+        size_t off = 0;
+        auto carve = [&](auto *&p, size_t bytes) {
+            p = (std::remove_reference_t<decltype(p)>)(base ? base + off : nullptr);
+            off += (bytes + 255) & ~(size_t)255;
+        };
+        auto layout = [&] {
+            off = 0;
+            carve(dx, (size_t)nsamples * 2 * N * 4);
+            carve(dt, (size_t)nsamples * N * 4);
+            carve(m1, NPARAM * 4);
+            carve(m2, NPARAM * 4);
+            carve(dsmp, (size_t)draws * sizeof(int));
+            carve(dloss, NET_LOSSES * sizeof(double));
+            if (mask) carve(dm, (size_t)N);
+        };
+        layout();
+        const int rc = work_alloc(W, use, group, false, off, &base);
+        if (rc == EKL_OK) {
+            layout();
+            break;
+        }
+        if (group > 1) group = (group + 1) / 2;
+        else if (use == NET_TRAIN) use = NET_TRAIN_TIGHT;
+        else return rc;
+    }
+    std::unique_ptr<int[]> smp(new (std::nothrow) int[draws]);
+    if (!smp) {
+        work_free(W);
+        return EKL_ERR_ALLOC;
+    }
     const long long cnt = mask_count(mask, N);
-    // seeded sample order (splitmix64)
+    // seeded sample order (splitmix64), drawn and uploaded `draws` at a time
     uint64_t st = seed;
-    auto next = [&]() {
+    auto next_draw = [&]() {
         st += 0x9E3779B97F4A7C15ull;
         uint64_t z = st;
         z = (z ^ (z >> 30)) * 0xBF58476D1CE4E5B9ull;
         z = (z ^ (z >> 27)) * 0x94D049BB133111EBull;
         return z ^ (z >> 31);
     };
-    std::vector<int> smp((size_t)iters * batch);
-    for (auto &v : smp) v = (int)(next() % (uint64_t)nsamples);
+    int64_t drawn = 0;
+    int at = 0, have = 0;  // the next sample's place and the number uploaded
+    auto refill = [&] {    // (the copy follows the passes that read the last ones)
+        std::copy(smp.get() + at, smp.get() + have, smp.get());
+        have -= at;
+        at = 0;
+        for (; have < draws && drawn < total; have++, drawn++) smp[have] = (int)(next_draw() % (uint64_t)nsamples);
+        return cudaMemcpy(dsmp, smp.get(), (size_t)have * sizeof(int), cudaMemcpyHostToDevice);
+    };
     cudaError_t e = wgrad_opt_in();
     if (e == cudaSuccess) e = cudaMemcpy(dx, x, (size_t)nsamples * 2 * N * 4, cudaMemcpyHostToDevice);
     if (e == cudaSuccess) e = cudaMemcpy(dt, target, (size_t)nsamples * N * 4, cudaMemcpyHostToDevice);
     if (e == cudaSuccess && mask) e = cudaMemcpy(dm, mask, N, cudaMemcpyHostToDevice);
     if (e == cudaSuccess) e = cudaMemcpy(W.w, w, NPARAM * 4, cudaMemcpyHostToDevice);
-    if (e == cudaSuccess && !smp.empty())
-        e = cudaMemcpy(dsmp, smp.data(), smp.size() * sizeof(int), cudaMemcpyHostToDevice);
     if (e == cudaSuccess) e = cudaMemset(m1, 0, NPARAM * 4);
     if (e == cudaSuccess) e = cudaMemset(m2, 0, NPARAM * 4);
     const float b1 = 0.9f, b2 = 0.999f, eps = 1e-8f;
     const float inv_cnt = 1.f / (float)(cnt * batch);
+    double losses[NET_LOSSES];
     for (int it = 0; it < iters && e == cudaSuccess; it++) {
         net_prepare(W, 0);
-        for (int k = 0; k < batch; k += group) {
-            const int ns = batch - k < group ? batch - k : group;
-            const NetInput in{dx, dsmp + (size_t)it * batch + k};
+        for (int64_t k = 0; k < batch; k += group) {
+            const int ns = (int)std::min<int64_t>(batch - k, group);
+            if (have - at < ns) e = refill();
+            if (e != cudaSuccess) break;
+            const NetInput in{dx, dsmp + at};
             net_forward(W, in, ns, 0);
-            net_backward(W, in, ns, dt, dm, inv_cnt, k > 0, (double)inv_cnt, dloss + it, 0);
+            net_backward(W, in, ns, dt, dm, inv_cnt, k > 0, (double)inv_cnt, dloss + it % NET_LOSSES, 0);
+            at += ns;
         }
         const float c1 = 1.f - powf(b1, (float)(it + 1)), c2 = 1.f - powf(b2, (float)(it + 1));
         adam_k<<<(NPARAM + 255) / 256, 256>>>(NPARAM, W.w, W.grad, m1, m2, lr, b1, b2, eps, c1, c2);
-        e = cudaGetLastError();
+        if (e == cudaSuccess) e = cudaGetLastError();
+        const int filled = it % NET_LOSSES + 1;
+        if (e == cudaSuccess && loss_out && (filled == NET_LOSSES || it + 1 == iters)) {
+            e = cudaMemcpy(losses, dloss, (size_t)filled * sizeof(double), cudaMemcpyDeviceToHost);
+            for (int k = 0; k < filled; k++) loss_out[it + 1 - filled + k] = (float)losses[k];
+        }
     }
     if (e == cudaSuccess) e = cudaMemcpy(w, W.w, NPARAM * 4, cudaMemcpyDeviceToHost);
-    if (e == cudaSuccess && loss_out && iters > 0) {
-        std::vector<double> l(iters);
-        e = cudaMemcpy(l.data(), dloss, (size_t)iters * sizeof(double), cudaMemcpyDeviceToHost);
-        for (int it = 0; it < iters; it++) loss_out[it] = (float)l[it];
-    }
     work_free(W);
     if (e == cudaSuccess) return tc_check();
     return cuda_err(e);
+}
+
+int ekl_net_train_grid(int32_t nsamples, const int32_t dims[3], const int32_t periodic[3], const float *x,
+                       const float *target, const uint8_t *mask, float *w, int32_t iters, int32_t batch, float lr,
+                       uint64_t seed, float *loss_out)
+{
+    return train_grid(nsamples, dims, periodic, x, target, mask, w, iters, batch, lr, seed, loss_out, NET_PASS_BYTES);
+}
+
+// ekl_net_train_grid in passes of at most pass_bytes (at least one sample; 0: one
+// sample and the partials of one layer at a time): the splits that a large batch or
+// a nearly full device leads to, for the tests; not part of the interface
+int ekl_net_train_in_passes(int32_t nsamples, const int32_t dims[3], const int32_t periodic[3], const float *x,
+                            const float *target, const uint8_t *mask, float *w, int32_t iters, int32_t batch,
+                            float lr, uint64_t seed, float *loss_out, uint64_t pass_bytes)
+{
+    return train_grid(nsamples, dims, periodic, x, target, mask, w, iters, batch, lr, seed, loss_out, pass_bytes);
 }
 
 int ekl_net_train(int32_t nsamples, const int32_t dims[3], const float *x, const float *target,
