@@ -533,30 +533,45 @@ __global__ void __launch_bounds__(TL_T) l4_fwd(NetGrid g, NetTile T, const __nv_
     extern __shared__ __align__(1024) uint8_t tc_sm[];
     float *sw = (float *)tc_sm;                              // [offset][channel], then the bias
     uint4 *sA = (uint4 *)(tc_sm + K27 * TC_B_BYTES + 64);    // as in conv16_tc
-    for (int t = threadIdx.x; t < 16 * 27; t += blockDim.x) sw[(t % 27) * 16 + t / 27] = w[OW4 + t];
+    int finite = 1;
+    for (int t = threadIdx.x; t < 16 * 27; t += blockDim.x) {
+        const float v = w[OW4 + t];
+        sw[(t % 27) * 16 + t / 27] = v;
+        finite &= isfinite(v);
+    }
     if (threadIdx.x == 0) sw[16 * 27] = w[OB4];
     const TilePos P = tile_pos(g, T, blockIdx.x);
     tile_stage(g, T, P, act, sA);
-    __syncthreads();
+    finite = __syncthreads_and(finite);
     const int WH = T.W * T.H;
     const int z = threadIdx.x / TC_M, r = threadIdx.x & (TC_M - 1);
     const int n = tile_node(g, T, P, r, z);
-    if (n >= 0) {
-        const int first = 1 + T.W + WH * (z + 1) + r;
-        float acc = sw[16 * 27];
-#pragma unroll 3
-        for (int k = 0; k < K27; k++) {
-            const int row = first + (k % 3 - 1) + T.W * ((k / 3) % 3 - 1) + WH * (k / 9 - 1);
-            const uint4 v[2] = {sA[row], sA[T.rows + row]};
-            const __nv_bfloat162 *a = (const __nv_bfloat162 *)v;
+    if (n < 0) return;
+    const int first = 1 + T.W + WH * (z + 1) + r;
+    auto add = [&](float &acc, int k) {
+        const int row = first + (k % 3 - 1) + T.W * ((k / 3) % 3 - 1) + WH * (k / 9 - 1);
+        const uint4 v[2] = {sA[row], sA[T.rows + row]};
+        const __nv_bfloat162 *a = (const __nv_bfloat162 *)v;
 #pragma unroll
-            for (int c = 0; c < 8; c++) {
-                const float2 f = __bfloat1622float2(a[c]);
-                acc += sw[16 * k + 2 * c] * f.x + sw[16 * k + 2 * c + 1] * f.y;
-            }
+        for (int c = 0; c < 8; c++) {
+            const float2 f = __bfloat1622float2(a[c]);
+            acc += sw[16 * k + 2 * c] * f.x + sw[16 * k + 2 * c + 1] * f.y;
         }
-        y[n] = acc;
+    };
+    float acc = sw[16 * 27];
+    if (finite) {
+#pragma unroll 3
+        for (int k = 0; k < K27; k++) add(acc, k);
+    } else {
+        // zero rows beyond closed faces times a weight that has overflowed
+        // would be NaN: only neighbours on the grid take part
+        int X, Y, Z;
+        xyz_of(g, n - P.base, X, Y, Z);
+#pragma unroll 1
+        for (int k = 0; k < K27; k++)
+            if (nbr_off(g, X, Y, Z, k) >= 0) add(acc, k);
     }
+    y[n] = acc;
 }
 
 // loss gradient g = 2 (y - t) / cnt on masked nodes (target of sample s:
