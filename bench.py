@@ -54,8 +54,8 @@ KERNEL_SOURCES = {
     "lb_fused_kernel": ("ekl_kernels.cuh", "ekl_dev.cuh"),
     "poisson_mg_kernel": ("ekl_mg.cuh", "ekl_kernels.cuh", "ekl_dev.cuh"),
     "poisson_mg_wide_kernel": ("ekl_mg.cuh", "ekl_kernels.cuh", "ekl_dev.cuh"),
-    "multigrid_split_solve": ("ekl_mgs.cuh", "ekl_mg.cuh", "ekl_kernels.cuh", "ekl_dev.cuh"),
-    "poisson_tiled_kernel": ("ekl_kernels.cuh", "ekl_dev.cuh"),
+    "multigrid_split_solve": ("ekl_mgs.cuh", "ekl_mgf.cuh", "ekl_mg.cuh", "ekl_kernels.cuh", "ekl_dev.cuh"),
+    "poisson_tiled_kernel": ("ekl_kernels.cuh", "ekl_rim.h", "ekl_dev.cuh"),
 }
 
 
@@ -163,6 +163,17 @@ def mg_bytes_per_solve(L):
     return (12 + L) + 2 * (22 + L)
 
 
+# The same where the split solve takes two half sweeps per launch (1-byte link
+# array): r (4 B) and the link byte in every pass, and the colour-0 values
+# between passes, 2 B a node: pre-smoothing 5 + 2 written; restriction 5 + 2,
+# and the coarse right-hand side and first values 1; prolongation 5 + 2 + 2 and
+# the coarse correction 0.5; last pass 5 + 2 and z written 4; r.z 9; p/q pass 17;
+# update pass 33 (it no longer starts z); coarse levels 14.  The first residual no
+# longer starts z either.
+MG_FUSED_BYTES_PER_ITER = 7 + 8 + 9.5 + 11 + 9 + 17 + 33 + 14
+MG_FUSED_BYTES_PER_SOLVE = 13 + 21 + 23
+
+
 MG_SPLIT_KERNELS_PER_SOLVE = 5  # start, first true residual, init, final residual, report
 
 
@@ -170,15 +181,25 @@ def mg_split(W, wl, sms=152):
     return bool(wl.flags & W.FLAG_POISSON_MG) and not (wl.flags & W.FLAG_POISSON_MG_SINGLE)
 
 
-def mg_split_kernels_per_iter(wl, sms=152):
-    """Launches per CG iteration of the split solve: 14, plus 8 when level 1
-    is too large for shared-memory tiles (more than 1024 cells per block)."""
+def mg_fused(W, wl, sms=152):
+    """Two half sweeps per launch: lattices whose solve (37 B a node) does not
+    stay in 126 MB of L2, in 1024-thread blocks, with rows of whole groups of four."""
+    return (mg_split(W, wl, sms) and wl.nx % 4 == 0 and wl.n_nodes >= 16384 * sms
+            and wl.n_nodes * 37 > 126 << 20)
+
+
+def mg_split_kernels_per_iter(wl, sms=152, fused=False):
+    """Launches per CG iteration of the split solve: 14, or 11 with two half
+    sweeps per launch, plus 8 when level 1 is too large for shared-memory tiles
+    (more than 1024 cells per block)."""
     level1 = ((wl.nx + 1) // 2) * ((wl.ny + 1) // 2) * ((wl.nz + 1) // 2)
-    return 14 + (8 if level1 > 1024 * sms else 0)
+    return (11 if fused else 14) + (8 if level1 > 1024 * sms else 0)
 
 
-def mg_algorithmic_bytes(wl, iters, link_bytes=4):
+def mg_algorithmic_bytes(wl, iters, link_bytes=4, fused=False):
     nf = int((wl.solid == 0).sum())
+    if fused:
+        return nf * (iters * MG_FUSED_BYTES_PER_ITER + MG_FUSED_BYTES_PER_SOLVE)
     return nf * (iters * mg_bytes_per_iter(link_bytes) + mg_bytes_per_solve(link_bytes))
 
 
@@ -542,9 +563,10 @@ def rooflines(W, wl, m, store):
     mg = bool(wl.flags & W.FLAG_POISSON_MG)
     ph = m["phase"]
     split = mg and mg_split(W, wl, n_sms())
+    fused = split and mg_fused(W, wl, n_sms())
     if split:
         pk = "multigrid_split_solve"
-        pb = mg_algorithmic_bytes(wl, m["phase_iters"], link_bytes=1)
+        pb = mg_algorithmic_bytes(wl, m["phase_iters"], link_bytes=1, fused=fused)
     elif mg:
         pk = "poisson_mg_wide_kernel" if wl.n_nodes >= 152 * 16384 else "poisson_mg_kernel"
         pb = mg_algorithmic_bytes(wl, m["phase_iters"])
@@ -561,10 +583,11 @@ def rooflines(W, wl, m, store):
         pois["traffic_note"] = ("ncu, one pass: the start kernel plus the solve's graph, mean over the capture's "
                                 "solves (6.4 CG iterations on 256x256x512, 5.2 on 64x64x128)")
     if split:
-        pois["launches_per_solve"] = round(MG_SPLIT_KERNELS_PER_SOLVE + mg_split_kernels_per_iter(wl, n_sms())
+        pois["launches_per_solve"] = round(MG_SPLIT_KERNELS_PER_SOLVE + mg_split_kernels_per_iter(wl, n_sms(), fused)
                                            * m["phase_iters"], 1)
         pois["unit_measured"] = ("the whole solve, timed with CUDA events on its stream: a start kernel and one graph "
-                                 "launch (lattice passes one kernel each, the coarse levels of each V-cycle one "
+                                 "launch (lattice passes " + ("two half sweeps" if fused else "one half sweep") +
+                                 " per kernel, the coarse levels of each V-cycle one "
                                  "cooperative kernel, the CG loop a conditional WHILE node); bytes and time per solve")
     lbr = {"kernel": "lb_fused_kernel", "bound": "hbm", "achieved": round(la, 1), "peak": hbm,
            "unit": "GB/s", "frac": round(la / hbm, 4), "peak_kind": peak_kind,

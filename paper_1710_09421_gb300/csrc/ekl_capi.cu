@@ -823,14 +823,14 @@ static const char *build_multigrid(Ctx &c, const uint8_t *solid, Alloc &A, long 
     c.mg_split = split;
     c.mgs_threads = c.mg_wide ? MG_WIDE_THREADS : MG_THREADS;
     c.mgs_l1 = c.mg_split && c.mg_cta_from > 1 && c.mg_tile_from > 1;
-    // two half sweeps per launch on lattices whose solve does not stay in L2
-    // (37 bytes a node: r, z, p, p', q, the link byte, and phi and b of 8),
+    // two half sweeps per launch on lattices whose solve does not stay in L2,
     // where rows split into aligned pieces of four nodes: 256x256x512 takes 5.46
     // ms per solve with it and 7.64 with one half sweep per launch, 128x128x256
     // 1.09 and 1.40, and 64x64x128, bound by the chain of plane steps, 0.59 and
-    // 0.50.
-    const size_t l2 = 126u << 20;
-    c.mg_fused = c.mg_split && c.mg_wide && c.nx % 4 == 0 && (size_t)N * 37 > l2;
+    // 0.50.  Pieces of four nodes (nx = 4 mod 8), us per iteration: 100x192x192,
+    // the smallest such lattices, 214 and 251, 180x152x152 248 and 284, 508x256x256
+    // 1321 and 1495.
+    c.mg_fused = c.mg_split && c.mg_wide && c.nx % 4 == 0 && mgf_beyond_l2(N);
     c.mgs_iter_kernels = (c.mg_fused ? 11 : 2 * (2 * MG_NU - 1) + 8) +
                          (c.mgs_l1 ? 2 * (2 * MG_NU_COARSE - 1) + 2 : 0);
     if (ops(c.prec).mg_blocks(c.mg_smem, c.mg_wide) < 1) return "multigrid kernel cannot be resident";
@@ -1670,14 +1670,15 @@ int ekl_batch_create(int32_t nrep, const ekl_params *params, void *stream, ekl_b
             B.d_mgs_part = (double *)A(sizeof(double) * MGS_PART_SLOTS * (size_t)nrep * B.mgs_part_stride);
             // two half sweeps per launch, as on single lattices: where the
             // replicas together do not stay in L2 (ten of 6.5 M nodes: 3.65 ms a
-            // step without it, 3.22 with it) and all rows split into aligned pieces
+            // step without it, 3.22 with it; six of 100x128x128, in pieces of four
+            // nodes, 5.24 and 4.69) and all rows split into aligned pieces
             long long total = 0;
             int vmax = 4;
             for (int r = 0; r < nrep; r++) {
                 total += B.reps[r]->N;
                 if (B.reps[r]->nx % 8) vmax = B.reps[r]->nx % 4 ? 0 : std::min(vmax, 2);
             }
-            if (B.mgs_split && vmax && (size_t)total * 37 > ((size_t)126 << 20)) {
+            if (B.mgs_split && vmax && mgf_beyond_l2(total)) {
                 std::vector<MgfGeom> geom(nrep);
                 std::vector<MgfBlock> blocks;
                 B.mgs_fused = 1;

@@ -27,7 +27,9 @@
 // What bounds it: the chain of a plane step (0.9 us: a plane's loads, the two
 // dependent updates and the barrier) at 15 to 16 warps an SM, so it serves
 // lattices larger than L2, where the one-half-sweep passes are bound by their
-// traffic.  256x256x512, us per launch: PRE 66, RESTR 108, PRO 79, POST 86 and
+// traffic.  Counters on 128x128x256 (10 warps an SM): issue slots 30 to 34 % busy,
+// DRAM 18 to 23 % of its peak; warps wait for loads (1.8 to 3.2 cycles per
+// instruction issued) and at the barrier (1.3 to 2.2).  256x256x512, us per launch: PRE 66, RESTR 108, PRO 79, POST 86 and
 // the r.z partials 47, in place of three half sweeps of 88, the restriction of
 // 101, and half sweeps of 127, 88, 88 and 106.  Two half sweeps per launch on
 // 64x64x128 (13 us each), a whole pass per launch in tiles with a halo of four
@@ -40,6 +42,10 @@ namespace ekl {
 
 constexpr int MGF_THREADS = 512;   // 128 registers a thread
 enum { MGF_PRE = 0, MGF_RESTR = 1, MGF_PRO = 2, MGF_POST = 3 };
+
+// whether a solve over this many nodes does not stay in L2 (126 MB): 37 bytes a
+// node, r, z, p, p', q, the link byte, and phi and b of 8
+inline bool mgf_beyond_l2(long long nodes) { return (size_t)nodes * 37 > (size_t)126 << 20; }
 
 struct MgfGeom {
     int nx, ny, nz, per[3];

@@ -649,10 +649,13 @@ __global__ void __launch_bounds__(NT) l4_bwd_data(NetGrid g, const float *__rest
 // memory (16 bytes of BF16 channels per load, the next chunk's loads in
 // flight under this chunk's arithmetic), and a thread keeps 4 x 4 outputs (4
 // output by 4 input channels of one offset), so two 16-byte shared loads feed
-// 16 FMAs.  What bounds it: FMA issue, 6928 per node for a 16 -> 16 layer.
-// The form before gathered one value per thread with its index arithmetic and
-// two scalar shared loads per FMA: 710 us per layer on an 8192-node sample,
-// against 30 us now for eight samples in one launch.
+// 16 FMAs.  What bounds it: latency, the chain of a block's 32 chunks (staging,
+// barrier, arithmetic) with one block of 14 warps on an SM.  Eight samples of
+// 8192 nodes are 128 blocks and take 66 us for a 16 -> 16 layer (issue slots 51 %
+// busy, FMA pipe 28 %; its 6928 FMAs a node alone would take 11 us), 45 us for the
+// last layer and 47 us for the first; fewer samples take no less.  The form before
+// gathered one value per thread with its index arithmetic and two scalar shared
+// loads per FMA: 710 us per 16 -> 16 layer and sample.
 constexpr int WG_CH = 16;
 constexpr int WG_NODES = 512;
 constexpr int WG_T = 448;
