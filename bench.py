@@ -44,11 +44,11 @@ PROFILED = {
     # ncu pass over the benchmark command (--graph-profiling graph; the split solve's figure is its start
     # kernel plus its graph, the mean over the capture's solves: 6.4 CG iterations on 256x256x512, 5.2 on
     # 64x64x128)
-    ("lb_fused_kernel", "pore_256x256x512_r8_N128"): ("3748fc75630d6ab3", 7824183011 + 7365414755),
-    ("multigrid_split_solve", "pore_256x256x512_r8_N128"): ("b54e3161bf0d0b0c",
-                                                         674939861 + 696828516 + 30335018012 + 13175362446),
-    ("lb_fused_kernel", "pore_64x64x128_r4_N32"): ("3748fc75630d6ab3", 119387372 + 63406887),
-    ("multigrid_split_solve", "pore_64x64x128_r4_N32"): ("b54e3161bf0d0b0c", 10722363 + 0 + 17252569 + 42673),
+    ("lb_fused_kernel", "pore_256x256x512_r8_N128"): ("10a11f244e6a891f", 7824038613 + 7365457280),
+    ("multigrid_split_solve", "pore_256x256x512_r8_N128"): ("709bbd944d326a48",
+                                                         674914076 + 696878222 + 20891236423 + 7463117483),
+    ("lb_fused_kernel", "pore_64x64x128_r4_N32"): ("10a11f244e6a891f", 119390228 + 63359449),
+    ("multigrid_split_solve", "pore_64x64x128_r4_N32"): ("709bbd944d326a48", 10722934 + 0 + 17523436 + 45076),
 }
 KERNEL_SOURCES = {
     "lb_fused_kernel": ("ekl_kernels.cuh", "ekl_dev.cuh"),
