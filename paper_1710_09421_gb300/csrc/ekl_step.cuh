@@ -564,10 +564,16 @@ template <typename S, typename R, typename PhiT, bool DEV> int batch_tables(Batc
     std::vector<StepArgs<S, R, PhiT>> args(n);
     std::vector<BeadArgs<R>> bargs(n);
     std::vector<MdArgs<S, R, PhiT, DEV>> md(n);
+    // one launch with the fluctuating term serves replicas with and without it
+    // (these with thermal mass 0, which leaves every population as it is); the
+    // latter have no table of their own and read another's
+    const R *wchi = nullptr;
+    for (int r = 0; r < n && !wchi; r++) wchi = (const R *)B.reps[r]->wchi;
     for (int q = 0; q < 2; q++) {
         for (int r = 0; r < n; r++) {
             Ctx &c = *B.reps[r];
             args[r] = make_args<S, R, PhiT>(c, q);
+            if (!args[r].wchi) args[r].wchi = wchi;
             bargs[r] = make_bead_args<R>(c);
             md[r] = make_md_args<S, R, PhiT, DEV>(c, args[r], bargs[r]);
         }
