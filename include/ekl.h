@@ -312,7 +312,11 @@ void ekl_batch_destroy(ekl_batch *b);
  * k = (dz+1)*9 + (dy+1)*3 + (dx+1).  Inputs x[2][N] (channel-major), output
  * y[N]; periodic wrap on periodic axes, zeros beyond closed ones.  The two
  * 16 -> 16 layers run as BF16 implicit GEMMs on tensor cores with FP32
- * accumulation.  All pointers are host memory. */
+ * accumulation.  All pointers are host memory.  Grids have extents of at least
+ * 1 and at most 2^30 nodes (else EKL_ERR_ARG).  A training batch goes through the
+ * network in passes of at most 4 GB of device memory, smaller ones where the
+ * device has less to give; the result does not depend on the split (the losses
+ * up to the rounding of their FP64 sums). */
 #define EKL_NET_PARAMS 15169
 int ekl_net_eval(const int32_t dims[3], const int32_t periodic[3], const float *x, const float *w,
                  float *y);
